@@ -161,7 +161,7 @@ __global__ void __launch_bounds__(AT_THREADS, 1)
       mbar_init(kv_full + i, 1);
       mbar_init(kv_empty + i, 1);
       mbar_init(s_full + i, 1);
-      mbar_init(p_full + i, 128);
+      mbar_init(p_full + i, 4);  // one arrival per softmax warp of the tile
       mbar_init(o_done + i, 1);
     }
     mbar_init(drain, 1);
@@ -219,73 +219,78 @@ __global__ void __launch_bounds__(AT_THREADS, 1)
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      // ---------------- MMA issuer ----------------
-      constexpr uint32_t idesc = F16 ? idesc_f16_f32(AT_M, AT_N) : idesc_bf16_f32(AT_M, AT_N);
-      const uint32_t q_addr = smem_u32(sQ);
-      auto issue_s = [&](int x, int j) {
-        const uint32_t qa = q_addr + x * AT_TILE;
-        const uint32_t ka = smem_u32(sKV + (j % AT_STAGES) * 2 * AT_TILE);
+    // ---------------- MMA issuer (converged warp, one elected lane issues) ----------------
+    constexpr uint32_t idesc = F16 ? idesc_f16_f32(AT_M, AT_N) : idesc_bf16_f32(AT_M, AT_N);
+    const uint32_t q_addr = smem_u32(sQ), kv_addr = smem_u32(sKV);
+    // K step kk of a tile: 64-column chunk kk / 4, 32 bytes per step inside it (16-byte units)
+    auto koff = [](int kk) { return (uint64_t)(((kk >> 2) * AT_CHUNK + (kk & 3) * 32) >> 4); };
+    auto issue_s = [&](int x, int j) {
+      const uint64_t qd = sw128_desc(q_addr + x * AT_TILE);
+      const uint64_t kd = sw128_desc(kv_addr + (j % AT_STAGES) * 2 * AT_TILE);
+      if (elect_one()) {
 #pragma unroll
-        for (int kk = 0; kk < AT_D / 16; ++kk) {
-          const uint32_t off = (kk >> 2) * AT_CHUNK + (kk & 3) * 32;
-          mma_bf16(tmem + x * 128, sw128_desc(qa + off), sw128_desc(ka + off), idesc,
-                   kk > 0 ? 1u : 0u);
-        }
+        for (int kk = 0; kk < AT_D / 16; ++kk)
+          mma_bf16(tmem + x * 128, qd + koff(kk), kd + koff(kk), idesc, kk > 0 ? 1u : 0u);
         mma_commit(s_full + x);
-      };
-      auto issue_pv = [&](int x, int j) {
-        const uint32_t va = smem_u32(sKV + (j % AT_STAGES) * 2 * AT_TILE + AT_TILE);
+      }
+      __syncwarp();
+    };
+    // commit: a barrier to signal once these products are done (null: none)
+    auto issue_pv = [&](int x, int j, uint64_t* commit) {
+      const uint64_t vd = sw128_desc(kv_addr + (j % AT_STAGES) * 2 * AT_TILE + AT_TILE);
+      if (elect_one()) {
 #pragma unroll
-        for (int kk = 0; kk < AT_N / 16; ++kk) {
-          const uint32_t off = (kk >> 2) * AT_CHUNK + (kk & 3) * 32;
-          mma_bf16_ts(tmem + 256 + x * 128, tmem + x * 128 + kk * 8, sw128_desc(va + off), idesc,
+        for (int kk = 0; kk < AT_N / 16; ++kk)
+          mma_bf16_ts(tmem + 256 + x * 128, tmem + x * 128 + kk * 8, vd + koff(kk), idesc,
                       (j > 0 || kk > 0) ? 1u : 0u);
-        }
-      };
-      bool ok = mbar_wait(q_full, 0, abort_flag) && mbar_wait(kv_full, 0, abort_flag);
-      if (ok) {
-        tc_fence_after();
-        issue_s(0, 0);
-        issue_s(1, 0);
+        if (commit) mma_commit(commit);
       }
-      for (int j = 0; j < nkb && ok; ++j) {
-        const bool more = j + 1 < nkb;
-        // tile A: PV_j, then S_{j+1} into the columns P_j came from (in issue order)
-        if (!mbar_wait(p_full + 0, j & 1, abort_flag)) {
+      __syncwarp();
+    };
+    bool ok = mbar_wait_warp(q_full, 0, abort_flag) && mbar_wait_warp(kv_full, 0, abort_flag);
+    if (ok) {
+      tc_fence_after();
+      issue_s(0, 0);
+      issue_s(1, 0);
+    }
+    for (int j = 0; j < nkb && ok; ++j) {
+      const bool more = j + 1 < nkb;
+      // tile A: PV_j, then S_{j+1} into the columns P_j came from (in issue order)
+      if (!mbar_wait_warp(p_full + 0, j & 1, abort_flag)) {
+        ok = false;
+        break;
+      }
+      tc_fence_after();
+      issue_pv(0, j, more ? nullptr : o_done + 0);
+      if (more) {
+        if (!mbar_wait_warp(kv_full + (j + 1) % AT_STAGES, ((j + 1) / AT_STAGES) & 1, abort_flag)) {
           ok = false;
           break;
         }
         tc_fence_after();
-        issue_pv(0, j);
-        if (more) {
-          if (!mbar_wait(kv_full + (j + 1) % AT_STAGES, ((j + 1) / AT_STAGES) & 1, abort_flag)) {
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-          issue_s(0, j + 1);
-        } else {
-          mma_commit(o_done + 0);
-        }
-        // tile B
-        if (!mbar_wait(p_full + 1, j & 1, abort_flag)) {
-          ok = false;
-          break;
-        }
-        tc_fence_after();
-        issue_pv(1, j);
-        mma_commit(kv_empty + j % AT_STAGES);
-        if (more)
-          issue_s(1, j + 1);
-        else
-          mma_commit(o_done + 1);
+        issue_s(0, j + 1);
       }
+      // tile B
+      if (!mbar_wait_warp(p_full + 1, j & 1, abort_flag)) {
+        ok = false;
+        break;
+      }
+      tc_fence_after();
+      issue_pv(1, j, kv_empty + j % AT_STAGES);
+      if (more) {
+        issue_s(1, j + 1);
+      } else {
+        if (elect_one()) mma_commit(o_done + 1);
+        __syncwarp();
+      }
+    }
+    if (elect_one()) {
       mma_commit(drain);
       const uint64_t t0 = global_ns();
       while (!mbar_try_wait(drain, 0) && global_ns() - t0 < kWaitLimitNs) {
       }
     }
+    __syncwarp();
   } else {
     // ---------------- softmax warpgroups (warps 2..5: tile A, 6..9: tile B) ----------------
     const int x = (warp - 2) >> 2;
@@ -363,7 +368,8 @@ __global__ void __launch_bounds__(AT_THREADS, 1)
       }
       tmem_st_wait();
       tc_fence_before();
-      mbar_arrive(p_full + x);
+      __syncwarp();
+      if (lane == 0) mbar_arrive(p_full + x);
     }
     if (ok) {
       const bool w = mbar_wait(o_done + x, 0, abort_flag);

@@ -126,6 +126,24 @@ BAG_DEV bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort) {
   }
 }
 
+// The same for a converged warp that keeps running as one: every lane waits, and all get
+// the same answer (false as soon as one lane gave up), so the code after it stays uniform.
+BAG_DEV bool mbar_wait_warp(uint64_t* bar, uint32_t parity, volatile int* abort) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort));
+}
+
+// One lane of a converged warp (the same one at every call: the election is
+// deterministic for a given member mask).
+BAG_DEV bool elect_one() {
+  uint32_t p;
+  asm volatile(
+      "{\n\t.reg .pred P;\n\t"
+      "elect.sync _|P, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, P;\n\t}"
+      : "=r"(p));
+  return p != 0;
+}
+
 // ---------------------------------------------------------------------------
 // TMA
 // ---------------------------------------------------------------------------
@@ -152,6 +170,17 @@ BAG_DEV void tma_prefetch_desc(const CUtensorMap* map) {
 
 // ---------------------------------------------------------------------------
 // tcgen05 (tensor memory + 5th-gen MMA), cta_group::1
+//
+// Issuing.  The warp that issues the MMAs runs its loop converged, computes descriptors
+// as a warp-uniform base plus constants, and lets one elected lane issue a group of MMAs.
+// Its operands then live in uniform registers.  A loop run by one lane alone (if (lane ==
+// 0)) moves every descriptor from vector to uniform registers before each MMA, and loses
+// those issue slots to the arithmetic of the other warps on its scheduler: measured with
+// eight warps of FMA and EX2 beside it, 158 cycles per M128 N128 K16 MMA (64 at the tensor
+// rate) against 95-105 for the converged warp, and 66 in either form with idle neighbours.
+// Electing around each single MMA is slower than either (264-279 cycles).  In the kernels,
+// at the power cap: attention of 7145 tokens x 24 heads 511 -> 495 us, a FLUX-shaped
+// double-stream block 997 -> 970 us, Wan's 32,760-token block 29.3 -> 28.4 ms.
 // ---------------------------------------------------------------------------
 BAG_DEV void tmem_alloc(uint32_t* slot_smem, uint32_t ncols) {
   asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(

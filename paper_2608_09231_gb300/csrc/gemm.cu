@@ -343,8 +343,8 @@ __global__ void __launch_bounds__(192, 1)
     }
     mbar_init(tfull, 1);
     mbar_init(tfull + 1, 1);
-    mbar_init(tempty, 128);
-    mbar_init(tempty + 1, 128);
+    mbar_init(tempty, 4);       // one arrival per epilogue warp
+    mbar_init(tempty + 1, 4);
     mbar_init(drain, 1);
     *abort_flag = 0;
     fence_mbar_init();
@@ -409,50 +409,55 @@ __global__ void __launch_bounds__(192, 1)
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      // ---------------- MMA issuer ----------------
-      constexpr uint32_t idesc = idesc_bf16_f32(TC_BM, BN);
-      int s = 0;
-      uint32_t ph = 0;
-      int acc = 0;
-      uint32_t aph = 0;
-      bool ok = true;
-      for (int tile = blockIdx.x; tile < tiles && ok; tile += gridDim.x) {
-        if (!mbar_wait(tempty + acc, aph ^ 1, abort_flag)) {
+    // ---------------- MMA issuer (converged warp, one elected lane issues) ----------------
+    constexpr uint32_t idesc = idesc_bf16_f32(TC_BM, BN);
+    const uint32_t a_base = smem_u32(sA), b_base = smem_u32(sB);
+    int s = 0;
+    uint32_t ph = 0;
+    int acc = 0;
+    uint32_t aph = 0;
+    bool ok = true;
+    for (int tile = blockIdx.x; tile < tiles && ok; tile += gridDim.x) {
+      if (!mbar_wait_warp(tempty + acc, aph ^ 1, abort_flag)) {
+        ok = false;
+        break;
+      }
+      tc_fence_after();
+      const uint32_t dt = tmem_base + (uint32_t)(acc * BN);
+      for (int kb = 0; kb < kit; ++kb) {
+        if (!mbar_wait_warp(full + s, ph, abort_flag)) {
           ok = false;
           break;
         }
         tc_fence_after();
-        const uint32_t dt = tmem_base + (uint32_t)(acc * BN);
-        for (int kb = 0; kb < kit; ++kb) {
-          if (!mbar_wait(full + s, ph, abort_flag)) {
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-          const uint32_t a0 = smem_u32(sA + s * C::A_BYTES);
-          const uint32_t b0 = smem_u32(sB + s * C::B_BYTES);
+        const uint64_t ad = sw128_desc(a_base + s * C::A_BYTES);
+        const uint64_t bd = sw128_desc(b_base + s * C::B_BYTES);
+        if (elect_one()) {
 #pragma unroll
-          for (int k = 0; k < TC_BK / 16; ++k)
-            mma_bf16(dt, sw128_desc(a0 + k * 32), sw128_desc(b0 + k * 32), idesc,
-                     (kb | k) != 0 ? 1u : 0u);
+          for (int k = 0; k < TC_BK / 16; ++k)  // 32 bytes along K: two 16-byte units
+            mma_bf16(dt, ad + 2 * k, bd + 2 * k, idesc, (kb | k) != 0 ? 1u : 0u);
           mma_commit(empty + s);
-          if (++s == C::STAGES) {
-            s = 0;
-            ph ^= 1;
-          }
         }
-        if (!ok) break;
-        mma_commit(tfull + acc);
-        acc ^= 1;
-        if (acc == 0) aph ^= 1;
+        __syncwarp();
+        if (++s == C::STAGES) {
+          s = 0;
+          ph ^= 1;
+        }
       }
-      // make sure every issued MMA has finished before TMEM is released
+      if (!ok) break;
+      if (elect_one()) mma_commit(tfull + acc);
+      __syncwarp();
+      acc ^= 1;
+      if (acc == 0) aph ^= 1;
+    }
+    // make sure every issued MMA has finished before TMEM is released
+    if (elect_one()) {
       mma_commit(drain);
       const uint64_t t0 = global_ns();
       while (!mbar_try_wait(drain, 0) && global_ns() - t0 < kWaitLimitNs) {
       }
     }
+    __syncwarp();
   } else {
     // ---------------- epilogue (warps 2..5 cover TMEM lane quarters 2,3,0,1) ----------------
     const int q = warp & 3;
@@ -469,7 +474,8 @@ __global__ void __launch_bounds__(192, 1)
       const uint32_t tb = tmem_base + (uint32_t)(acc * BN) + ((uint32_t)(q * 32) << 16);
       drain_accumulator<BN>(e, t, row, nt * BN, tb, vt_scratch + (warp - 2) * kVtScratchFloats);
       tc_fence_before();
-      mbar_arrive(tempty + acc);
+      __syncwarp();
+      if (lane == 0) mbar_arrive(tempty + acc);
       acc ^= 1;
       if (acc == 0) aph ^= 1;
     }
@@ -571,8 +577,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(192, 1)
     }
     mbar_init(tfull, 1);
     mbar_init(tfull + 1, 1);
-    mbar_init(tempty, 256);     // even CTA: every epilogue thread of both CTAs
-    mbar_init(tempty + 1, 256);
+    mbar_init(tempty, 8);     // even CTA: every epilogue warp of both CTAs
+    mbar_init(tempty + 1, 8);
     mbar_init(drain, 1);
     *abort_flag = 0;
     fence_mbar_init();
@@ -640,49 +646,56 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(192, 1)
       }
     }
   } else if (warp == 1) {
-    if (lane == 0 && rank == 0) {
-      // ---------------- MMA issuer (even CTA) ----------------
+    if (rank == 0) {
+      // -------- MMA issuer (even CTA; converged warp, one elected lane issues) --------
       constexpr uint32_t idesc = idesc_bf16_f32(PR_BM, PR_BN);
+      const uint32_t a_base = smem_u32(sA), b_base = smem_u32(sB);
       int s = 0;
       uint32_t ph = 0;
       int acc = 0;
       uint32_t aph = 0;
       bool ok = true;
       for (int tile = pair; tile < tiles && ok; tile += npairs) {
-        if (!mbar_wait(tempty + acc, aph ^ 1, abort_flag)) {
+        if (!mbar_wait_warp(tempty + acc, aph ^ 1, abort_flag)) {
           ok = false;
           break;
         }
         tc_fence_after();
         const uint32_t dt = tmem_base + (uint32_t)(acc * PR_BN);
         for (int kb = 0; kb < kit; ++kb) {
-          if (!mbar_wait(full + s, ph, abort_flag)) {
+          if (!mbar_wait_warp(full + s, ph, abort_flag)) {
             ok = false;
             break;
           }
           tc_fence_after();
-          const uint32_t a0 = smem_u32(sA + s * PR_HALF_BYTES);
-          const uint32_t b0 = smem_u32(sB + s * PR_HALF_BYTES);
+          const uint64_t ad = sw128_desc(a_base + s * PR_HALF_BYTES);
+          const uint64_t bd = sw128_desc(b_base + s * PR_HALF_BYTES);
+          if (elect_one()) {
 #pragma unroll
-          for (int k = 0; k < TC_BK / 16; ++k)
-            mma_bf16_pair(dt, sw128_desc(a0 + k * 32), sw128_desc(b0 + k * 32), idesc,
-                          (kb | k) != 0 ? 1u : 0u);
-          mma_commit_pair(empty + s, 3);
+            for (int k = 0; k < TC_BK / 16; ++k)  // 32 bytes along K: two 16-byte units
+              mma_bf16_pair(dt, ad + 2 * k, bd + 2 * k, idesc, (kb | k) != 0 ? 1u : 0u);
+            mma_commit_pair(empty + s, 3);
+          }
+          __syncwarp();
           if (++s == PR_STAGES) {
             s = 0;
             ph ^= 1;
           }
         }
         if (!ok) break;
-        mma_commit_pair(tfull + acc, 3);
+        if (elect_one()) mma_commit_pair(tfull + acc, 3);
+        __syncwarp();
         acc ^= 1;
         if (acc == 0) aph ^= 1;
       }
       // every issued MMA has finished before tensor memory is released
-      mma_commit_pair(drain, 1);
-      const uint64_t t0 = global_ns();
-      while (!mbar_try_wait(drain, 0) && global_ns() - t0 < kWaitLimitNs) {
+      if (elect_one()) {
+        mma_commit_pair(drain, 1);
+        const uint64_t t0 = global_ns();
+        while (!mbar_try_wait(drain, 0) && global_ns() - t0 < kWaitLimitNs) {
+        }
       }
+      __syncwarp();
     }
   } else {
     // ---------------- epilogue (both CTAs: their 128 rows of each tile) ----------------
@@ -701,10 +714,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(192, 1)
       const uint32_t tb = tmem_base + (uint32_t)(acc * PR_BN) + ((uint32_t)(q * 32) << 16);
       drain_accumulator<PR_BN>(e, t, row, nt * PR_BN, tb, vt_scratch + (warp - 2) * kVtScratchFloats);
       tc_fence_before();
-      if (rank == 0)
-        mbar_arrive(tempty + acc);
-      else
-        mbar_arrive_remote(te_remote + (uint32_t)(acc * sizeof(uint64_t)));
+      __syncwarp();
+      if (lane == 0) {
+        if (rank == 0)
+          mbar_arrive(tempty + acc);
+        else
+          mbar_arrive_remote(te_remote + (uint32_t)(acc * sizeof(uint64_t)));
+      }
       acc ^= 1;
       if (acc == 0) aph ^= 1;
     }
