@@ -3,7 +3,7 @@
 //  * ln_mod: row LayerNorm + adaLN modulation (1 + scale) * LN(x) + shift, optionally
 //    fused with the trajectory signal (per-row partial sums of |m_t - m_last| and
 //    |m_last|, the relative-L1 drift of the first block's modulated input).
-//  * gate_step: one warp; reduces the signal partials in a fixed order, forms the gate
+//  * gate_step: one CTA; reduces the signal partials in a fixed order, forms the gate
 //    inputs, evaluates the 3->16->1 gate in fp32 with every product and sum rounded
 //    separately, applies Algorithm 2's two forced rules, updates the counters and the
 //    step log, and hands the decision to a CUDA-graph conditional node.
@@ -309,7 +309,7 @@ cudaError_t rel_l1_partials(const void* a, const void* b, int a_bf16, long rows,
 }
 
 // out[0] = sum(num) / sum(den), out[1] = sum(num), out[2] = sum(den) over the per-row
-// partials, summed in the same fixed order as the gate kernel's drift reduction.
+// partials, summed in a fixed order.
 __global__ void rel_l1_finalize_kernel(const float* partial, long rows, float* out) {
   grid_dep_sync();
   const int lane = threadIdx.x;
@@ -336,57 +336,82 @@ cudaError_t rel_l1_finalize(const float* partial, long rows, float* out, cudaStr
 }
 
 // ---------------------------------------------------------------------------
-// gate + pacing (one warp)
+// gate + pacing (one CTA)
 // ---------------------------------------------------------------------------
 // Gate parameters: every layer's W [out][in] (row-major) then b, in evaluation order,
 // from offset 0; z-score mean at kGateMu, standard deviation at kGateSd (3 or 6 used).
 //   kind 0 (3 inputs): 3 -> 16 -> 1
 //   kind 1 (6 inputs): 6 -> 8 -> 8 -> 32 -> 1
 //   kind 2 (6 inputs): [budget 3 -> 8 -> 8 | trajectory 3 -> 8 -> 8] -> 16 -> 32 -> 1
-// Every hidden layer is followed by ReLU.  Each dense layer runs in a fixed order (bias
-// first, then inputs in index order, every product and sum rounded on its own) so the
-// logit is reproducible bit for bit by any IEEE fp32 evaluation in the same order.
-BAG_DEV const float* dense32(const float* p, int out, int in, const float* x, float* y, bool relu) {
-  const float* W = p;
-  const float* b = p + out * in;
-  for (int j = 0; j < out; ++j) {
-    float h = b[j];
-    for (int i = 0; i < in; ++i) h = __fadd_rn(h, __fmul_rn(W[j * in + i], x[i]));
-    if (relu && !(h > 0.f)) h = 0.f;
-    y[j] = h;
-  }
-  return b + out;
+// Every hidden layer is followed by ReLU.  Each output of a dense layer is summed by one
+// lane in a fixed order (bias first, then inputs in index order, every product and sum
+// rounded on its own) so the logit is reproducible bit for bit by any IEEE fp32
+// evaluation in the same order; the outputs of a layer are independent of one another
+// and run on the lanes of one warp.
+//
+// The kernel is pure latency: it sits between the signal pass and the decision, and
+// nothing overlaps it.  128 threads (512 from 1024 rows on) sum the row partials, and the
+// parameters are in shared memory before the predecessor finishes.  One warp that walked
+// the rows alone, its first lane reading the parameters from global memory one dependent
+// sum after another, took 10.6 us (3-input gate, 4096 rows), 15.3 us (WAN6, 390 rows),
+// 73.7 us (WAN6, 32,760 rows) per launch in a chain; this takes 3.8, 3.3 and 12.9 us.
+constexpr int GATE_THREADS = 512;
+
+// Output `lane` (< out) of a layer at p with inputs x (shared memory); its W and b in p.
+BAG_DEV float dense_lane(const float* p, int out, int in, const float* x, int lane, bool relu) {
+  float h = p[out * in + lane];
+  for (int i = 0; i < in; ++i) h = __fadd_rn(h, __fmul_rn(p[lane * in + i], x[i]));
+  return relu && !(h > 0.f) ? 0.f : h;
 }
 
-__global__ void gate_kernel(DevState* st, const float* partial, int rows, const float* gp,
-                            int kind, float thr, int T, int B, int policy, const uint8_t* pmask,
-                            float delta, float* log, cudaGraphConditionalHandle handle,
-                            int use_cond) {
+__global__ void __launch_bounds__(GATE_THREADS)
+    gate_kernel(DevState* st, const float* partial, int rows, const float* gp, int kind, float thr, int T,
+                int B, int policy, const uint8_t* pmask, float delta, float* log,
+                cudaGraphConditionalHandle handle, int use_cond) {
+  __shared__ float gs[kGateFloats];
+  __shared__ float4 red[GATE_THREADS / 32];
+  __shared__ float xs[6], la[32], lb[32];
+  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  // the gate's parameters are written by no kernel of a step: read ahead of the wait
+  const int np = kind == 0 ? 81 : (kind == 1 ? 449 : 785);
+  for (int i = threadIdx.x; i < np; i += blockDim.x) gs[i] = gp[i];
+  if (threadIdx.x < kGateFloats - kGateMu) gs[kGateMu + threadIdx.x] = gp[kGateMu + threadIdx.x];
   grid_dep_sync();
-  const int lane = threadIdx.x;
   const int t = st->t, c = st->c, t_last = st->t_last;
-  float num = 0.f, den = 0.f, num2 = 0.f, den2 = 0.f;
+  // sums over rows: thread k takes rows k, k + blockDim, ...; then a fixed tree of lanes and warps
+  float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
   if (t > 0) {
-    for (int r = lane; r < rows; r += 32) {
-      num += partial[4 * r];
-      den += partial[4 * r + 1];
-      num2 += partial[4 * r + 2];
-      den2 += partial[4 * r + 3];
-    }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-      num += __shfl_xor_sync(0xffffffffu, num, off);
-      den += __shfl_xor_sync(0xffffffffu, den, off);
-      num2 += __shfl_xor_sync(0xffffffffu, num2, off);
-      den2 += __shfl_xor_sync(0xffffffffu, den2, off);
+    const float4* p4 = reinterpret_cast<const float4*>(partial);
+#pragma unroll 4
+    for (int r = threadIdx.x; r < rows; r += blockDim.x) {
+      const float4 v = p4[r];
+      s.x += v.x;
+      s.y += v.y;
+      s.z += v.z;
+      s.w += v.w;
     }
   }
-  if (lane != 0) return;
+  auto warp_sum = [](float4 v) {
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+      v.x += __shfl_xor_sync(0xffffffffu, v.x, off);
+      v.y += __shfl_xor_sync(0xffffffffu, v.y, off);
+      v.z += __shfl_xor_sync(0xffffffffu, v.z, off);
+      v.w += __shfl_xor_sync(0xffffffffu, v.w, off);
+    }
+    return v;
+  };
+  s = warp_sum(s);
+  if (lane == 0) red[warp] = s;
+  __syncthreads();
+  if (warp != 0) return;
+  s = warp_sum(lane < blockDim.x / 32 ? red[lane] : make_float4(0.f, 0.f, 0.f, 0.f));
+  const float num = s.x, den = s.y, num2 = s.z, den2 = s.w;
   float* L = log + (long)t * kLogFloats;
   int m = 1, gbit = 1;
   float z = 0.f, f0 = 0.f, f1 = 0.f, drift = 0.f, step = 0.f;
   float sb[3] = {0.f, 0.f, 0.f};
-  if (t > 0) {
+  if (t > 0) {  // uniform over the warp
     f0 = __fdiv_rn((float)(B - c), (float)B);
     f1 = __fdiv_rn((float)(T - t), (float)T);
     drift = __fdiv_rn(num, den);
@@ -394,33 +419,48 @@ __global__ void gate_kernel(DevState* st, const float* partial, int rows, const 
     sb[0] = __fdiv_rn((float)B, (float)T);
     sb[1] = f0;
     sb[2] = __fdiv_rn((float)(B - c), (float)(T - t));
-    const float* mu = gp + kGateMu;
-    const float* sd = gp + kGateSd;
-    float x[6], h1[32], h2[32];
-    if (kind == 0) {
-      const float f[3] = {f0, f1, drift};
-      for (int i = 0; i < 3; ++i) x[i] = __fdiv_rn(__fsub_rn(f[i], mu[i]), sd[i]);
-      const float* p = dense32(gp, 16, 3, x, h1, true);
-      dense32(p, 1, 16, h1, h2, false);
-    } else {
-      const float f[6] = {sb[0], sb[1], sb[2], (float)(t - t_last), drift, step};
-      for (int i = 0; i < 6; ++i) x[i] = __fdiv_rn(__fsub_rn(f[i], mu[i]), sd[i]);
-      if (kind == 1) {
-        const float* p = dense32(gp, 8, 6, x, h1, true);
-        p = dense32(p, 8, 8, h1, h2, true);
-        p = dense32(p, 32, 8, h2, h1, true);
-        dense32(p, 1, 32, h1, h2, false);
-      } else {
-        float hb[8], cat[16];
-        const float* p = dense32(gp, 8, 3, x, hb, true);
-        p = dense32(p, 8, 8, hb, cat, true);
-        p = dense32(p, 8, 3, x + 3, hb, true);
-        p = dense32(p, 8, 8, hb, cat + 8, true);
-        p = dense32(p, 32, 16, cat, h1, true);
-        dense32(p, 1, 32, h1, h2, false);
-      }
+    const int nin = kind == 0 ? 3 : 6;
+    if (lane < nin) {
+      float f;
+      if (kind == 0)
+        f = lane == 0 ? f0 : (lane == 1 ? f1 : drift);
+      else
+        f = lane < 3 ? sb[lane] : (lane == 3 ? (float)(t - t_last) : (lane == 4 ? drift : step));
+      xs[lane] = __fdiv_rn(__fsub_rn(f, gs[kGateMu + lane]), gs[kGateSd + lane]);
     }
-    z = h2[0];
+    __syncwarp();
+    const float* last;  // the output layer's parameters and inputs
+    const float* hin;
+    int nh;
+    if (kind == 0) {
+      if (lane < 16) la[lane] = dense_lane(gs, 16, 3, xs, lane, true);
+      last = gs + 16 * 3 + 16;
+      hin = la;
+      nh = 16;
+    } else if (kind == 1) {
+      if (lane < 8) la[lane] = dense_lane(gs, 8, 6, xs, lane, true);
+      __syncwarp();
+      if (lane < 8) lb[lane] = dense_lane(gs + 56, 8, 8, la, lane, true);
+      __syncwarp();
+      la[lane] = dense_lane(gs + 56 + 72, 32, 8, lb, lane, true);
+      last = gs + 56 + 72 + 288;
+      hin = la;
+      nh = 32;
+    } else {
+      // the two branches side by side: lanes 0-7 budget, 8-15 trajectory (each branch's
+      // two layers are 32 + 72 parameters)
+      const int br = lane / 8;
+      if (lane < 16) la[lane] = dense_lane(gs + br * 104, 8, 3, xs + 3 * br, lane % 8, true);
+      __syncwarp();
+      if (lane < 16) lb[lane] = dense_lane(gs + br * 104 + 32, 8, 8, la + 8 * br, lane % 8, true);
+      __syncwarp();
+      la[lane] = dense_lane(gs + 208, 32, 16, lb, lane, true);
+      last = gs + 208 + 544;
+      hin = la;
+      nh = 32;
+    }
+    __syncwarp();
+    z = dense_lane(last, 1, nh, hin, 0, false);  // every lane, the same sum
     gbit = z > thr ? 1 : 0;
     if (policy == 0) {  // Algorithm 2
       m = gbit;
@@ -434,35 +474,25 @@ __global__ void gate_kernel(DevState* st, const float* partial, int rows, const 
       m = pmask[t] ? 1 : 0;
     }
   }
-  L[0] = f0;
-  L[1] = f1;
-  L[2] = drift;
-  L[3] = z;
-  L[4] = (float)gbit;
-  L[5] = (float)m;
-  L[6] = (float)c;
-  L[7] = t > 0 ? (float)(t - t_last) : 0.f;
-  L[8] = sb[0];
-  L[9] = sb[1];
-  L[10] = sb[2];
-  L[11] = num;
-  L[12] = den;
-  L[13] = step;
-  L[14] = num2;
-  L[15] = den2;
+  if (lane != 0) return;
+  if (use_cond) cudaGraphSetConditional(handle, (unsigned)m);
   st->flag = m;
   if (m) {
     st->c = c + 1;
     st->t_last = t;
   }
-  if (use_cond) cudaGraphSetConditional(handle, (unsigned)m);
+  float4* L4 = reinterpret_cast<float4*>(L);  // kLogFloats is a multiple of four
+  L4[0] = make_float4(f0, f1, drift, z);
+  L4[1] = make_float4((float)gbit, (float)m, (float)c, t > 0 ? (float)(t - t_last) : 0.f);
+  L4[2] = make_float4(sb[0], sb[1], sb[2], num);
+  L4[3] = make_float4(den, step, num2, den2);
 }
 
 cudaError_t gate_step(DevState* st, const float* sig_partial, int sig_rows, const float* gate_params,
                       int gate_kind, float thr, int T, int B, int policy, const uint8_t* policy_mask,
                       float delta, float* log, unsigned long long cond_handle, int use_cond,
                       cudaStream_t s) {
-  launch_kernel(gate_kernel, 1, 32, 0, s, st, sig_partial, sig_rows, gate_params, gate_kind, thr, T, B,
+  launch_kernel(gate_kernel, 1, sig_rows < 1024 ? 128 : GATE_THREADS, 0, s, st, sig_partial, sig_rows, gate_params, gate_kind, thr, T, B,
                 policy, policy_mask, delta, log, (cudaGraphConditionalHandle)cond_handle, use_cond);
   return cudaGetLastError();
 }
