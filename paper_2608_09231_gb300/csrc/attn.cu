@@ -18,88 +18,144 @@ BAG_DEV float ldv(const void* p, long i) {
     return reinterpret_cast<const float*>(p)[i];
 }
 
-// CTA = 4 warps = 16 queries of one head; each warp owns 4 queries.  Key tiles of 32
-// are staged in shared memory (K transposed so that lane j reads key j's column).
+// Four consecutive elements (fp32 rows of the contexts are 16-byte aligned).
+template <typename T>
+BAG_DEV float4 ldv4(const void* p, long i) {
+  if constexpr (sizeof(T) == 4)
+    return *reinterpret_cast<const float4*>(reinterpret_cast<const float*>(p) + i);
+  else
+    return make_float4(ldv<T>(p, i), ldv<T>(p, i + 1), ldv<T>(p, i + 2), ldv<T>(p, i + 3));
+}
+
+// CTA = eight queries of one head; its eight warps take the key tiles (32 keys) in turn,
+// each with its own running maximum, sum and output for all eight queries, merged in warp
+// order at the end.  Scores: lane = key, which reads its own K row four elements at a time
+// against the queries broadcast from shared memory (8 x 4 products per K load); the
+// weights pass through shared memory so that the output has lane = head dimensions and
+// reads V rows coalesced.  Bound: latency (the fp32 backbones have a few hundred tokens);
+// few queries per CTA and the keys split over warps keep every SM busy with a short chain.
+// Measured against sixteen queries per CTA whose four warps walked all keys one barrier
+// after another (profiled launches): 288 tokens x 4 heads of 64 41 -> 20 us.
+constexpr int SA_Q = 8, SA_WARPS = 8, SA_KT = 32;
+
 template <typename T, int DH>
-__global__ void __launch_bounds__(128) attn_simt_kernel(const AttnArgs a) {
+__global__ void __launch_bounds__(SA_WARPS * 32) attn_simt_kernel(const AttnArgs a) {
   grid_dep_sync();
   if (epi_skip(a.st, a.flag_want)) return;
-  constexpr int QPW = 4, QPB = 16, KT = 32, R = DH / 32;
-  __shared__ float Qs[QPB][DH];
-  __shared__ float Kt[DH][KT + 1];
-  __shared__ float Vs[KT][DH];
-  const int head = blockIdx.y, q0 = blockIdx.x * QPB;
+  constexpr int R = DH / 32;  // head dimensions per lane: lane * R .. lane * R + R - 1
+  __shared__ __align__(16) float Qs[SA_Q][DH];
+  __shared__ __align__(16) float Ps[SA_WARPS][SA_Q][SA_KT];
+  __shared__ float Os[SA_WARPS][SA_Q][DH], ms[SA_WARPS][SA_Q], ls[SA_WARPS][SA_Q];
+  const int head = blockIdx.y, q0 = blockIdx.x * SA_Q;
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   const float scale = rsqrtf((float)DH);
-  for (int i = threadIdx.x; i < QPB * DH; i += blockDim.x) {
+  for (int i = threadIdx.x; i < SA_Q * DH; i += blockDim.x) {
     const int r = i / DH, c = i % DH, q = q0 + r;
     Qs[r][c] = q < a.nq ? ldv<T>(a.q, (long)q * a.ldq + head * DH + c) * scale : 0.f;
   }
-  float m[QPW], l[QPW], o[QPW][R];
+  __syncthreads();
+  float m[SA_Q], l[SA_Q], o[SA_Q][R];  // l: this lane's keys only
 #pragma unroll
-  for (int i = 0; i < QPW; ++i) {
+  for (int i = 0; i < SA_Q; ++i) {
     m[i] = -INFINITY;
     l[i] = 0.f;
 #pragma unroll
     for (int r = 0; r < R; ++r) o[i][r] = 0.f;
   }
-  for (int kb = 0; kb < a.nk; kb += KT) {
-    __syncthreads();
-    for (int i = threadIdx.x; i < KT * DH; i += blockDim.x) {
-      const int j = i / DH, c = i % DH, kk = kb + j;
-      float kv = 0.f, vv = 0.f;
-      if (kk < a.nk) {
-        kv = ldv<T>(a.k, (long)kk * a.ldk + head * DH + c);
-        vv = a.v_mode == 0 ? ldv<T>(a.v, (long)kk * a.ldv + head * DH + c)
-                           : ldv<T>(a.v, (long)(head * DH + c) * a.vpad + kk);
-      }
-      Kt[c][j] = kv;
-      Vs[j][c] = vv;
-    }
-    __syncthreads();
+  for (int kb = warp * SA_KT; kb < a.nk; kb += SA_WARPS * SA_KT) {
     const bool valid = kb + lane < a.nk;
+    const long krow = (long)(valid ? kb + lane : a.nk - 1) * a.ldk + head * DH;
+    float s[SA_Q];
 #pragma unroll
-    for (int qi = 0; qi < QPW; ++qi) {
-      const int qr = warp * QPW + qi;
-      float s = 0.f;
+    for (int i = 0; i < SA_Q; ++i) s[i] = 0.f;
 #pragma unroll 8
-      for (int c = 0; c < DH; ++c) s += Qs[qr][c] * Kt[c][lane];
-      s = valid ? s : -INFINITY;
-      float mx = s;
+    for (int c = 0; c < DH; c += 4) {
+      const float4 k4 = ldv4<T>(a.k, krow + c);
+#pragma unroll
+      for (int i = 0; i < SA_Q; ++i) {
+        const float4 q4 = *reinterpret_cast<const float4*>(&Qs[i][c]);
+        s[i] += q4.x * k4.x;
+        s[i] += q4.y * k4.y;
+        s[i] += q4.z * k4.z;
+        s[i] += q4.w * k4.w;
+      }
+    }
+    __syncwarp();  // every lane has read the previous tile's weights
+#pragma unroll
+    for (int i = 0; i < SA_Q; ++i) {
+      const float si = valid ? s[i] : -INFINITY;
+      float mx = si;
 #pragma unroll
       for (int off = 16; off > 0; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
-      const float mn = fmaxf(m[qi], mx);
-      const float p = valid ? expf(s - mn) : 0.f;
-      const float corr = expf(m[qi] - mn);
-      float ps = p;
+      const float mn = fmaxf(m[i], mx);
+      // scores that all underflowed to -inf weigh nothing unless every warp's did
+      const float base = mn == -INFINITY ? 0.f : mn;
+      const float p = expf(si - base);  // 0 past the last key
+      const float corr = expf(m[i] - base);
+      Ps[warp][i][lane] = p;
+      l[i] = l[i] * corr + p;
 #pragma unroll
-      for (int off = 16; off > 0; off >>= 1) ps += __shfl_xor_sync(0xffffffffu, ps, off);
-      l[qi] = l[qi] * corr + ps;
+      for (int r = 0; r < R; ++r) o[i][r] *= corr;
+      m[i] = mn;
+    }
+    __syncwarp();
+    const int nkt = min(SA_KT, a.nk - kb);
+#pragma unroll 2
+    for (int j = 0; j < nkt; j += 4) {
+      float v[4][R];
 #pragma unroll
-      for (int r = 0; r < R; ++r) o[qi][r] *= corr;
-      for (int j = 0; j < KT; ++j) {
-        const float pj = __shfl_sync(0xffffffffu, p, j);
+      for (int u = 0; u < 4; ++u) {
+        const long kk = min(kb + j + u, a.nk - 1);  // past the last key the weight is zero
 #pragma unroll
-        for (int r = 0; r < R; ++r) o[qi][r] += pj * Vs[j][lane + 32 * r];
+        for (int r = 0; r < R; ++r)
+          v[u][r] = a.v_mode == 0 ? ldv<T>(a.v, kk * a.ldv + head * DH + lane * R + r)
+                                  : ldv<T>(a.v, (long)(head * DH + lane * R + r) * a.vpad + kk);
       }
-      m[qi] = mn;
+#pragma unroll
+      for (int i = 0; i < SA_Q; ++i) {
+        const float4 p4 = *reinterpret_cast<const float4*>(&Ps[warp][i][j]);
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          o[i][r] += p4.x * v[0][r];
+          o[i][r] += p4.y * v[1][r];
+          o[i][r] += p4.z * v[2][r];
+          o[i][r] += p4.w * v[3][r];
+        }
+      }
     }
   }
 #pragma unroll
-  for (int qi = 0; qi < QPW; ++qi) {
-    const int q = q0 + warp * QPW + qi;
-    if (q >= a.nq) continue;
-    const float inv = 1.f / l[qi];
+  for (int i = 0; i < SA_Q; ++i) {
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-      const long idx = (long)q * a.ldo + head * DH + lane + 32 * r;
-      const float val = o[qi][r] * inv;
-      void* ob = (a.o2 && q >= a.o_split) ? a.o2 : a.o;
-      if (a.bf16)
-        reinterpret_cast<__nv_bfloat16*>(ob)[idx] = __float2bfloat16_rn(val);
-      else
-        reinterpret_cast<float*>(ob)[idx] = val;
+    for (int off = 16; off > 0; off >>= 1) l[i] += __shfl_xor_sync(0xffffffffu, l[i], off);
+    if (lane == 0) {
+      ms[warp][i] = m[i];
+      ls[warp][i] = l[i];
     }
+#pragma unroll
+    for (int r = 0; r < R; ++r) Os[warp][i][lane * R + r] = o[i][r];
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < SA_Q * DH; i += blockDim.x) {
+    const int r = i / DH, c = i % DH, q = q0 + r;
+    if (q >= a.nq) continue;
+    float mx = ms[0][r];  // warp 0 always has a key tile
+#pragma unroll
+    for (int w = 1; w < SA_WARPS; ++w) mx = fmaxf(mx, ms[w][r]);
+    float num = 0.f, den = 0.f;
+#pragma unroll
+    for (int w = 0; w < SA_WARPS; ++w) {
+      const float f = expf(ms[w][r] - mx);  // 0 for a warp without keys
+      num += f * Os[w][r][c];
+      den += f * ls[w][r];
+    }
+    const float val = num / den;
+    const long idx = (long)q * a.ldo + head * DH + c;
+    void* ob = (a.o2 && q >= a.o_split) ? a.o2 : a.o;
+    if (a.bf16)
+      reinterpret_cast<__nv_bfloat16*>(ob)[idx] = __float2bfloat16_rn(val);
+    else
+      reinterpret_cast<float*>(ob)[idx] = val;
   }
 }
 
@@ -115,17 +171,17 @@ cudaError_t attention(const AttnArgs& a, int* err, cudaStream_t s, int force_sim
     return attention_tc(a, err, s);
   }
   if (a.f16 || a.nbr > 1) return cudaErrorNotSupported;  // tensor-core kernel only
-  dim3 grid((a.nq + 15) / 16, a.heads);
+  dim3 grid((a.nq + SA_Q - 1) / SA_Q, a.heads);
   if (a.dh == 64) {
     if (a.bf16)
-      launch_kernel(attn_simt_kernel<__nv_bfloat16, 64>, grid, 128, 0, s, a);
+      launch_kernel(attn_simt_kernel<__nv_bfloat16, 64>, grid, SA_WARPS * 32, 0, s, a);
     else
-      launch_kernel(attn_simt_kernel<float, 64>, grid, 128, 0, s, a);
+      launch_kernel(attn_simt_kernel<float, 64>, grid, SA_WARPS * 32, 0, s, a);
   } else if (a.dh == 128) {
     if (a.bf16)
-      launch_kernel(attn_simt_kernel<__nv_bfloat16, 128>, grid, 128, 0, s, a);
+      launch_kernel(attn_simt_kernel<__nv_bfloat16, 128>, grid, SA_WARPS * 32, 0, s, a);
     else
-      launch_kernel(attn_simt_kernel<float, 128>, grid, 128, 0, s, a);
+      launch_kernel(attn_simt_kernel<float, 128>, grid, SA_WARPS * 32, 0, s, a);
   } else {
     return cudaErrorInvalidValue;
   }

@@ -34,3 +34,27 @@ def test_gate_reduction_and_logit_at_thread_edges(grid, gate_kind, lib):
         f = [np.float32(v) for v in log[t, cols]]
         z = O.gate_logit(f, g) if gate_kind == "mlp3" else O.gate_logit6(f, g)
         assert z == np.float32(log[t, 3]) and bool(log[t, 4]) == bool(z > 0), t
+
+
+@pytest.mark.parametrize("heads,hidden,grid,n_txt", [
+    (2, 128, (1, 1, 1), 1),      # 2 tokens: one query group, one key tile, seven warps without keys
+    (2, 128, (1, 3, 9), 5),      # 32 tokens: whole tiles
+    (3, 192, (1, 4, 7), 5),      # 33 tokens: one row and one key past a tile
+    (2, 256, (1, 1, 250), 7),    # 257 tokens, head width 128: a second round of key tiles
+    (2, 128, (1, 17, 29), 20),   # 513 tokens
+])
+def test_fp32_backbone_at_tile_edges(heads, hidden, grid, n_txt, lib):
+    """The fp32 projections (32 x 32 tiles, K in slices of 64 split over eight warps) and the
+    fp32 attention (eight queries a CTA, key tiles of 32 over eight warps): latents against
+    the fp64 oracle to 1e-5 of their RMS (fp32 sums over up to 640 products)."""
+    dh = hidden // heads
+    cfg = configs.get_config("tiny", hidden=hidden, heads=heads, mlp=4 * hidden, grid=grid, n_txt=n_txt, n_single=1,
+                             rope_axes=(0, 32, 32) if dh == 64 else (16, 56, 56))
+    ctx = bag.create(cfg, T=2, B=2)
+    inp = synth.make_inputs(cfg)
+    x = torch.from_numpy(inp["x"].copy()).cuda()
+    ctx.run(x, torch.from_numpy(inp["txt"]).cuda(), torch.from_numpy(inp["pooled"]).cuda())
+    ctx.close()
+    ref = O.sample(cfg, synth.make_weights(cfg), synth.make_gate(cfg["gate_seed"]), inp, T=2, B=2)["x"]
+    rms = float(np.sqrt(np.mean(ref ** 2)))
+    assert float(np.max(np.abs(x.cpu().numpy() - ref))) <= 1e-5 * rms
