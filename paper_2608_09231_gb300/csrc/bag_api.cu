@@ -767,6 +767,13 @@ static Epi base_epi(const bag_ctx* ctx, const DevState* st, int flag_want) {
   return e;
 }
 
+// Epilogue of a projection of the stack (see Epi::plan_rows).
+static Epi stack_epi(const bag_ctx* ctx, const DevState* st, int flag_want) {
+  Epi e = base_epi(ctx, st, flag_want);
+  e.plan_rows = ctx->arch.kind == BAG_KIND_WAN ? ctx->ni : ctx->N;
+  return e;
+}
+
 static inline void* off_act(const bag_ctx* ctx, void* p, long elems) {
   return (char*)p + elems * (long)ctx->act_size;
 }
@@ -995,11 +1002,11 @@ static void enq_block(Enq& q, int b, float* h, const DevState* st, int fw, int n
   };
   if (blk.type == BT_SINGLE) {
     ln_joint(mod, modu, mod, modu, 0);
-    Epi e = base_epi(ctx, st, fw);
+    Epi e = stack_epi(ctx, st, fw);
     enq_qkv_epi(ctx, e, 0, true);
     qk_norm(e, "");
     e.bias = (const float*)blk.w.at("lin1_b").p;
-    Epi r = base_epi(ctx, st, fw);
+    Epi r = stack_epi(ctx, st, fw);
     r.kind = EPI_GATED_RES;
     r.bias = (const float*)blk.w.at("lin2_b").p;
     r.resid = h;
@@ -1041,12 +1048,12 @@ static void enq_block(Enq& q, int b, float* h, const DevState* st, int fw, int n
     // attention half
     ln_joint(mt, mtu, mi, miu, 0);
     {
-      Epi e = base_epi(ctx, st, fw);
+      Epi e = stack_epi(ctx, st, fw);
       enq_qkv_epi(ctx, e, nx, true);
       e.bias = (const float*)blk.w.at("img_qkv_b").p;
       qk_norm(e, "img_");
       epi_branches(ctx, e, nb, ni, N, ctx->vpad);
-      Epi e2 = base_epi(ctx, st, fw);
+      Epi e2 = stack_epi(ctx, st, fw);
       enq_qkv_epi(ctx, e2, 0, true);
       e2.bias = (const float*)blk.w.at("txt_qkv_b").p;
       qk_norm(e2, "txt_");
@@ -1056,7 +1063,7 @@ static void enq_block(Enq& q, int b, float* h, const DevState* st, int fw, int n
     }
     attn_joint();
     {
-      Epi r = base_epi(ctx, st, fw);
+      Epi r = stack_epi(ctx, st, fw);
       r.kind = EPI_GATED_RES;
       r.bias = (const float*)blk.w.at("img_proj_b").p;
       r.resid = h_img;
@@ -1077,7 +1084,7 @@ static void enq_block(Enq& q, int b, float* h, const DevState* st, int fw, int n
     // MLP half
     ln_joint(mt, mtu, mi, miu, 3 * d);
     {
-      Epi u = base_epi(ctx, st, fw);
+      Epi u = stack_epi(ctx, st, fw);
       u.kind = EPI_GELU;
       u.out_bf16 = ctx->act_bf16;
       u.ldo = ldc;
@@ -1088,7 +1095,7 @@ static void enq_block(Enq& q, int b, float* h, const DevState* st, int fw, int n
       u2.out = off_act(ctx, ctx->cat, d);
       enq_gemm2(q, off_act(ctx, ctx->xn, ti * d), d, blk.w.at("img_up_w"), d, nb * ni, u,
                 ctx->xn, d, blk.w.at("txt_up_w"), d, nb * nx, u2, (int)F, (int)d);
-      Epi r = base_epi(ctx, st, fw);
+      Epi r = stack_epi(ctx, st, fw);
       r.kind = EPI_GATED_RES;
       r.bias = (const float*)blk.w.at("img_down_b").p;
       r.resid = h_img;
@@ -1114,7 +1121,7 @@ static void enq_block(Enq& q, int b, float* h, const DevState* st, int fw, int n
   const long vtw_br = v_br(ni, ctx->vpad), vtc_br = v_br(nx, ctx->vpad_c);
   enq_ln(q, h, d, ctx->xn, d, R, ni, mod, mod + d, modu, modu + d, st, fw);
   {
-    Epi e = base_epi(ctx, st, fw);
+    Epi e = stack_epi(ctx, st, fw);
     enq_qkv_epi(ctx, e, 0, true);
     e.bias = (const float*)blk.w.at("sa_qkv_b").p;
     epi_branches(ctx, e, nb, ni, ni, ctx->vpad);
@@ -1132,7 +1139,7 @@ static void enq_block(Enq& q, int b, float* h, const DevState* st, int fw, int n
              off_act(ctx, ctx->vt, br * vtw_br), ctx->vpad, off_act(ctx, ctx->cat, (long)br * ni * ldc),
              ldc, ni, ni, st, fw, nullptr, 0, ab);
   {
-    Epi r = base_epi(ctx, st, fw);
+    Epi r = stack_epi(ctx, st, fw);
     r.kind = EPI_GATED_RES;
     r.bias = (const float*)blk.w.at("sa_o_b").p;
     r.resid = h;
@@ -1145,14 +1152,14 @@ static void enq_block(Enq& q, int b, float* h, const DevState* st, int fw, int n
   }
   enq_ln(q, h, d, ctx->xn, d, R, 0, nullptr, nullptr, nullptr, nullptr, st, fw);
   {
-    Epi e = base_epi(ctx, st, fw);
+    Epi e = stack_epi(ctx, st, fw);
     e.kind = EPI_STORE;
     e.out = ctx->qc;
     e.ldo = d;
     e.out_bf16 = ctx->act_bf16 ? kStoreF16 : kStoreF32;  // an attention operand
     e.bias = (const float*)blk.w.at("ca_q_b").p;
     enq_gemm(q, ctx->xn, d, blk.w.at("ca_q_w"), d, R, (int)d, (int)d, e);
-    Epi kv = base_epi(ctx, st, fw);
+    Epi kv = stack_epi(ctx, st, fw);
     kv.kind = EPI_QKV;
     kv.q = nullptr;
     kv.k = ctx->kc;
@@ -1176,7 +1183,7 @@ static void enq_block(Enq& q, int b, float* h, const DevState* st, int fw, int n
              off_act(ctx, ctx->vtc, br * vtc_br), ctx->vpad_c, off_act(ctx, ctx->cat, (long)br * ni * ldc),
              ldc, ni, nx, st, fw, nullptr, 0, abc);
   {
-    Epi r = base_epi(ctx, st, fw);
+    Epi r = stack_epi(ctx, st, fw);
     r.kind = EPI_RES_ADD;
     r.bias = (const float*)blk.w.at("ca_o_b").p;
     r.resid = h;
@@ -1185,14 +1192,14 @@ static void enq_block(Enq& q, int b, float* h, const DevState* st, int fw, int n
   }
   enq_ln(q, h, d, ctx->xn, d, R, ni, mod + 3 * d, mod + 4 * d, modu + 3 * d, modu + 4 * d, st, fw);
   {
-    Epi u = base_epi(ctx, st, fw);
+    Epi u = stack_epi(ctx, st, fw);
     u.kind = EPI_GELU;
     u.out_bf16 = ctx->act_bf16;
     u.ldo = ldc;
     u.bias = (const float*)blk.w.at("ffn_up_b").p;
     u.out = off_act(ctx, ctx->cat, d);
     enq_gemm(q, ctx->xn, d, blk.w.at("ffn_up_w"), d, R, (int)F, (int)d, u);
-    Epi r = base_epi(ctx, st, fw);
+    Epi r = stack_epi(ctx, st, fw);
     r.kind = EPI_GATED_RES;
     r.bias = (const float*)blk.w.at("ffn_down_b").p;
     r.resid = h;

@@ -581,6 +581,237 @@ static cudaError_t launch_tc(const void* A0, long lda0, const void* W0, long ldw
 }
 
 // ---------------------------------------------------------------------------
+// Split-K GEMM: a cluster of S CTAs computes one 128 x 64 tile, each CTA a contiguous
+// share of the K blocks.  The CTAs then exchange accumulator rows through distributed
+// shared memory (rank o receives rows [o, o + 1) * 128 / S of every CTA), sum them in rank
+// order and apply the epilogue to their rows, so the result is deterministic.
+// Bound: latency.  A launch with few tiles leaves most SMs idle while each busy one takes
+// its operands at one SM's L2 rate (24 KB a K block, measured about 0.28 us); the split
+// divides that chain by S.  Epilogues that need whole heads or 32 x 32 blocks (EPI_QKV)
+// stay on the unsplit kernels.
+// Measured (profiled launches): 4096 x 64 x 3072 30.7 -> 16.3 us, 910 x 512 x 2560 19.0 -> 16.2,
+// 390 x 512 x 1536 16.1 -> 12.1, 378 x 64 x 512 17.2 -> 11.4.
+// ---------------------------------------------------------------------------
+constexpr int SK_BN = 64, SK_STAGES = 3, SK_LD = SK_BN + 4;
+constexpr int SK_A_BYTES = TC_BM * TC_BK * 2, SK_B_BYTES = SK_BN * TC_BK * 2;
+constexpr int SK_STAGE_BYTES = SK_A_BYTES + SK_B_BYTES;
+constexpr int SK_RECV_BYTES = TC_BM * SK_LD * 4;  // S slots of 128 / S rows
+constexpr int SK_SMEM = SK_STAGES * SK_STAGE_BYTES + SK_RECV_BYTES + 1024 + 256;
+
+BAG_DEV void st_cluster4(uint32_t addr, float a, float b, float c, float d) {
+  asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(a), "f"(b), "f"(c), "f"(d)
+               : "memory");
+}
+
+template <int S>
+__global__ void __launch_bounds__(192)
+    gemm_splitk_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUtensorMap tmB0,
+                       const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ CUtensorMap tmB1,
+                       const __grid_constant__ Epi e0, const __grid_constant__ Epi e1, int M0, int M1,
+                       int N, int K, int a_split, int* err) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
+                                             ~static_cast<uintptr_t>(1023));
+  uint8_t* sA = smem;
+  uint8_t* sB = smem + SK_STAGES * SK_A_BYTES;
+  float* recv = reinterpret_cast<float*>(smem + SK_STAGES * SK_STAGE_BYTES);
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + SK_STAGES * SK_STAGE_BYTES + SK_RECV_BYTES);
+  uint64_t* empty = full + SK_STAGES;
+  uint64_t* tfull = empty + SK_STAGES;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tfull + 1);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+
+  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  const int rank = (int)cluster_ctarank();
+  const int num_n = N / SK_BN, tiles0 = (M0 + TC_BM - 1) / TC_BM * num_n;
+  int tile = blockIdx.x / S;
+  const bool pb = tile >= tiles0;  // problem 1's tiles follow problem 0's
+  if (pb) tile -= tiles0;
+  const int mt = tile / num_n, nt = tile % num_n;
+  const CUtensorMap* tmA = pb ? &tmA1 : &tmA0;
+  const CUtensorMap* tmB = pb ? &tmB1 : &tmB0;
+  const Epi& e = pb ? e1 : e0;
+  const int kit = (a_split ? 2 : 1) * (K / TC_BK);
+  const int kb0 = rank * kit / S, kb1 = (rank + 1) * kit / S;
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < SK_STAGES; ++s) {
+      mbar_init(full + s, 1);
+      mbar_init(empty + s, 1);
+    }
+    mbar_init(tfull, 1);
+    *abort_flag = 0;
+    fence_mbar_init();
+    tma_prefetch_desc(tmA);
+    tma_prefetch_desc(tmB);
+  }
+  grid_dep_sync();
+  // every CTA of a cluster sees the same flag, so they leave together
+  if (epi_skip(e0.st, e0.flag_want)) return;
+  const int t = epi_step(e0);
+  __syncwarp();
+  if (warp == 1) {
+    tmem_alloc(tmem_slot, SK_BN);
+    tmem_relinquish();
+  }
+  tc_fence_before();
+  __syncwarp();
+  cluster_sync_all();  // barriers initialised, tensor memory allocated, every CTA running
+  tc_fence_after();
+  const uint32_t tmem_base = *tmem_slot;
+
+  if (warp == 0) {
+    if (lane == 0) {
+      // ---------------- TMA producer ----------------
+      int s = 0;
+      uint32_t ph = 0;
+      int issued = 0;
+      bool ok = true;
+      for (int kb = kb0; kb < kb1; ++kb) {
+        if (!mbar_wait(empty + s, ph ^ 1, abort_flag)) {
+          ok = false;
+          break;
+        }
+        mbar_arrive_expect_tx(full + s, SK_STAGE_BYTES);
+        const int ka = a_split ? (kb & 1) * K + (kb >> 1) * TC_BK : kb * TC_BK;
+        const int kw = a_split ? (kb >> 1) * TC_BK : kb * TC_BK;
+        tma_load_2d(sA + s * SK_A_BYTES, tmA, ka, mt * TC_BM, full + s);
+        tma_load_2d(sB + s * SK_B_BYTES, tmB, kw, nt * SK_BN, full + s);
+        ++issued;
+        if (++s == SK_STAGES) {
+          s = 0;
+          ph ^= 1;
+        }
+      }
+      if (!ok) {
+        // drain: wait (bounded) for the copies this thread may still have in flight
+        const uint64_t t0 = global_ns();
+        for (int i = 0; i < SK_STAGES && i < issued; ++i) {
+          if (--s < 0) {
+            s = SK_STAGES - 1;
+            ph ^= 1;
+          }
+          while (!mbar_try_wait(full + s, ph) && global_ns() - t0 < kWaitLimitNs) {
+          }
+        }
+      }
+    }
+  } else if (warp == 1) {
+    // ---------------- MMA issuer (converged warp, one elected lane issues) ----------------
+    constexpr uint32_t idesc = idesc_bf16_f32(TC_BM, SK_BN);
+    const uint32_t a_base = smem_u32(sA), b_base = smem_u32(sB);
+    int s = 0;
+    uint32_t ph = 0;
+    for (int kb = kb0; kb < kb1; ++kb) {
+      if (!mbar_wait_warp(full + s, ph, abort_flag)) break;
+      tc_fence_after();
+      const uint64_t ad = sw128_desc(a_base + s * SK_A_BYTES);
+      const uint64_t bd = sw128_desc(b_base + s * SK_B_BYTES);
+      if (elect_one()) {
+#pragma unroll
+        for (int k = 0; k < TC_BK / 16; ++k)
+          mma_bf16(tmem_base, ad + 2 * k, bd + 2 * k, idesc, (kb > kb0 || k > 0) ? 1u : 0u);
+        mma_commit(empty + s);
+      }
+      __syncwarp();
+      if (++s == SK_STAGES) {
+        s = 0;
+        ph ^= 1;
+      }
+    }
+    // all MMAs issued so far (whatever happened above) finish before tfull completes, and
+    // the bounded wait keeps tensor memory until then
+    if (elect_one()) {
+      mma_commit(tfull);
+      const uint64_t t0 = global_ns();
+      while (!mbar_try_wait(tfull, 0) && global_ns() - t0 < kWaitLimitNs) {
+      }
+    }
+    __syncwarp();
+  } else {
+    // ---------------- exchange: each warp's 32 accumulator rows to their owners ----------------
+    const int q = warp & 3;
+    const bool ok = mbar_wait(tfull, 0, abort_flag);
+    if (__all_sync(0xffffffffu, ok)) {
+      tc_fence_after();
+      constexpr int RPO = TC_BM / S;  // rows per owner
+      const int r = q * 32 + lane;
+      const uint32_t dst = mapa_shared(smem_u32(recv), (uint32_t)(r / RPO)) +
+                           (uint32_t)((rank * RPO + r % RPO) * SK_LD * 4);
+      const uint32_t tb = tmem_base + ((uint32_t)(q * 32) << 16);
+#pragma unroll
+      for (int c = 0; c < SK_BN; c += 32) {
+        float v[32];
+        tmem_ld32(tb + (uint32_t)c, v);
+#pragma unroll
+        for (int j = 0; j < 32; j += 4) st_cluster4(dst + (uint32_t)(c + j) * 4, v[j], v[j + 1], v[j + 2], v[j + 3]);
+      }
+    }
+  }
+  tc_fence_before();
+  __syncwarp();
+  cluster_sync_all();  // every CTA's rows have arrived; no access to another CTA follows
+  if (warp >= 2 && !*abort_flag) {
+    constexpr int RPO = TC_BM / S, NV = SK_BN / S;  // 128 threads: S per row, NV columns each
+    const int i = threadIdx.x - 64, lr = i / S, c = (i % S) * NV;
+    float v[NV];
+#pragma unroll
+    for (int j = 0; j < NV; ++j) v[j] = 0.f;
+#pragma unroll
+    for (int p = 0; p < S; ++p) {
+      float w[NV];
+      ld_chunk<NV>(recv + (p * RPO + lr) * SK_LD + c, w);
+#pragma unroll
+      for (int j = 0; j < NV; ++j) v[j] += w[j];
+    }
+    epi_apply<NV>(e, t, mt * TC_BM + rank * RPO + lr, nt * SK_BN + c, v);
+  }
+  if (threadIdx.x == 0 && *abort_flag && err) atomicOr(err, 1);
+  if (warp == 1) {
+    tc_fence_after();
+    tmem_dealloc(tmem_base, SK_BN);
+  }
+}
+
+// CTAs per tile for a launch of `tiles` 128 x 64 tiles and `kit` K blocks: the largest
+// split that leaves every CTA SK_MIN_KB blocks and keeps the launch within one CTA per SM
+// (1: the unsplit kernels).  A guided launch may hold twice the planned tiles; two CTAs fit
+// on an SM.
+#ifndef BAG_SPLITK_MIN_KB
+#define BAG_SPLITK_MIN_KB 4
+#endif
+static int splitk_ctas(int tiles, int kit, int ns) {
+  for (int s = 8; s > 1; s /= 2)
+    if (tiles * s <= ns && kit >= s * BAG_SPLITK_MIN_KB) return s;
+  return 1;
+}
+
+static cudaError_t launch_splitk(int S, const void* A0, long lda0, const void* W0, long ldw0, int M0,
+                                 const Epi& e0, const void* A1, long lda1, const void* W1, long ldw1,
+                                 int M1, const Epi& e1, int N, int K, int* err, cudaStream_t s,
+                                 int a_split) {
+  const uint64_t ka = (uint64_t)K * (a_split ? 2 : 1);
+  CUtensorMap ta0, tb0, ta1, tb1;
+  if (encode_tmap_2d_bf16(&ta0, A0, ka, (uint64_t)M0, (uint64_t)lda0 * 2, TC_BK, TC_BM) ||
+      encode_tmap_2d_bf16(&tb0, W0, (uint64_t)K, (uint64_t)N, (uint64_t)ldw0 * 2, TC_BK, SK_BN))
+    return cudaErrorInvalidValue;
+  if (M1 > 0) {
+    if (encode_tmap_2d_bf16(&ta1, A1, ka, (uint64_t)M1, (uint64_t)lda1 * 2, TC_BK, TC_BM) ||
+        encode_tmap_2d_bf16(&tb1, W1, (uint64_t)K, (uint64_t)N, (uint64_t)ldw1 * 2, TC_BK, SK_BN))
+      return cudaErrorInvalidValue;
+  } else {
+    ta1 = ta0;
+    tb1 = tb0;
+  }
+  const int tiles = ((M0 + TC_BM - 1) / TC_BM + (M1 + TC_BM - 1) / TC_BM) * (N / SK_BN);
+  auto launch = [&](auto kernel) {
+    return launch_cluster(kernel, (unsigned)S, (unsigned)(tiles * S), 192, SK_SMEM, s, ta0, tb0, ta1, tb1, e0, e1,
+                          M0, M1, N, K, a_split, err);
+  };
+  return S == 8 ? launch(gemm_splitk_kernel<8>) : (S == 4 ? launch(gemm_splitk_kernel<4>) : launch(gemm_splitk_kernel<2>));
+}
+
+// ---------------------------------------------------------------------------
 // CTA-pair GEMM: clusters of two CTAs compute 256 x 256 tiles with cta_group::2 MMAs
 // (M = 256, N = 256, K = 16 per instruction).  Each CTA stages its own 128 rows of A
 // and 128 rows of W per k-block (32 KB instead of the single-CTA 128 x 256 tile's
@@ -847,6 +1078,10 @@ cudaError_t kernels_init() {
                              TcCfg<64>::SMEM);
   if (r == cudaSuccess)
     r = cudaFuncSetAttribute(gemm_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, PR_SMEM);
+  const void* splitk[] = {(const void*)gemm_splitk_kernel<2>, (const void*)gemm_splitk_kernel<4>,
+                          (const void*)gemm_splitk_kernel<8>};
+  for (const void* k : splitk)
+    if (r == cudaSuccess) r = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, SK_SMEM);
   if (r == cudaSuccess)
     r = cudaFuncSetAttribute(gemm_simt_kernel<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SG_SMEM);
   if (r == cudaSuccess)
@@ -881,6 +1116,13 @@ static cudaError_t gemm_tc2(const void* A0, long lda0, const void* W0, long ldw0
   const bool qkn = e0.qn_q || (M1 > 0 && e1.qn_q);
   const int min_bn = qkn ? e0.dh : 64;
   if (qkn && (e0.dh % 32 || (M1 > 0 && e1.dh != e0.dh) || min_bn > 256)) return cudaErrorNotSupported;
+  if (e0.kind != EPI_QKV && (M1 <= 0 || e1.kind != EPI_QKV)) {
+    const int mtp = e0.plan_rows > 0 ? (e0.plan_rows + TC_BM - 1) / TC_BM : mt;
+    const int split = splitk_ctas(mtp * (N / SK_BN), (a_split ? 2 : 1) * (K / TC_BK), ns);
+    if (split > 1)
+      return launch_splitk(split, A0, lda0, W0, ldw0, M0, e0, A1, lda1, W1, ldw1, M1 > 0 ? M1 : 0, e1, N, K, err,
+                           s, a_split);
+  }
   if (gemm_uses_pair(M0, M1 > 0 ? M1 : 0, N))
     return launch_pair(A0, lda0, W0, ldw0, M0, e0, A1, lda1, W1, ldw1, M1 > 0 ? M1 : 0, e1, N, K, err, s,
                        a_split);

@@ -16,20 +16,35 @@ namespace bag {
 // and waiting (grid_dep_sync) when its predecessor completes.
 extern thread_local bool g_pdl;
 
+// cluster: CTAs per cluster along x (0: the kernel's own, if any)
 template <typename... P, typename... A>
-inline cudaError_t launch_kernel(void (*k)(P...), dim3 grid, dim3 block, size_t smem,
-                                 cudaStream_t s, A&&... args) {
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
+inline cudaError_t launch_cluster(void (*k)(P...), unsigned cluster, dim3 grid, dim3 block, size_t smem,
+                                  cudaStream_t s, A&&... args) {
+  cudaLaunchAttribute at[2];
+  unsigned n = 0;
+  if (g_pdl) {
+    at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[n++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (cluster) {
+    at[n].id = cudaLaunchAttributeClusterDimension;
+    at[n].val.clusterDim.x = cluster;
+    at[n].val.clusterDim.y = 1;
+    at[n++].val.clusterDim.z = 1;
+  }
   cudaLaunchConfig_t c = {};
   c.gridDim = grid;
   c.blockDim = block;
   c.dynamicSmemBytes = smem;
   c.stream = s;
   c.attrs = at;
-  c.numAttrs = g_pdl ? 1 : 0;
+  c.numAttrs = n;
   return cudaLaunchKernelEx(&c, k, std::forward<A>(args)...);
+}
+template <typename... P, typename... A>
+inline cudaError_t launch_kernel(void (*k)(P...), dim3 grid, dim3 block, size_t smem,
+                                 cudaStream_t s, A&&... args) {
+  return launch_cluster(k, 0u, grid, block, smem, s, std::forward<A>(args)...);
 }
 
 // Per-sample state the step kernels read and write on the device, so that a whole
@@ -132,6 +147,10 @@ struct Epi {
   float* uni_xl = nullptr;
   float* uni_m0 = nullptr;
   float* uni_m1 = nullptr;
+  // rows the launch is planned for when the split of K is chosen (0: its own rows).  The
+  // stack sets one branch's rows, so that a guided sample, whose launches hold both
+  // branches' rows, sums in the same order and gives the same bits as an unguided one.
+  int plan_rows = 0;
   // step-dependent addressing and early exit
   const DevState* st = nullptr;  // null: step 0, no flag check
   int flag_want = -1;            // -1: always run; 0/1: run only when st->flag equals it

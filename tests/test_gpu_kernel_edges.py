@@ -58,3 +58,33 @@ def test_fp32_backbone_at_tile_edges(heads, hidden, grid, n_txt, lib):
     ref = O.sample(cfg, synth.make_weights(cfg), synth.make_gate(cfg["gate_seed"]), inp, T=2, B=2)["x"]
     rms = float(np.sqrt(np.mean(ref ** 2)))
     assert float(np.max(np.abs(x.cpu().numpy() - ref))) <= 1e-5 * rms
+
+
+@pytest.mark.parametrize("M,N,K", [
+    (1, 64, 512),        # one row, two CTAs of four K blocks
+    (127, 64, 64 * 9),   # nine blocks over two CTAs
+    (129, 128, 64 * 17), # four CTAs, 4 or 5 blocks each, one row in the last row tile
+    (300, 192, 64 * 35), # eight CTAs
+    (1100, 512, 1024),   # 72 tiles: two CTAs
+    (640, 1024, 2048),   # 80 tiles: not split
+])
+@pytest.mark.parametrize("epilogue", [0, 1])
+def test_split_k_gemm(M, N, K, epilogue, lib):
+    """Shapes around the split-K rule (tiles x CTAs against the SM count, K blocks per CTA)
+    against fp64: a bf16 product's fp32 sum over K, bounded by 4 K 2^-24 sum|a||w|."""
+    ctx = bag.create("tiny", T=2, B=1)
+    g = torch.Generator(device="cuda").manual_seed(M + N + K)
+    A = torch.randn(M, K, generator=g, device="cuda").bfloat16()
+    W = (0.05 * torch.randn(N, K, generator=g, device="cuda")).bfloat16()
+    bias = 0.1 * torch.randn(N, generator=g, device="cuda")
+    C = torch.full((M + 1, N), -7.0, device="cuda")
+    ctx.gemm_bf16(A, W, bias, C, M, N, K, epilogue)
+    torch.cuda.synchronize()
+    ctx.close()
+    ref = A.double() @ W.double().T + bias.double()
+    # GELU's slope is at most 1.13
+    bound = 1.2 * (4 * K * 2.0 ** -24 * (A.double().abs() @ W.double().abs().T) + 1e-6)
+    if epilogue:
+        ref = torch.nn.functional.gelu(ref, approximate="tanh")
+    assert bool(((C[:M].double() - ref).abs() <= bound).all())
+    assert bool((C[M] == -7.0).all())
