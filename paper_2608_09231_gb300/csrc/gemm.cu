@@ -774,14 +774,15 @@ __global__ void __launch_bounds__(192)
 }
 
 // CTAs per tile for a launch of `tiles` 128 x 64 tiles and `kit` K blocks: the largest
-// split that leaves every CTA SK_MIN_KB blocks and keeps the launch within one CTA per SM
+// split, up to 4, that leaves every CTA SK_MIN_KB blocks and keeps the launch within one CTA
+// per SM (clusters of eight leave 32 of the 152 SMs without a place)
 // (1: the unsplit kernels).  A guided launch may hold twice the planned tiles; two CTAs fit
 // on an SM.
 #ifndef BAG_SPLITK_MIN_KB
 #define BAG_SPLITK_MIN_KB 4
 #endif
 static int splitk_ctas(int tiles, int kit, int ns) {
-  for (int s = 8; s > 1; s /= 2)
+  for (int s = 4; s > 1; s /= 2)
     if (tiles * s <= ns && kit >= s * BAG_SPLITK_MIN_KB) return s;
   return 1;
 }
@@ -808,7 +809,7 @@ static cudaError_t launch_splitk(int S, const void* A0, long lda0, const void* W
     return launch_cluster(kernel, (unsigned)S, (unsigned)(tiles * S), 192, SK_SMEM, s, ta0, tb0, ta1, tb1, e0, e1,
                           M0, M1, N, K, a_split, err);
   };
-  return S == 8 ? launch(gemm_splitk_kernel<8>) : (S == 4 ? launch(gemm_splitk_kernel<4>) : launch(gemm_splitk_kernel<2>));
+  return S == 4 ? launch(gemm_splitk_kernel<4>) : launch(gemm_splitk_kernel<2>);
 }
 
 // ---------------------------------------------------------------------------
@@ -1078,8 +1079,7 @@ cudaError_t kernels_init() {
                              TcCfg<64>::SMEM);
   if (r == cudaSuccess)
     r = cudaFuncSetAttribute(gemm_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, PR_SMEM);
-  const void* splitk[] = {(const void*)gemm_splitk_kernel<2>, (const void*)gemm_splitk_kernel<4>,
-                          (const void*)gemm_splitk_kernel<8>};
+  const void* splitk[] = {(const void*)gemm_splitk_kernel<2>, (const void*)gemm_splitk_kernel<4>};
   for (const void* k : splitk)
     if (r == cudaSuccess) r = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, SK_SMEM);
   if (r == cudaSuccess)
