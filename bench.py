@@ -164,7 +164,7 @@ def oracle_s_per_sample(cfg, B, rep):
 # ---------------------------------------------------------------------------
 KERNEL_NAMES = {"gemm": "gemm_tc_kernel", "attention": "attn_tc_kernel",
                 "norm": "ln_mod_kernel", "signal": "ln_mod_kernel (signal)",
-                "gate": "gate_kernel", "cache": "cache_refresh/reuse_kernel"}
+                "gate": "gate_kernel", "cache": "stream_init_kernel"}
 KERNEL_SOURCES = {"gemm_tc_kernel": ["gemm.cu", "epilogue.cuh", "common.cuh"],
                   "gemm_pair_kernel": ["gemm.cu", "epilogue.cuh", "common.cuh"],
                   "attn_tc_kernel": ["attn_tc.cu", "common.cuh"]}

@@ -244,7 +244,7 @@ enum {
   BAG_PROF_NORM = 2,   /* LayerNorm + modulation inside the stack and the final layer */
   BAG_PROF_SIGNAL = 3, /* trajectory signal (block-0 LN-mod fused with the rel-L1 partials) */
   BAG_PROF_GATE = 4,   /* gate + pacing */
-  BAG_PROF_CACHE = 5,  /* cache refresh (full step) and residual reuse (cached step) */
+  BAG_PROF_CACHE = 5,  /* stream set-up of a full step (the cache itself is part of the final norm) */
   BAG_PROF_KINDS = 6
 };
 typedef struct {

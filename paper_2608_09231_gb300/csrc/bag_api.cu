@@ -161,7 +161,7 @@ struct bag_ctx {
   cudaStream_t cap_stream = nullptr;
   int use_graph = 1;
   bool pdl = true;  // programmatic dependent launch between the kernels of a segment
-  long n_prefix = 0, n_full = 0, n_skip = 0, n_suffix = 0, n_prepare = 0;
+  long n_prefix = 0, n_full = 0, n_suffix = 0, n_prepare = 0;
   long launches = 0;
 
   int next_t = 0;
@@ -811,43 +811,43 @@ static void enq_gemm2(Enq& q, const void* A0, long lda0, const Tensor& W0, long 
               q.ctx->st ? &q.ctx->st->err : nullptr, q.s));
 }
 
-static void enq_ln(Enq& q, const float* x, long ldx, void* y, long ldy, int rows, int split,
-                   const float* sh_a, const float* sc_a, const float* sh_b, const float* sc_b,
-                   const DevState* st, int flag_want) {
+// LayerNorm of `rows` rows of the hidden width, x fp32 and y in the operand precision, both
+// row-contiguous; segments and modulation left to the caller.
+static LnArgs ln_args(const bag_ctx* ctx, const float* x, void* y, int rows, const DevState* st, int flag_want) {
   LnArgs a{};
   a.x = x;
-  a.ldx = ldx;
+  a.ldx = ctx->d;
   a.y = y;
-  a.ldy = ldy;
-  a.y_bf16 = q.ctx->act_bf16;
+  a.ldy = ctx->d;
+  a.y_bf16 = ctx->act_bf16;
   a.rows = rows;
-  a.cols = q.ctx->d;
+  a.cols = (int)ctx->d;
+  a.mod_step = ctx->mod_stride;
+  a.st = st;
+  a.flag_want = flag_want;
+  return a;
+}
+
+static void enq_ln(Enq& q, const float* x, void* y, int rows, int split,
+                   const float* sh_a, const float* sc_a, const float* sh_b, const float* sc_b,
+                   const DevState* st, int flag_want) {
+  LnArgs a = ln_args(q.ctx, x, y, rows, st, flag_want);
   a.split = split;
   a.shift_a = sh_a;
   a.scale_a = sc_a;
   a.shift_b = sh_b;
   a.scale_b = sc_b;
-  a.mod_step = q.ctx->mod_stride;
-  a.st = st;
-  a.flag_want = flag_want;
   q.pre(BAG_PROF_NORM, 0.0, (double)rows * q.ctx->d * (4.0 + q.ctx->act_size));
   q.chk(ln_mod(a, q.s));
 }
 
 // LayerNorm + modulation with four row segments [0, s1), [s1, s2), [s2, s3), [s3, rows),
 // each under its own modulation (shift at m, scale at m + d).
-static void enq_ln4(Enq& q, const float* x, long ldx, void* y, long ldy, int rows, int s1, int s2, int s3,
+static void enq_ln4(Enq& q, const float* x, void* y, int rows, int s1, int s2, int s3,
                     const float* ma, const float* mb, const float* mc, const float* md, const DevState* st,
                     int flag_want) {
   const long d = q.ctx->d;
-  LnArgs a{};
-  a.x = x;
-  a.ldx = ldx;
-  a.y = y;
-  a.ldy = ldy;
-  a.y_bf16 = q.ctx->act_bf16;
-  a.rows = rows;
-  a.cols = (int)d;
+  LnArgs a = ln_args(q.ctx, x, y, rows, st, flag_want);
   a.split = s1;
   a.split2 = s2;
   a.split3 = s3;
@@ -859,9 +859,6 @@ static void enq_ln4(Enq& q, const float* x, long ldx, void* y, long ldy, int row
   a.scale_c = mc + d;
   a.shift_d = md;
   a.scale_d = md + d;
-  a.mod_step = q.ctx->mod_stride;
-  a.st = st;
-  a.flag_want = flag_want;
   q.pre(BAG_PROF_NORM, 0.0, (double)rows * d * (4.0 + q.ctx->act_size));
   q.chk(ln_mod(a, q.s));
 }
@@ -972,10 +969,10 @@ static void enq_block(Enq& q, int b, float* h, const DevState* st, int fw, int n
   auto ln_joint = [&](const float* mt_c, const float* mt_u, const float* mi_c, const float* mi_u,
                       long off) {
     if (nb == 1) {
-      enq_ln(q, h, d, ctx->xn, d, N, nx, mt_c + off, mt_c + off + d, mi_c + off, mi_c + off + d, st, fw);
+      enq_ln(q, h, ctx->xn, N, nx, mt_c + off, mt_c + off + d, mi_c + off, mi_c + off + d, st, fw);
       return;
     }
-    enq_ln4(q, h, d, ctx->xn, d, 2 * N, nx, 2 * nx, 2 * nx + ni, mt_c + off, mt_u + off, mi_c + off,
+    enq_ln4(q, h, ctx->xn, 2 * N, nx, 2 * nx, 2 * nx + ni, mt_c + off, mt_u + off, mi_c + off,
             mi_u + off, st, fw);
   };
   // attention of every branch: q / k / v of branch br at row br * N (transposed V at
@@ -1119,7 +1116,7 @@ static void enq_block(Enq& q, int b, float* h, const DevState* st, int fw, int n
   // [image_c; image_u] and the staged contexts [context_c; context_u]
   const int R = nb * ni;
   const long vtw_br = v_br(ni, ctx->vpad), vtc_br = v_br(nx, ctx->vpad_c);
-  enq_ln(q, h, d, ctx->xn, d, R, ni, mod, mod + d, modu, modu + d, st, fw);
+  enq_ln(q, h, ctx->xn, R, ni, mod, mod + d, modu, modu + d, st, fw);
   {
     Epi e = stack_epi(ctx, st, fw);
     enq_qkv_epi(ctx, e, 0, true);
@@ -1150,7 +1147,7 @@ static void enq_block(Enq& q, int b, float* h, const DevState* st, int fw, int n
     if (nb > 1) r.br_rows = ni;
     enq_gemm(q, ctx->cat, ldc, blk.w.at("sa_o_w"), d, R, (int)d, (int)d, r);
   }
-  enq_ln(q, h, d, ctx->xn, d, R, 0, nullptr, nullptr, nullptr, nullptr, st, fw);
+  enq_ln(q, h, ctx->xn, R, 0, nullptr, nullptr, nullptr, nullptr, st, fw);
   {
     Epi e = stack_epi(ctx, st, fw);
     e.kind = EPI_STORE;
@@ -1190,7 +1187,7 @@ static void enq_block(Enq& q, int b, float* h, const DevState* st, int fw, int n
     r.ldr = d;
     enq_gemm(q, ctx->cat, ldc, blk.w.at("ca_o_w"), d, R, (int)d, (int)d, r);
   }
-  enq_ln(q, h, d, ctx->xn, d, R, ni, mod + 3 * d, mod + 4 * d, modu + 3 * d, modu + 4 * d, st, fw);
+  enq_ln(q, h, ctx->xn, R, ni, mod + 3 * d, mod + 4 * d, modu + 3 * d, modu + 4 * d, st, fw);
   {
     Epi u = stack_epi(ctx, st, fw);
     u.kind = EPI_GELU;
@@ -1222,17 +1219,17 @@ static void enq_prefix(Enq& q, int use_cond, unsigned long long handle) {
   bag_ctx* ctx = q.ctx;
   const long d = ctx->d;
   Epi pe = base_epi(ctx, ctx->st, -1);
-  pe.kind = EPI_DUAL_F32;
+  pe.kind = EPI_STORE;
   pe.bias = (const float*)ctx->G.at("pe_b").p;
   pe.out = ctx->h_in;
   pe.ldo = d;
-  pe.out2 = img_stream(ctx);
-  pe.ldo2 = d;
+  pe.out_bf16 = kStoreF32;
+  pe.bump = ctx->st;  // DevState::t is -1 before a sample's first step
   if (ctx->act_bf16) {
     // the latent enters as bf16 hi + lo halves (split A): the patch embedding, and with
     // it the post-patch-embedding observable, carries no bf16 rounding of x
     q.pre(BAG_PROF_GEMM, 4.0 * ctx->ni * d * ctx->C,
-          ((double)ctx->ni * 2 + d) * ctx->C * 2 + (double)ctx->ni * d * 8, ctx->ni, (int)d, 2 * ctx->C,
+          ((double)ctx->ni * 2 + d) * ctx->C * 2 + (double)ctx->ni * d * 4, ctx->ni, (int)d, 2 * ctx->C,
           gemm_uses_pair(ctx->ni, 0, (int)d));
     q.chk(gemm(ctx->xb, 2L * ctx->C, ctx->G.at("pe_w").p, ctx->C, ctx->ni, (int)d, ctx->C, 1, pe,
                ctx->st ? &ctx->st->err : nullptr, q.s, 0, 1));
@@ -1275,49 +1272,42 @@ static void enq_prefix(Enq& q, int use_cond, unsigned long long handle) {
                   ctx->policy, ctx->d_pmask, ctx->delta, ctx->log, handle, use_cond, q.s));
 }
 
-// Full step: the whole stack for every branch, then each branch's residual is cached
-// (and the conditional branch's signal observable m_t becomes m_last).
+// Full step: the stream is set up from the text and the patch-embedded latent, then the
+// whole stack runs once for all branches (every projection takes both branches' rows).
+// A reused step runs nothing here: the final layer's pass adds the cached residual.
 static void enq_full(Enq& q, int fw) {
   bag_ctx* ctx = q.ctx;
-  const long d = ctx->d;
   const int nb = n_branches(ctx);
-  for (int br = 0; br < nb; ++br) {
-    if (ctx->arch.kind != BAG_KIND_WAN)
-      q.chk(copy_rows_f32(ctx->st, fw, ctx->hj + (long)br * ctx->nx * d, d, br_txt(ctx, br), d, ctx->act_bf16,
-                          ctx->nx, (int)d, q.s));
-    if (br) {  // the patch-embed epilogue filled only the conditional stream's image rows
-      q.pre(BAG_PROF_CACHE, 0.0, (double)ctx->ni * d * 8.0);
-      q.chk(copy_rows_f32(ctx->st, fw, img_stream(ctx, br), d, ctx->h_in, d, 0, ctx->ni, (int)d, q.s));
-    }
-  }
-  // the stack once for all branches (every projection takes both branches' rows)
+  const int nx = ctx->arch.kind == BAG_KIND_WAN ? 0 : ctx->nx;  // a Wan stream holds no text
+  q.pre(BAG_PROF_CACHE, 0.0, (double)nb * (ctx->ni * 8.0 + nx * (4.0 + ctx->act_size)) * ctx->d);
+  q.chk(stream_init(ctx->st, fw, ctx->hj, br_txt(ctx, 0), br_txt(ctx, nb - 1), ctx->act_bf16, ctx->h_in, nb, nx,
+                    ctx->ni, (int)ctx->d, q.s));
   for (int b = 0; b < ctx->nblk; ++b) enq_block(q, b, ctx->hj, ctx->st, fw, nb);
-  for (int br = 0; br < nb; ++br) {
-    q.pre(BAG_PROF_CACHE, 0.0, (double)ctx->ni * d * 12.0);
-    q.chk(cache_refresh(ctx->st, img_stream(ctx, br), ctx->h_in, br ? ctx->R_u : ctx->R,
-                        (long)ctx->ni * d, fw, q.s));
-  }
 }
 
-// Cached step: every branch adds its own cached residual (one shared mask, App. A.1).
-static void enq_skip(Enq& q, int fw) {
-  bag_ctx* ctx = q.ctx;
-  for (int br = 0; br < n_branches(ctx); ++br) {
-    q.pre(BAG_PROF_CACHE, 0.0, (double)ctx->ni * ctx->d * 12.0);
-    q.chk(cache_reuse(ctx->st, img_stream(ctx, br), ctx->h_in, br ? ctx->R_u : ctx->R,
-                      (long)ctx->ni * ctx->d, fw, q.s));
-  }
-}
-
-// Final layer and Euler update.  Under guidance the conditional velocity is stored and
+// Final layer and Euler update.  The LayerNorm pass reads every branch's image rows (a full
+// step: from the stream, caching the residual; a reused step: h_in plus the cached residual;
+// one shared mask, App. A.1).  Under guidance the conditional velocity is stored and
 // the unconditional branch's final GEMM applies v_u + g (v_c - v_u) in its epilogue.
 static void enq_suffix(Enq& q) {
   bag_ctx* ctx = q.ctx;
   const long d = ctx->d;
   const int nb = n_branches(ctx);
+  const float* fm0 = br_mod(ctx, 0) + ctx->fmod_off;
+  const float* fm1 = br_mod(ctx, nb - 1) + ctx->fmod_off;
+  LnArgs a = ln_args(ctx, img_stream(ctx), ctx->xn, nb * ctx->ni, ctx->st, -1);
+  a.split = ctx->ni;
+  a.shift_a = fm0;
+  a.scale_a = fm0 + d;
+  a.shift_b = fm1;
+  a.scale_b = fm1 + d;
+  a.cache_in = ctx->h_in;
+  a.cache_r = ctx->R;
+  a.cache_r2 = ctx->R_u;
+  // reads two fp32 rows (stream and h_in, or h_in and cache); a full step writes the cache
+  q.pre(BAG_PROF_NORM, 0.0, (double)nb * ctx->ni * d * (8.0 + ctx->act_size));
+  q.chk(ln_mod(a, q.s));
   for (int br = 0; br < nb; ++br) {
-    const float* fm = br_mod(ctx, br) + ctx->fmod_off;
-    enq_ln(q, img_stream(ctx, br), d, ctx->xn, d, ctx->ni, 0, fm, fm + d, fm, fm + d, ctx->st, -1);
     Epi e = base_epi(ctx, ctx->st, -1);
     e.bias = (const float*)ctx->G.at("fin_b").p;
     if (br + 1 < nb) {
@@ -1342,9 +1332,8 @@ static void enq_suffix(Enq& q) {
         e.uni_m1 = ctx->uni_m1;
       }
     }
-    enq_gemm(q, ctx->xn, d, ctx->G.at("fin_w"), d, ctx->ni, ctx->C, (int)d, e);
+    enq_gemm(q, off_act(ctx, ctx->xn, (long)br * ctx->ni * d), d, ctx->G.at("fin_w"), d, ctx->ni, ctx->C, (int)d, e);
   }
-  q.chk(advance_step(ctx->st, q.s));
 }
 
 // Per-sample conditioning: time embedding and every modulation vector for all T steps
@@ -1437,8 +1426,7 @@ static void destroy_graph(bag_ctx* ctx) {
   ctx->graph = nullptr;
 }
 
-// Capture one step: prefix, conditional node (body 0: full network; body 1: reuse),
-// suffix.  The gate kernel sets the condition on the device.
+// Capture one step: prefix, conditional node (the full network), suffix.  The gate kernel sets the condition on the device.
 static bag_status build_graph(bag_ctx* ctx) {
   destroy_graph(ctx);
   cudaStream_t s = ctx->stream;
@@ -1462,30 +1450,22 @@ static bag_status build_graph(bag_ctx* ctx) {
     p.type = cudaGraphNodeTypeConditional;
     p.conditional.handle = handle;
     p.conditional.type = cudaGraphCondTypeIf;
-    p.conditional.size = 2;
+    p.conditional.size = 1;
     e = cudaGraphAddNode(&cnode, cg, deps, nullptr, ndeps, &p);
   }
   if (e == cudaSuccess) e = cudaStreamUpdateCaptureDependencies(s, &cnode, nullptr, 1, cudaStreamSetCaptureDependencies);
   if (e == cudaSuccess) {
-    cudaGraph_t bodies[2] = {p.conditional.phGraph_out[0], p.conditional.phGraph_out[1]};
-    for (int bi = 0; bi < 2 && e == cudaSuccess; ++bi) {
-      e = cudaStreamBeginCaptureToGraph(ctx->cap_stream, bodies[bi], nullptr, nullptr, 0,
-                                        cudaStreamCaptureModeThreadLocal);
-      if (e != cudaSuccess) break;
+    e = cudaStreamBeginCaptureToGraph(ctx->cap_stream, p.conditional.phGraph_out[0], nullptr, nullptr, 0,
+                                      cudaStreamCaptureModeThreadLocal);
+    if (e == cudaSuccess) {
       long c2 = 0;
       Enq qb{ctx, ctx->cap_stream, &c2};
-      if (bi == 0)
-        enq_full(qb, 1);
-      else
-        enq_skip(qb, 0);
+      enq_full(qb, 1);
       cudaGraph_t tmp;
       cudaError_t e2 = cudaStreamEndCapture(ctx->cap_stream, &tmp);
       if (qb.e != cudaSuccess) e = qb.e;
       if (e2 != cudaSuccess && e == cudaSuccess) e = e2;
-      if (bi == 0)
-        ctx->n_full = c2;
-      else
-        ctx->n_skip = c2;
+      ctx->n_full = c2;
     }
   }
   cnt = 0;
@@ -1508,7 +1488,7 @@ static bag_status build_graph(bag_ctx* ctx) {
 }
 
 // Enqueue one step.  Graph mode replays the captured step; direct mode launches every
-// kernel and the two bodies' kernels skip themselves on the device flag.
+// kernel and the stack's kernels skip themselves on the device flag.
 static bag_status launch_step(bag_ctx* ctx) {
   if (ctx->use_graph) {
     if (!ctx->exec) CKS(build_graph(ctx));
@@ -1519,7 +1499,6 @@ static bag_status launch_step(bag_ctx* ctx) {
   Enq q{ctx, ctx->stream, &cnt};
   enq_prefix(q, 0, 0);
   enq_full(q, 1);
-  enq_skip(q, 0);
   enq_suffix(q);
   if (q.e != cudaSuccess) return fail(ctx, BAG_ECUDA, std::string("step: ") + cudaGetErrorString(q.e));
   return BAG_OK;
@@ -1552,10 +1531,7 @@ static bag_status profile_run_impl(bag_ctx* ctx, float* x_inout, const bag_cond*
         break;
       }
       nfe += flag;
-      if (flag)
-        enq_full(q, 1);
-      else
-        enq_skip(q, 0);
+      if (flag) enq_full(q, 1);
       enq_suffix(q);
       if (q.e != cudaSuccess) s = fail(ctx, BAG_ECUDA, std::string("profile step: ") + cudaGetErrorString(q.e));
     }
@@ -1596,7 +1572,7 @@ static bag_status check_device_error(bag_ctx* ctx) {
 
 static bag_status reset_state(bag_ctx* ctx) {
   DevState h{};
-  h.t = 0;
+  h.t = -1;  // the first step's first kernel advances it to 0
   h.c = 0;
   h.t_last = -1;
   CK(cudaMemcpyAsync(ctx->st, &h, sizeof(h), cudaMemcpyHostToDevice, ctx->stream));
@@ -1671,8 +1647,7 @@ static bag_status bag_run_impl(bag_ctx* ctx, float* x_inout, const bag_cond* con
   }
   CK(cudaStreamSynchronize(ctx->stream));
   const long per_step = ctx->n_prefix + ctx->n_suffix;
-  ctx->launches = ctx->n_prepare + 2 + (long)ctx->T * per_step + (long)h.c * ctx->n_full +
-                  (long)(ctx->T - h.c) * ctx->n_skip;
+  ctx->launches = ctx->n_prepare + 2 + (long)ctx->T * per_step + (long)h.c * ctx->n_full;
   if (stats) {
     stats->T = ctx->T;
     stats->B = ctx->B;

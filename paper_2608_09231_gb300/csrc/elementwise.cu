@@ -7,9 +7,10 @@
 //    inputs, evaluates the 3->16->1 gate in fp32 with every product and sum rounded
 //    separately, applies Algorithm 2's two forced rules, updates the counters and the
 //    step log, and hands the decision to a CUDA-graph conditional node.
-//  * cache_refresh / cache_reuse: R = h_out - h_in after a full step; h_out = h_in + R
-//    on a reused step (plain residual reuse).
-//  * small helpers: step counter, sinusoidal timestep features, seeded fills.
+//    The final layer's ln_mod also keeps the residual cache: R = h_out - h_in on a full
+//    step, h_out = h_in + R on a reused one (plain residual reuse).
+//  * stream_init: the residual stream a full step starts from.
+//  * small helpers: sinusoidal timestep features, seeded fills.
 #include <cmath>
 
 #include "common.cuh"
@@ -113,7 +114,12 @@ BAG_DEV void copy4(void* dst, const void* src, long off, int bf16) {
 // VPT float4 per thread (cols <= 128 * 4 * VPT): the row stays in registers, and the
 // smallest VPT that holds it keeps the register count low enough for many rows per SM
 // (the kernel is latency-bound at low occupancy).
-template <int VPT>
+//
+// CACHE: the final layer's pass also keeps the residual cache (see LnArgs).  As passes of
+// their own, the cache update or the reuse (12 bytes an element each) and this pass took
+// 26 + 20 us on 4096 x 3072 (profiled launches), together they take 29 us; and the patch
+// embedding, which no longer writes the stream's copy on every step, 60 -> 39 us.
+template <int VPT, bool CACHE>
 __global__ void __launch_bounds__(LN_THREADS, VPT <= 6 ? 8 : (VPT <= 10 ? 5 : 4)) ln_mod_kernel(const LnArgs a) {
   grid_dep_sync();
   if (epi_skip(a.st, a.flag_want)) return;
@@ -138,11 +144,38 @@ __global__ void __launch_bounds__(LN_THREADS, VPT <= 6 ? 8 : (VPT <= 10 ? 5 : 4)
   const int nv = a.cols / 4;
   float4 v[VPT];
   float s = 0.f;
+  if constexpr (CACHE) {
+    const bool second = row >= a.split;
+    const long crow = (long)(second ? row - a.split : row) * a.ldx;
+    const float4* hin = reinterpret_cast<const float4*>(a.cache_in + crow);
+    float4* R = reinterpret_cast<float4*>((second ? a.cache_r2 : a.cache_r) + crow);
+    const bool full = a.st->flag != 0;
+    const float4* src = full ? reinterpret_cast<const float4*>(x) : R;
+    float4 h[VPT];
+#pragma unroll
+    for (int i = 0; i < VPT; ++i) {
+      const int c = threadIdx.x + i * LN_THREADS;
+      if (c < nv) {
+        v[i] = src[c];
+        h[i] = hin[c];
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < VPT; ++i) {
+      const int c = threadIdx.x + i * LN_THREADS;
+      if (c < nv) {
+        if (full)
+          R[c] = make_float4(v[i].x - h[i].x, v[i].y - h[i].y, v[i].z - h[i].z, v[i].w - h[i].w);
+        else
+          v[i] = make_float4(h[i].x + v[i].x, h[i].y + v[i].y, h[i].z + v[i].z, h[i].w + v[i].w);
+      }
+    }
+  }
 #pragma unroll
   for (int i = 0; i < VPT; ++i) {
     const int c = threadIdx.x + i * LN_THREADS;
     if (c < nv) {
-      v[i] = reinterpret_cast<const float4*>(x)[c];
+      if constexpr (!CACHE) v[i] = reinterpret_cast<const float4*>(x)[c];
       s += (v[i].x + v[i].y) + (v[i].z + v[i].w);
     }
   }
@@ -264,12 +297,15 @@ cudaError_t ln_mod(const LnArgs& args, cudaStream_t s) {
                        (a.ldy * (a.y_bf16 ? 2 : 4)) % 16 == 0;
   const int per_sm = a.cols <= LN_THREADS * 4 * 6 ? 8 : (a.cols <= LN_THREADS * 4 * 10 ? 5 : 4);
   a.prefetch_rows = (a.sig_on && aligned) ? sm_count() * per_sm : 0;
+  auto launch = [&](auto plain, auto cache) {
+    launch_kernel(a.cache_in ? cache : plain, a.rows, LN_THREADS, 0, s, a);
+  };
   if (a.cols <= LN_THREADS * 4 * 6)
-    launch_kernel(ln_mod_kernel<6>, a.rows, LN_THREADS, 0, s, a);
+    launch(ln_mod_kernel<6, false>, ln_mod_kernel<6, true>);
   else if (a.cols <= LN_THREADS * 4 * 10)
-    launch_kernel(ln_mod_kernel<10>, a.rows, LN_THREADS, 0, s, a);
+    launch(ln_mod_kernel<10, false>, ln_mod_kernel<10, true>);
   else
-    launch_kernel(ln_mod_kernel<LN_MAXV>, a.rows, LN_THREADS, 0, s, a);
+    launch(ln_mod_kernel<LN_MAXV, false>, ln_mod_kernel<LN_MAXV, true>);
   return cudaGetLastError();
 }
 
@@ -497,29 +533,13 @@ cudaError_t gate_step(DevState* st, const float* sig_partial, int sig_rows, cons
   return cudaGetLastError();
 }
 
-// ---------------------------------------------------------------------------
-// residual cache
-// ---------------------------------------------------------------------------
-// (the drift reference m_last <- m_t is taken over by the next step's signal pass)
-__global__ void cache_refresh_kernel(const DevState* st, int flag_want, const float4* h_img,
-                                     const float4* h_in, float4* R, long n4) {
+// out = a + b
+__global__ void residual_add_kernel(float4* out, const float4* a, const float4* b, long n4) {
   grid_dep_sync();
-  if (epi_skip(st, flag_want)) return;
   const long stride = (long)gridDim.x * blockDim.x;
   for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += stride) {
-    const float4 a = h_img[i], b = h_in[i];
-    R[i] = make_float4(a.x - b.x, a.y - b.y, a.z - b.z, a.w - b.w);
-  }
-}
-
-__global__ void cache_reuse_kernel(const DevState* st, int flag_want, float4* h_img,
-                                   const float4* h_in, const float4* R, long n4) {
-  grid_dep_sync();
-  if (epi_skip(st, flag_want)) return;
-  const long stride = (long)gridDim.x * blockDim.x;
-  for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += stride) {
-    const float4 a = h_in[i], r = R[i];
-    h_img[i] = make_float4(a.x + r.x, a.y + r.y, a.z + r.z, a.w + r.w);
+    const float4 x = a[i], y = b[i];
+    out[i] = make_float4(x.x + y.x, x.y + y.y, x.z + y.z, x.w + y.w);
   }
 }
 
@@ -538,54 +558,45 @@ static int grid_for(long n, int threads) {
   return (int)b;
 }
 
-cudaError_t cache_refresh(const DevState* st, const float* h_img, const float* h_in, float* R, long n,
-                          int flag_want, cudaStream_t s) {
-  if (n % 4 != 0) return cudaErrorInvalidValue;
-  launch_kernel(cache_refresh_kernel, grid_for(n / 4, 256), 256, 0, s, st, flag_want,
-                reinterpret_cast<const float4*>(h_img), reinterpret_cast<const float4*>(h_in),
-                reinterpret_cast<float4*>(R), n / 4);
-  return cudaGetLastError();
-}
-
-cudaError_t cache_reuse(const DevState* st, float* h_img, const float* h_in, const float* R,
-                        long n, int flag_want, cudaStream_t s) {
-  if (n % 4 != 0) return cudaErrorInvalidValue;
-  launch_kernel(cache_reuse_kernel, grid_for(n / 4, 256), 256, 0, s, st, flag_want,
-                reinterpret_cast<float4*>(h_img), reinterpret_cast<const float4*>(h_in),
-                reinterpret_cast<const float4*>(R), n / 4);
-  return cudaGetLastError();
-}
-
 cudaError_t residual_add(float* out, const float* a, const float* b, long n, cudaStream_t s) {
-  return cache_reuse(nullptr, out, a, b, n, -1, s);
+  if (n % 4 != 0) return cudaErrorInvalidValue;
+  launch_kernel(residual_add_kernel, grid_for(n / 4, 256), 256, 0, s, reinterpret_cast<float4*>(out),
+                reinterpret_cast<const float4*>(a), reinterpret_cast<const float4*>(b), n / 4);
+  return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------
 // helpers
 // ---------------------------------------------------------------------------
-__global__ void copy_rows_kernel(const DevState* st, int flag_want, float* dst, long ldd,
-                                 const void* src, long lds, int src_bf16, int rows, int cols) {
+// Row-contiguous copies, so each block of the stream is one run of float4 groups (rows are
+// multiples of 64 elements).  One launch for all blocks: on small backbones a launch is what
+// such a copy costs.
+__global__ void stream_init_kernel(const DevState* st, int flag_want, float4* h, const void* txt0,
+                                   const void* txt1, int txt_bf16, const float4* h_in, int nb, long nx4, long ni4) {
   grid_dep_sync();
   if (epi_skip(st, flag_want)) return;
-  const long n = (long)rows * cols;
-  for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
-    const long r = i / cols, c = i % cols;
-    dst[r * ldd + c] = src_bf16 ? __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(src)[r * lds + c])
-                                : reinterpret_cast<const float*>(src)[r * lds + c];
+  const long n_txt = nb * nx4, n = n_txt + nb * ni4;
+  const long stride = (long)gridDim.x * blockDim.x;
+  for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
+    if (i < n_txt) {
+      float r[4];
+      load4(i < nx4 ? txt0 : txt1, 4 * (i < nx4 ? i : i - nx4), txt_bf16, r);
+      h[i] = make_float4(r[0], r[1], r[2], r[3]);
+    } else {
+      const long k = i - n_txt;
+      h[i] = h_in[k < ni4 ? k : k - ni4];
+    }
   }
 }
 
-cudaError_t copy_rows_f32(const DevState* st, int flag_want, float* dst, long ldd, const void* src,
-                          long lds, int src_bf16, int rows, int cols, cudaStream_t s) {
-  if (rows <= 0) return cudaSuccess;
-  launch_kernel(copy_rows_kernel, grid_for((long)rows * cols, 256), 256, 0, s, st, flag_want, dst, ldd,
-                src, lds, src_bf16, rows, cols);
+cudaError_t stream_init(const DevState* st, int flag_want, float* h, const void* txt0, const void* txt1,
+                        int txt_bf16, const float* h_in, int nb, int nx, int ni, int d, cudaStream_t s) {
+  if (d % 4 != 0) return cudaErrorInvalidValue;
+  const long nx4 = (long)nx * d / 4, ni4 = (long)ni * d / 4;
+  launch_kernel(stream_init_kernel, grid_for(nb * (nx4 + ni4), 256), 256, 0, s, st, flag_want,
+                reinterpret_cast<float4*>(h), txt0, txt1, txt_bf16, reinterpret_cast<const float4*>(h_in), nb, nx4,
+                ni4);
   return cudaGetLastError();
-}
-
-__global__ void advance_kernel(DevState* st) {
-  grid_dep_sync();
-  st->t += 1;
 }
 
 // The bounded-wait failure path on purpose: the barrier expects one arrival that never
@@ -604,11 +615,6 @@ __global__ void wait_timeout_kernel(DevState* st) {
 
 cudaError_t wait_timeout_probe(DevState* st, cudaStream_t s) {
   launch_kernel(wait_timeout_kernel, 1, 32, 0, s, st);
-  return cudaGetLastError();
-}
-
-cudaError_t advance_step(DevState* st, cudaStream_t s) {
-  launch_kernel(advance_kernel, 1, 1, 0, s, st);
   return cudaGetLastError();
 }
 

@@ -13,6 +13,12 @@ namespace bag {
 
 BAG_DEV int epi_step(const Epi& e) { return e.st ? e.st->t : 0; }
 
+// The first kernel of a step advances the step index (no kernel before it in the step
+// reads it, and this kernel does not).
+BAG_DEV void epi_bump(const Epi& e) {
+  if (e.bump && blockIdx.x == 0 && threadIdx.x == 0) e.bump->t += 1;
+}
+
 // Early exit for kernels captured on one side of the full/reuse branch.
 BAG_DEV bool epi_skip(const DevState* st, int flag_want) {
   return st != nullptr && flag_want >= 0 && st->flag != flag_want;
@@ -311,10 +317,6 @@ BAG_DEV void epi_apply(const Epi& e, int t, int row, int col0, float* v, float r
       store_vals<NV>(e.out2, (long)row * e.ldo2 + col0, v, e.out2_bf16);
       break;
     }
-    case EPI_DUAL_F32:
-      store_vals<NV>(e.out, (long)row * e.ldo + col0, v, 0);
-      store_vals<NV>(e.out2, (long)row * e.ldo2 + col0, v, 0);
-      break;
     default:
       break;
   }

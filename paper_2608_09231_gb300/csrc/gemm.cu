@@ -120,6 +120,7 @@ __global__ void __launch_bounds__(SG_WARPS * 32) gemm_simt_kernel(const T* __res
                                                                   int M, int N, int K, const Epi e) {
   grid_dep_sync();
   if (epi_skip(e.st, e.flag_want)) return;
+  epi_bump(e);
   const int t = epi_step(e);
   extern __shared__ __align__(16) float sg[];
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
@@ -369,6 +370,7 @@ __global__ void __launch_bounds__(192, 1)
   // problem fills the SMs the large one leaves idle in its last wave.
   using C = TcCfg<BN>;
   if (epi_skip(e0.st, e0.flag_want)) return;
+  epi_bump(e0);
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~static_cast<uintptr_t>(1023));
@@ -648,6 +650,7 @@ __global__ void __launch_bounds__(192)
   grid_dep_sync();
   // every CTA of a cluster sees the same flag, so they leave together
   if (epi_skip(e0.st, e0.flag_want)) return;
+  epi_bump(e0);
   const int t = epi_step(e0);
   __syncwarp();
   if (warp == 1) {
@@ -836,6 +839,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(192, 1)
   grid_dep_sync();
   // both CTAs of a pair see the same flag, so they leave together
   if (epi_skip(e0.st, e0.flag_want)) return;
+  epi_bump(e0);
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~static_cast<uintptr_t>(1023));

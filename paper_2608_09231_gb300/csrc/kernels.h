@@ -50,7 +50,7 @@ inline cudaError_t launch_kernel(void (*k)(P...), dim3 grid, dim3 block, size_t 
 // Per-sample state the step kernels read and write on the device, so that a whole
 // denoising step can be replayed from a CUDA graph with no host round trip.
 struct DevState {
-  int t;          // current step index (advanced on device at the end of each step)
+  int t;          // current step index (advanced on device by each step's first kernel)
   int c;          // full evaluations spent so far (Algorithm 2's counter)
   int t_last;     // last fully computed step
   int flag;       // decision of the current step: 1 = full, 0 = reuse
@@ -82,7 +82,6 @@ enum EpiKind : int {
   EPI_RES_ADD = 5,    // resid += acc + bias
   EPI_EULER = 6,      // x += dsig[t] * (acc + bias); xb = bf16(x)
   EPI_VEC = 7,        // out = acc + bias + addend; out2 = silu(out) (bf16 or f32)
-  EPI_DUAL_F32 = 8,   // out = out2 = acc + bias (f32)
 };
 
 // UniPC coefficients per step: sigma_i; corrector weights of x_i, the previous corrected
@@ -151,6 +150,7 @@ struct Epi {
   // stack sets one branch's rows, so that a guided sample, whose launches hold both
   // branches' rows, sums in the same order and gives the same bits as an unguided one.
   int plan_rows = 0;
+  DevState* bump = nullptr;      // first kernel of a step: one thread advances bump->t
   // step-dependent addressing and early exit
   const DevState* st = nullptr;  // null: step 0, no flag check
   int flag_want = -1;            // -1: always run; 0/1: run only when st->flag equals it
@@ -225,6 +225,13 @@ struct LnArgs {
   void* sig_ref_w = nullptr;
   // identity: y = x (no normalisation or modulation; the observable is x itself)
   int identity = 0;
+  // residual cache (final layer of a step): on a full step (st->flag) each row x - cache_in
+  // is kept in the cache, on a reused step x is cache_in + the cached row instead of x.
+  // Rows >= split are the second guidance branch: they use cache_in's rows from 0 again and
+  // cache_r2.  cache_in null = off.
+  const float* cache_in = nullptr;
+  float* cache_r = nullptr;
+  float* cache_r2 = nullptr;
   // rows ahead whose x (and signal references) a CTA pulls into L2 for a CTA of a later
   // wave (set by the launcher: resident CTAs of the whole GPU; 0 = none)
   int prefetch_rows = 0;
@@ -236,13 +243,11 @@ cudaError_t gate_step(DevState* st, const float* sig_partial, int sig_rows, cons
                       int gate_kind, float thr, int T, int B, int policy,
                       const uint8_t* policy_mask, float delta, float* log,
                       unsigned long long cond_handle, int use_cond, cudaStream_t s);
-cudaError_t cache_refresh(const DevState* st, const float* h_img, const float* h_in, float* R, long n,
-                          int flag_want, cudaStream_t s);
-cudaError_t cache_reuse(const DevState* st, float* h_img, const float* h_in, const float* R,
-                        long n, int flag_want, cudaStream_t s);
-cudaError_t copy_rows_f32(const DevState* st, int flag_want, float* dst, long ldd, const void* src,
-                          long lds, int src_bf16, int rows, int cols, cudaStream_t s);
-cudaError_t advance_step(DevState* st, cudaStream_t s);
+// The residual stream of a full step, [text of branch 0; text of branch 1; image of branch 0;
+// image of branch 1] with nb branches: text rows converted from txt0 / txt1, every image
+// block a copy of h_in.
+cudaError_t stream_init(const DevState* st, int flag_want, float* h, const void* txt0, const void* txt1,
+                        int txt_bf16, const float* h_in, int nb, int nx, int ni, int d, cudaStream_t s);
 // one thread waits (bounded) on an mbarrier nothing arrives on, then sets st->err
 cudaError_t wait_timeout_probe(DevState* st, cudaStream_t s);
 cudaError_t sinusoid_all(void* out, int out_bf16, const double* sigma, int T, int dim, cudaStream_t s);
