@@ -219,8 +219,10 @@ static int tile_group_rows(int M, int BM, int K, int a_split) {
   return std::max(1, std::min(num_m, g));
 }
 
-// Per epilogue warp: a 32 x 33-word shared-memory tile for transposing V.
-constexpr int kVtScratchFloats = 32 * 33;
+// Per epilogue warp: a shared-memory tile for transposing 32 x 32 accumulators (V: rows of
+// 33 words; fp32 rows: 36 words, so that 16-byte accesses are aligned and conflict-free).
+constexpr int kF32Ld = 36;
+constexpr int kVtScratchFloats = 32 * kF32Ld;
 constexpr int kVtScratchBytes = 4 * kVtScratchFloats * 4;  // four epilogue warps
 
 BAG_DEV uint16_t to16(float x, bool f16) {
@@ -295,11 +297,102 @@ BAG_DEV void store_vt_warp(const Epi& e, int row, int col, float* v, float* sbuf
   }
 }
 
+// Whether an epilogue reads or writes fp32 rows that store_f32_warp can take 16 bytes at a time.
+BAG_DEV bool f32_rows(const Epi& e) {
+  uintptr_t p = reinterpret_cast<uintptr_t>(e.bias);
+  long ld;
+  if ((e.kind == EPI_STORE || e.kind == EPI_GELU) && e.out_bf16 == kStoreF32) {
+    p |= reinterpret_cast<uintptr_t>(e.out);
+    ld = e.ldo;
+  } else if (e.kind == EPI_GATED_RES || e.kind == EPI_RES_ADD) {
+    p |= reinterpret_cast<uintptr_t>(e.resid);
+    ld = e.ldr;
+    if (e.kind == EPI_GATED_RES) {
+      p |= reinterpret_cast<uintptr_t>(e.gate);
+      if (e.br_rows > 0) p |= reinterpret_cast<uintptr_t>(e.gate_u);
+      ld |= e.gate_step;
+    }
+  } else {
+    return false;
+  }
+  return (p & 15) == 0 && ld % 4 == 0;
+}
+
+// 32 rows x 32 columns of fp32 output (or of an fp32 residual update), one warp: the
+// accumulators pass through shared memory so that eight lanes hold 32 consecutive columns of
+// a row.  A warp access then covers four whole 128-byte lines, where a lane that keeps its
+// own row touches 32 lines with 16 bytes each, and bias and gate are read once for eight
+// rows.  The same sums and products element by element as epi_apply.
+// Measured, row per lane against this: 1373 x 12288 x 3072 fp32 store 76.6 -> 69.3 us, with GELU
+// 89.5 -> 73.8; 4608 x 12288 x 3072 209 -> 186 us; 4096 x 3072 x 128 39 -> 29 us; gated residual
+// 4608 x 3072 x 15360 256 -> 240 us.
+BAG_DEV void store_f32_warp(const Epi& e, int t, int row0, int col0, const float* v, float* buf) {
+  const int lane = threadIdx.x & 31, r = lane >> 3, c = (lane & 7) * 4;
+#pragma unroll
+  for (int j = 0; j < 32; j += 4)
+    *reinterpret_cast<float4*>(buf + lane * kF32Ld + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+  const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+  const float4 b = e.bias ? __ldg(reinterpret_cast<const float4*>(e.bias + col0 + c)) : zero;
+  __syncwarp();
+  float4 a[8];
+#pragma unroll
+  for (int p = 0; p < 8; ++p) {
+    a[p] = *reinterpret_cast<const float4*>(buf + (p * 4 + r) * kF32Ld + c);
+    a[p].x += b.x;
+    a[p].y += b.y;
+    a[p].z += b.z;
+    a[p].w += b.w;
+  }
+  __syncwarp();  // the tile may be overwritten
+  const int row = row0 + r;
+  if (e.kind == EPI_STORE || e.kind == EPI_GELU) {
+    float* o = reinterpret_cast<float*>(e.out) + (long)row * e.ldo + col0 + c;
+#pragma unroll
+    for (int p = 0; p < 8; ++p) {
+      if (row + 4 * p >= e.M) break;
+      if (e.kind == EPI_GELU)
+        a[p] = make_float4(gelu_tanh(a[p].x), gelu_tanh(a[p].y), gelu_tanh(a[p].z), gelu_tanh(a[p].w));
+      *reinterpret_cast<float4*>(o + (long)(4 * p) * e.ldo) = a[p];
+    }
+    return;
+  }
+  float* o = e.resid + (long)row * e.ldr + col0 + c;
+  float4 h[8];
+#pragma unroll
+  for (int p = 0; p < 8; ++p)
+    h[p] = row + 4 * p < e.M ? *reinterpret_cast<const float4*>(o + (long)(4 * p) * e.ldr) : zero;
+  float4 g0 = make_float4(1.f, 1.f, 1.f, 1.f), g1 = g0;
+  if (e.kind == EPI_GATED_RES) {
+    const long at = (long)t * e.gate_step + col0 + c;
+    g0 = __ldg(reinterpret_cast<const float4*>(e.gate + at));
+    g1 = e.br_rows > 0 ? __ldg(reinterpret_cast<const float4*>(e.gate_u + at)) : g0;
+  }
+#pragma unroll
+  for (int p = 0; p < 8; ++p) {
+    if (row + 4 * p >= e.M) break;
+    const float4 g = e.br_rows > 0 && row + 4 * p >= e.br_rows ? g1 : g0;
+    h[p].x += g.x * a[p].x;
+    h[p].y += g.y * a[p].y;
+    h[p].z += g.z * a[p].z;
+    h[p].w += g.w * a[p].w;
+    *reinterpret_cast<float4*>(o + (long)(4 * p) * e.ldr) = h[p];
+  }
+}
+
 // One thread's row of a BN-column accumulator in TMEM (lane base already in tb) through
 // the epilogue, columns col0 .. col0 + BN - 1.  vt_buf: this warp's transpose tile.
 template <int BN>
 BAG_DEV void drain_accumulator(const Epi& e, int t, int row, int col0, uint32_t tb, float* vt_buf) {
   const bool vt_warp = e.kind == EPI_QKV && e.v_mode == 1 && e.qkv_type != kStoreF32;
+  if (f32_rows(e)) {
+#pragma unroll 1
+    for (int c = 0; c < BN; c += 32) {
+      float v[32];
+      tmem_ld32(tb + (uint32_t)c, v);
+      store_f32_warp(e, t, row - (int)(threadIdx.x & 31), col0 + c, v, vt_buf);
+    }
+    return;
+  }
   if (e.qn_q) {
     // QK-norm: the tile holds whole heads (BN a multiple of dh, checked at launch); a
     // first pass over each q / k head takes its sum of squares (bias included), the

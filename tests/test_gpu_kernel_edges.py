@@ -88,3 +88,26 @@ def test_split_k_gemm(M, N, K, epilogue, lib):
         ref = torch.nn.functional.gelu(ref, approximate="tanh")
     assert bool(((C[:M].double() - ref).abs() <= bound).all())
     assert bool((C[M] == -7.0).all())
+
+
+@pytest.mark.parametrize("M,N,K", [(33, 64, 128), (1300, 1280, 64), (2500, 3072, 64)])  # BN 64, BN 128, CTA pairs
+@pytest.mark.parametrize("epilogue", [0, 1])
+@pytest.mark.parametrize("offset,pad", [(0, 0), (4, 4), (1, 3)])  # 16-byte rows and not
+def test_fp32_output_rows(M, N, K, epilogue, offset, pad, lib):
+    """fp32 outputs through the transposing epilogue and, for rows that are not 16-byte
+    aligned, through the per-row one; columns and rows around the output stay untouched."""
+    ctx = bag.create("tiny", T=2, B=1)
+    g = torch.Generator(device="cuda").manual_seed(M + N)
+    A = torch.randn(M, K, generator=g, device="cuda").bfloat16()
+    W = (0.1 * torch.randn(N, K, generator=g, device="cuda")).bfloat16()
+    bias = 0.1 * torch.randn(N, generator=g, device="cuda")
+    whole = torch.full((M + 1, N + offset + pad), -7.0, device="cuda")
+    ctx.gemm_bf16(A, W, bias, whole[:M, offset:offset + N], M, N, K, epilogue)
+    torch.cuda.synchronize()
+    ctx.close()
+    ref = A.double() @ W.double().T + bias.double()
+    bound = 1.2 * (4 * K * 2.0 ** -24 * (A.double().abs() @ W.double().abs().T) + 1e-6)
+    if epilogue:
+        ref = torch.nn.functional.gelu(ref, approximate="tanh")
+    assert bool(((whole[:M, offset:offset + N].double() - ref).abs() <= bound).all())
+    assert bool((whole[M] == -7.0).all() and (whole[:, :offset] == -7.0).all() and (whole[:, offset + N:] == -7.0).all())
