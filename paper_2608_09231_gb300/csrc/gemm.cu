@@ -230,71 +230,50 @@ BAG_DEV uint16_t to16(float x, bool f16) {
 }
 BAG_DEV uint32_t pack16x2(float a, float b, bool f16) { return f16 ? pack_f16x2(a, b) : pack_bf16x2(a, b); }
 
-// 32 consecutive 16-bit tokens of one V^T row starting at dst: 16-byte stores when dst is
-// 16-byte aligned, else 4-byte stores (with a single leading element when dst is odd).
-BAG_DEV void store_vt_run(uint16_t* dst, const float* tc, bool f16) {
-  if ((reinterpret_cast<uintptr_t>(dst) & 15) == 0) {
-#pragma unroll
-    for (int k = 0; k < 32; k += 8) {
-      uint4 w;
-      w.x = pack16x2(tc[k], tc[k + 1], f16);
-      w.y = pack16x2(tc[k + 2], tc[k + 3], f16);
-      w.z = pack16x2(tc[k + 4], tc[k + 5], f16);
-      w.w = pack16x2(tc[k + 6], tc[k + 7], f16);
-      *reinterpret_cast<uint4*>(dst + k) = w;
-    }
-  } else if ((reinterpret_cast<uintptr_t>(dst) & 3) == 0) {
-#pragma unroll
-    for (int k = 0; k < 32; k += 2) *reinterpret_cast<uint32_t*>(dst + k) = pack16x2(tc[k], tc[k + 1], f16);
-  } else {
-    dst[0] = to16(tc[0], f16);
-#pragma unroll
-    for (int k = 1; k < 31; k += 2) *reinterpret_cast<uint32_t*>(dst + k) = pack16x2(tc[k], tc[k + 1], f16);
-    dst[31] = to16(tc[31], f16);
-  }
-}
-
 // V columns of a QKV projection with 16-bit (bf16 or fp16) storage, stored transposed per head
-// (vt[(head * dh + e) * vpad + token]): the warp's 32 rows x 32 columns pass through
-// shared memory, so each lane writes one column's 32 consecutive tokens as four 16-byte
-// stores instead of 32 two-byte stores.  Rows past M (the last tile) and token offsets
-// that are not 16-byte aligned take per-element stores.
+// (vt[(head * dh + e) * vpad + token]): the warp's 32 rows x 32 columns.  Whole blocks of one
+// branch whose token offset is 16-byte aligned pass through shared memory (rows of 33 words)
+// so that four lanes hold 32 consecutive tokens of a column and a warp store covers eight
+// columns' 64-byte runs; the others (a ragged text length, the last rows) store from
+// registers, lane = token, 64 bytes of one column at a time.
 BAG_DEV void store_vt_warp(const Epi& e, int row, int col, float* v, float* sbuf) {
   const int lane = threadIdx.x & 31;
-  if (e.bias) {
-#pragma unroll
-    for (int j = 0; j < 32; ++j) v[j] += __ldg(e.bias + col + j);
-  }
-#pragma unroll
-  for (int j = 0; j < 32; ++j) sbuf[j * 33 + lane] = v[j];
-  __syncwarp();
-  float tc[32];
-#pragma unroll
-  for (int k = 0; k < 32; ++k) tc[k] = sbuf[lane * 33 + k];
-  __syncwarp();
   const int row0 = row - lane;
-  // guidance branches (br_rows > 0): the warp's 32 rows take the fast path only when
-  // they all belong to one branch
+  const bool f16 = e.qkv_type == kStoreF16;
+  const int cc = col + e.col_base - 2 * e.d;  // column within V
+  uint16_t* vbase = reinterpret_cast<uint16_t*>(e.v);
   const bool br1 = e.br_rows > 0 && row0 >= e.br_rows;
   const bool one_branch = e.br_rows == 0 || br1 || row0 + 31 < e.br_rows;
-  const int jr0 = row0 - (br1 ? e.br_rows : 0) + e.row_off;
-  const int cc = col + e.col_base - 2 * e.d + lane;  // this lane's column within V
-  const bool f16 = e.qkv_type == kStoreF16;
-  uint16_t* vbase = reinterpret_cast<uint16_t*>(e.v);
+  const long jr0 = row0 - (br1 ? e.br_rows : 0) + e.row_off;
   uint16_t* dst = vbase + (br1 ? e.br_vt : 0) + (long)cc * e.vpad + jr0;
-  if (row0 + 31 < e.M && one_branch) {
-    store_vt_run(dst, tc, f16);
-  } else {
+  if (row0 + 31 < e.M && one_branch && (reinterpret_cast<uintptr_t>(dst) & 15) == 0 && e.vpad % 8 == 0) {
 #pragma unroll
-    for (int k = 0; k < 32; ++k) {
-      const int rk = row0 + k;
-      if (rk < e.M) {
-        const bool b1 = e.br_rows > 0 && rk >= e.br_rows;
-        const long at = (b1 ? e.br_vt : 0) + (long)cc * e.vpad + rk - (b1 ? e.br_rows : 0) + e.row_off;
-        vbase[at] = to16(tc[k], f16);
-      }
+    for (int j = 0; j < 32; ++j) sbuf[lane * 33 + j] = v[j];
+    __syncwarp();
+    const int r = lane >> 2, c = (lane & 3) * 8;  // column r of each group of eight, tokens c .. c + 7
+#pragma unroll
+    for (int p = 0; p < 4; ++p) {
+      const int cl = p * 8 + r;
+      const float b = e.bias ? __ldg(e.bias + col + cl) : 0.f;
+      float x[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) x[k] = sbuf[(c + k) * 33 + cl] + b;
+      uint4 w;
+      w.x = pack16x2(x[0], x[1], f16);
+      w.y = pack16x2(x[2], x[3], f16);
+      w.z = pack16x2(x[4], x[5], f16);
+      w.w = pack16x2(x[6], x[7], f16);
+      *reinterpret_cast<uint4*>(dst + (long)cl * e.vpad + c) = w;
     }
+    __syncwarp();  // the tile may be overwritten
+    return;
   }
+  if (row >= e.M) return;
+  epi_add_bias<32>(e, col, v);
+  const bool b1 = e.br_rows > 0 && row >= e.br_rows;
+  uint16_t* d = vbase + (b1 ? e.br_vt : 0) + (long)cc * e.vpad + row - (b1 ? e.br_rows : 0) + e.row_off;
+#pragma unroll
+  for (int j = 0; j < 32; ++j) d[(long)j * e.vpad] = to16(v[j], f16);
 }
 
 // Whether an epilogue reads or writes fp32 rows that store_f32_warp can take 16 bytes at a time.
@@ -379,6 +358,115 @@ BAG_DEV void store_f32_warp(const Epi& e, int t, int row0, int col0, const float
   }
 }
 
+// Whether store_16_warp takes an epilogue's 16-bit outputs (V goes to store_vt_warp).
+BAG_DEV bool rows16(const Epi& e) {
+  uintptr_t p = reinterpret_cast<uintptr_t>(e.bias);
+  long ld;
+  if (e.kind == EPI_STORE || e.kind == EPI_GELU) {
+    if (e.out_bf16 == kStoreF32) return false;
+    p |= reinterpret_cast<uintptr_t>(e.out);
+    ld = e.ldo;
+  } else if (e.kind == EPI_QKV) {
+    if (e.v_mode != 1 || e.qkv_type == kStoreF32 || !e.act_bf16) return false;
+    p |= reinterpret_cast<uintptr_t>(e.q) | reinterpret_cast<uintptr_t>(e.k) | reinterpret_cast<uintptr_t>(e.mlp) |
+         reinterpret_cast<uintptr_t>(e.rope) | reinterpret_cast<uintptr_t>(e.qn_q) |
+         reinterpret_cast<uintptr_t>(e.qn_k);
+    ld = e.ldqk | e.ldm;
+  } else {
+    return false;
+  }
+  return (p & 15) == 0 && ld % 8 == 0;
+}
+
+// 32 rows x 32 columns of 16-bit output, one warp, through shared memory as in
+// store_f32_warp: four lanes hold 32 consecutive columns of a row, so that a warp access
+// covers eight rows' 64-byte runs (and eight rows' rotation table entries, 128 bytes each).
+// rs: 1 / RMS of this lane's row (QK-norm).  The same operations element by element as
+// epi_apply.  Loads inside each row's branch instead of up front cost one L2 round trip per
+// row (910 x 3584 x 512 with QK-norm 30 -> 37 us).
+// Measured, row per lane against this (with store_vt_warp): 4608 x 21504 x 3072, QKV with
+// rotation and GELU, 365 -> 331 us; 910 x 1536 x 512 unchanged.
+BAG_DEV void store_16_warp(const Epi& e, int row0, int col0, const float* v, float* buf, float rs) {
+  const int lane = threadIdx.x & 31, r = lane >> 2, c = (lane & 3) * 8;
+#pragma unroll
+  for (int j = 0; j < 32; j += 4)
+    *reinterpret_cast<float4*>(buf + lane * kF32Ld + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+  float b[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) b[j] = 0.f;
+  if (e.bias) ld_chunk<8>(e.bias + col0 + c, b);
+  void* base = e.out;
+  long ld = e.ldo;
+  int type = e.out_bf16, cc = col0 + c, region = 3;
+  bool gelu = e.kind == EPI_GELU;
+  if (e.kind == EPI_QKV) {
+    const int lc = col0 + e.col_base;
+    region = min(lc / e.d, 3);
+    cc = lc - region * e.d + c;
+    gelu = region == 3;
+    base = region == 0 ? e.q : (region == 1 ? e.k : e.mlp);
+    ld = region < 2 ? e.ldqk : e.ldm;
+    type = region < 2 ? e.qkv_type : kStoreBF16;
+  }
+  // every row's operands before any row's arithmetic: four rows a lane, one round trip
+  const int row = row0 + r;
+  int orow[4];
+#pragma unroll
+  for (int p = 0; p < 4; ++p) orow[p] = row + 8 * p;
+  float4 q[8];  // rotation: (cos, sin) pairs of columns c .. c + 7
+  const bool rot = region < 2 && e.rope;
+  if (region < 2) {
+#pragma unroll
+    for (int p = 0; p < 4; ++p) {
+      const int at = min(row + 8 * p, e.M - 1);
+      const bool br1 = e.br_rows > 0 && at >= e.br_rows;     // unconditional branch
+      const int jr = at - (br1 ? e.br_rows : 0) + e.row_off;  // joint-sequence row
+      orow[p] = jr + (br1 ? (int)e.br_qk : 0);
+      if (rot) {
+        const float4* cs = reinterpret_cast<const float4*>(e.rope + (long)jr * (e.dh / 2) + cc % e.dh / 2);
+        q[2 * p] = __ldg(cs);
+        q[2 * p + 1] = __ldg(cs + 1);
+      }
+    }
+  }
+  __syncwarp();
+  float a[32];
+#pragma unroll
+  for (int p = 0; p < 4; ++p) ld_chunk<8>(buf + (p * 8 + r) * kF32Ld + c, a + 8 * p);
+  __syncwarp();  // the tile may be overwritten
+#pragma unroll
+  for (int j = 0; j < 32; ++j) a[j] += b[j & 7];
+  if (gelu) {
+#pragma unroll
+    for (int j = 0; j < 32; ++j) a[j] = gelu_tanh_fast(a[j]);
+  } else if (region < 2) {
+    if (e.qn_q) {
+      float w[8];
+      ld_chunk<8>((region == 0 ? e.qn_q : e.qn_k) + cc % e.dh, w);
+#pragma unroll
+      for (int p = 0; p < 4; ++p) {
+        const float rr = __shfl_sync(0xffffffffu, rs, p * 8 + r);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) a[8 * p + j] = a[8 * p + j] * rr * w[j];
+      }
+    }
+    if (rot) {
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        float* y = a + 4 * u;
+        const float x0 = y[0], x1 = y[1], x2 = y[2], x3 = y[3];
+        y[0] = x0 * q[u].x - x1 * q[u].y;
+        y[1] = x0 * q[u].y + x1 * q[u].x;
+        y[2] = x2 * q[u].z - x3 * q[u].w;
+        y[3] = x2 * q[u].w + x3 * q[u].z;
+      }
+    }
+  }
+#pragma unroll
+  for (int p = 0; p < 4; ++p)
+    if (row + 8 * p < e.M) store_vals<8>(base, (long)orow[p] * ld + cc, a + 8 * p, type);
+}
+
 // One thread's row of a BN-column accumulator in TMEM (lane base already in tb) through
 // the epilogue, columns col0 .. col0 + BN - 1.  vt_buf: this warp's transpose tile.
 template <int BN>
@@ -393,6 +481,8 @@ BAG_DEV void drain_accumulator(const Epi& e, int t, int row, int col0, uint32_t 
     }
     return;
   }
+  const bool h16 = rows16(e);
+  const int row0 = row - (int)(threadIdx.x & 31);
   if (e.qn_q) {
     // QK-norm: the tile holds whole heads (BN a multiple of dh, checked at launch); a
     // first pass over each q / k head takes its sum of squares (bias included), the
@@ -423,6 +513,8 @@ BAG_DEV void drain_accumulator(const Epi& e, int t, int row, int col0, uint32_t 
         tmem_ld32(tb + (uint32_t)(h0 + c), v);
         if (vt_warp && col + c < e.N && (col + c + e.col_base) / e.d == 2)
           store_vt_warp(e, row, col + c, v, vt_buf);
+        else if (h16)
+          store_16_warp(e, row0, col + c, v, vt_buf, rs);
         else
           epi_apply<32>(e, t, row, col + c, v, rs);
       }
@@ -435,6 +527,8 @@ BAG_DEV void drain_accumulator(const Epi& e, int t, int row, int col0, uint32_t 
       const int col = col0 + c * 32;
       if (vt_warp && col < e.N && (col + e.col_base) / e.d == 2)
         store_vt_warp(e, row, col, v, vt_buf);  // warp-uniform branch
+      else if (h16)
+        store_16_warp(e, row0, col, v, vt_buf, 1.f);
       else
         epi_apply<32>(e, t, row, col, v);
     }
