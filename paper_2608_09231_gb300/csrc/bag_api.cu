@@ -1785,8 +1785,7 @@ static bag_status bag_rel_l1_impl(bag_ctx* ctx, const void* a, const void* b, in
   if (!a || !b || !scratch || !out) return fail(ctx, BAG_EINVAL, "null pointer");
   if (rows <= 0 || cols <= 0 || (dtype != BAG_F32 && dtype != BAG_BF16))
     return fail(ctx, BAG_EINVAL, "bad rel_l1 shape or dtype");
-  CK(rel_l1_partials(a, b, dtype == BAG_BF16, rows, cols, scratch, ctx->stream));
-  CK(rel_l1_finalize(scratch, rows, out, ctx->stream));
+  CK(rel_l1(a, b, dtype == BAG_BF16, rows, cols, scratch, out, ctx->pdl, ctx->stream));
   return BAG_OK;
 }
 

@@ -257,9 +257,10 @@ cudaError_t to_bf16(__nv_bfloat16* dst, const float* src, long n, cudaStream_t s
 cudaError_t fill_synth(void* dst, long n, uint64_t start, float offset, float c32, int bf16,
                        cudaStream_t s);
 cudaError_t residual_add(float* out, const float* a, const float* b, long n, cudaStream_t s);
-cudaError_t rel_l1_partials(const void* a, const void* b, int a_bf16, long rows, long cols,
-                            float* partial, cudaStream_t s);
-cudaError_t rel_l1_finalize(const float* partial, long rows, float* out, cudaStream_t s);
+// out = {sum|a - b| / sum|b|, sum|a - b|, sum|b|}; scratch receives {sum|a - b|, sum|b|} of
+// each row.  pdl: programmatic launch between its two kernels.
+cudaError_t rel_l1(const void* a, const void* b, int bf16, long rows, long cols, float* scratch, float* out, int pdl,
+                   cudaStream_t s);
 
 // message returned by bag_last_error(NULL) (entry points without a context)
 }  // namespace bag

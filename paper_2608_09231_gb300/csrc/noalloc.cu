@@ -116,8 +116,7 @@ extern "C" bag_status bag_rel_l1_noalloc(const void* a, const void* b, int dtype
   const bag_status s = noalloc_scratch(&scratch);
   if (s != BAG_OK) return s;
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-  cudaError_t e = bag::rel_l1_partials(a, b, dtype == BAG_BF16, rows, cols, scratch, st);
-  if (e == cudaSuccess) e = bag::rel_l1_finalize(scratch, rows, out, st);
+  const cudaError_t e = bag::rel_l1(a, b, dtype == BAG_BF16, rows, cols, scratch, out, 1, st);
   if (e != cudaSuccess) {
     bag::set_global_error(std::string("bag_rel_l1_noalloc: ") + cudaGetErrorString(e));
     return BAG_ECUDA;

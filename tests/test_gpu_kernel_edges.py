@@ -111,3 +111,40 @@ def test_fp32_output_rows(M, N, K, epilogue, offset, pad, lib):
         ref = torch.nn.functional.gelu(ref, approximate="tanh")
     assert bool(((whole[:M, offset:offset + N].double() - ref).abs() <= bound).all())
     assert bool((whole[M] == -7.0).all() and (whole[:, :offset] == -7.0).all() and (whole[:, offset + N:] == -7.0).all())
+
+
+@pytest.mark.parametrize("rows,cols", [
+    (1, 1), (3, 8), (129, 256),   # one cluster: fewer rows than warps, a round and one row
+    (300, 255),                   # one cluster (bf16), rows that are not 16-byte groups
+    (1215, 520), (1217, 1023),    # around a warp per row (eight rows an SM)
+    (64, 40000), (4099, 130)])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("offset", [0, 1])  # inputs and scratch off 16-byte alignment
+def test_rel_l1_routes(rows, cols, dtype, offset, lib):
+    """Every route of the relative L1 (cluster, four warps or one a row; 16-byte groups or
+    elements): sums against fp64 to 2e-6 (fp32 chains of at most a few hundred terms, then a
+    tree), the same bits again and through the allocation-free entry."""
+    ctx = bag.create("tiny", T=2, B=1)
+    g = torch.Generator(device="cuda").manual_seed(rows * 7 + cols)
+
+    def tensor():
+        buf = torch.randn(rows * cols + offset, generator=g, device="cuda").to(dtype)
+        return buf[offset:].reshape(rows, cols)
+
+    a, b = tensor(), tensor()
+    scratch = torch.zeros(2 * rows + 2, device="cuda")
+    out, again, noalloc = (torch.zeros(3, device="cuda") for _ in range(3))
+    ctx.rel_l1(a, b, rows, cols, scratch[offset:], out)
+    ctx.rel_l1(a, b, rows, cols, scratch[offset:], again)
+    torch.cuda.synchronize()
+    bag.rel_l1_noalloc(a, b, rows, cols, noalloc)
+    torch.cuda.synchronize()
+    ctx.close()
+    num, den = (a.double() - b.double()).abs(), b.double().abs()
+    ref = torch.stack([num.sum() / den.sum(), num.sum(), den.sum()])
+    assert bool(((out.double() - ref).abs() <= 2e-6 * ref).all())
+    part = scratch[offset:offset + 2 * rows].reshape(rows, 2).double()
+    assert bool(((part[:, 0] - num.sum(1)).abs() <= 2e-6 * num.sum(1)).all())
+    assert bool(((part[:, 1] - den.sum(1)).abs() <= 2e-6 * den.sum(1)).all())
+    assert float(scratch[offset + 2 * rows]) == 0.0
+    assert torch.equal(out, again) and torch.equal(out, noalloc)
