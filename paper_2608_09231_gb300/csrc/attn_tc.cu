@@ -2,14 +2,24 @@
 //
 // One CTA owns two 128-row query tiles (A and B) of one head and walks the keys in
 // tiles of 128:
-//   warp 0      TMA producer: both Q tiles once, then K and V^T tiles into a 2-stage ring
-//   warp 1      MMA issuer, ping-pong between the tiles:
-//                 S_A,0  S_B,0 | PV_A,j  S_A,j+1 | PV_B,j  S_B,j+1 | ...
-//               so the tensor core computes one tile's products while the other tile's
-//               softmax runs
-//   warps 2..5  softmax of tile A, warps 6..9 softmax of tile B: thread = query row; S
-//               row read from TMEM into registers in one round trip, P = exp2(s - m)
-//               packed to 16 bits and written back into TMEM over the S columns.
+//   warp 0       TMA producer: both Q tiles once, then K and V^T tiles into 2-stage rings of
+//                their own
+//   warp 1       MMA issuer, ping-pong between the tiles:
+//                  S_A,0  S_B,0 | PV_A,j  S_A,j+1 | PV_B,j  S_B,j+1 | ...
+//                so the tensor core computes one tile's products while the other tile's
+//                softmax runs
+//   warps 4..7   softmax of tile A, warps 8..11 softmax of tile B: thread = query row; S
+//                row read from TMEM into registers in one round trip, P = exp2(s - m)
+//                packed to 16 bits and written back into TMEM over the S columns.
+// Bound: tensor core and softmax in turn (a key tile's 32 MMAs are 2,048 cycles).  K is free
+// again after the scores, V only after the PV product: with K and V in one ring stage, the
+// next K was requested when the last PV ended and awaited one product later, less than the
+// latency of 64 KB from L2.  Rings of their own give each load a key tile's time.  The
+// softmax groups hold a whole S row, so they take the issuing warps' registers.
+// Measured, one ring and 200 registers for all against this: 4608 tokens x 24 heads 204 -> 172
+// us (1517 TFLOP/s; rings alone 180), 7145 x 24 487 -> 421, 16,384 x 40 3450 -> 3176.  Slower:
+// an issuing warp for each query tile (212, 521, 3884: both softmaxes then run at the same
+// time and the tensor core idles).  No gain: PV issued in two halves as P arrives.
 // The PV product takes P straight from TMEM as its A operand, so P never touches
 // shared memory; shared memory only feeds Q, K and V^T.  O stays in TMEM for the whole
 // key loop.  The running max only moves (and O is rescaled in TMEM) when a tile's max
@@ -33,13 +43,18 @@ namespace {
 constexpr int AT_M = 128, AT_N = 128, AT_D = 128;
 constexpr int AT_CHUNK = 128 * 64 * 2;  // 128 rows x 64 bf16 = one 128-byte-swizzle column
 constexpr int AT_TILE = 2 * AT_CHUNK;   // 128 x 128 bf16
-constexpr int AT_STAGES = 2;
-constexpr int AT_OFF_Q = 0;                                     // Q_A, Q_B
-constexpr int AT_OFF_KV = 2 * AT_TILE;                          // stage s: K, then V^T
-constexpr int AT_OFF_BAR = AT_OFF_KV + AT_STAGES * 2 * AT_TILE;
+constexpr int AT_STAGES = 2;            // of the K ring and of the V ring
+constexpr int AT_OFF_Q = 0;             // Q_A, Q_B
+constexpr int AT_OFF_K = 2 * AT_TILE;
+constexpr int AT_OFF_V = AT_OFF_K + AT_STAGES * AT_TILE;
+constexpr int AT_OFF_BAR = AT_OFF_V + AT_STAGES * AT_TILE;
 constexpr int AT_SMEM = AT_OFF_BAR + 256 + 1024;
 constexpr int AT_TMEM_COLS = 512;  // S_A [0,128) S_B [128,256) O_A [256,384) O_B [384,512)
-constexpr int AT_THREADS = 320;
+constexpr int AT_THREADS = 384;
+// registers a thread: 168 at launch (65,536 / 384); the issuing warps' group gives up 96 and
+// the two softmax groups take 48 each: 128 * 72 + 256 * 216 = 384 * 168
+constexpr int AT_REGS_ISSUE = 72, AT_REGS_SOFTMAX = 216;
+constexpr int AT_OLD = 36;         // floats a row in the output transpose
 
 struct AttnTcParams {
   int nq, nk;
@@ -131,22 +146,23 @@ template <bool F16>
 __global__ void __launch_bounds__(AT_THREADS, 1)
     attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                    const __grid_constant__ CUtensorMap tmV, const AttnTcParams p) {
-  grid_dep_sync();
-  if (epi_skip(p.st, p.flag_want)) return;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~static_cast<uintptr_t>(1023));
   uint8_t* sQ = smem + AT_OFF_Q;
-  uint8_t* sKV = smem + AT_OFF_KV;
+  uint8_t* sK = smem + AT_OFF_K;
+  uint8_t* sV = smem + AT_OFF_V;
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + AT_OFF_BAR);
   uint64_t* q_full = bars + 0;
-  uint64_t* kv_full = bars + 1;   // [2]
-  uint64_t* kv_empty = bars + 3;  // [2]
-  uint64_t* s_full = bars + 5;    // [2] per query tile
-  uint64_t* p_full = bars + 7;    // [2]
-  uint64_t* o_done = bars + 9;    // [2]
-  uint64_t* drain = bars + 11;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 12);
+  uint64_t* k_full = bars + 1;    // [2]
+  uint64_t* k_empty = bars + 3;   // [2]
+  uint64_t* v_full = bars + 5;    // [2]
+  uint64_t* v_empty = bars + 7;   // [2]
+  uint64_t* s_full = bars + 9;    // [2] per query tile
+  uint64_t* p_full = bars + 11;   // [2]
+  uint64_t* o_done = bars + 13;   // [2]
+  uint64_t* drain = bars + 15;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 16);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
@@ -158,8 +174,10 @@ __global__ void __launch_bounds__(AT_THREADS, 1)
   if (threadIdx.x == 0) {
     mbar_init(q_full, 1);
     for (int i = 0; i < 2; ++i) {
-      mbar_init(kv_full + i, 1);
-      mbar_init(kv_empty + i, 1);
+      mbar_init(k_full + i, 1);
+      mbar_init(k_empty + i, 1);
+      mbar_init(v_full + i, 1);
+      mbar_init(v_empty + i, 1);
       mbar_init(s_full + i, 1);
       mbar_init(p_full + i, 4);  // one arrival per softmax warp of the tile
       mbar_init(o_done + i, 1);
@@ -167,12 +185,13 @@ __global__ void __launch_bounds__(AT_THREADS, 1)
     mbar_init(drain, 1);
     *abort_flag = 0;
     fence_mbar_init();
-  }
-  if (warp == 0 && lane == 0) {
     tma_prefetch_desc(&tmQ);
     tma_prefetch_desc(&tmK);
     tma_prefetch_desc(&tmV);
   }
+  grid_dep_sync();
+  if (epi_skip(p.st, p.flag_want)) return;
+  __syncwarp();
   if (warp == 1) {
     tmem_alloc(tmem_slot, AT_TMEM_COLS);
     tmem_relinquish();
@@ -182,120 +201,114 @@ __global__ void __launch_bounds__(AT_THREADS, 1)
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
 
-  if (warp == 0) {
-    if (lane == 0) {
+  if (warp < 4) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(AT_REGS_ISSUE));
+    if (warp == 0 && lane == 0) {
       // ---------------- TMA producer ----------------
       mbar_arrive_expect_tx(q_full, 2 * AT_TILE);
       for (int x = 0; x < 2; ++x) {
         tma_load_2d(sQ + x * AT_TILE, &tmQ, head * AT_D, qr0 + x * AT_M, q_full);
         tma_load_2d(sQ + x * AT_TILE + AT_CHUNK, &tmQ, head * AT_D + 64, qr0 + x * AT_M, q_full);
       }
-      int issued = 0;
-      bool ok = true;
+      int kj = 0, vj = 0;  // tiles issued
       for (int j = 0; j < nkb; ++j) {
         const int s = j % AT_STAGES;
-        if (!mbar_wait(kv_empty + s, ((j / AT_STAGES) & 1) ^ 1, abort_flag)) {
-          ok = false;
-          break;
-        }
-        uint8_t* k = sKV + s * 2 * AT_TILE;
-        uint8_t* v = k + AT_TILE;
-        mbar_arrive_expect_tx(kv_full + s, 2 * AT_TILE);
-        tma_load_2d(k, &tmK, head * AT_D, kr0 + j * AT_N, kv_full + s);
-        tma_load_2d(k + AT_CHUNK, &tmK, head * AT_D + 64, kr0 + j * AT_N, kv_full + s);
-        tma_load_2d(v, &tmV, j * AT_N, vr0 + head * AT_D, kv_full + s);
-        tma_load_2d(v + AT_CHUNK, &tmV, j * AT_N + 64, vr0 + head * AT_D, kv_full + s);
-        ++issued;
+        const uint32_t ph = ((j / AT_STAGES) & 1) ^ 1;
+        if (!mbar_wait(k_empty + s, ph, abort_flag)) break;
+        uint8_t* k = sK + s * AT_TILE;
+        mbar_arrive_expect_tx(k_full + s, AT_TILE);
+        tma_load_2d(k, &tmK, head * AT_D, kr0 + j * AT_N, k_full + s);
+        tma_load_2d(k + AT_CHUNK, &tmK, head * AT_D + 64, kr0 + j * AT_N, k_full + s);
+        ++kj;
+        if (!mbar_wait(v_empty + s, ph, abort_flag)) break;
+        uint8_t* v = sV + s * AT_TILE;
+        mbar_arrive_expect_tx(v_full + s, AT_TILE);
+        tma_load_2d(v, &tmV, j * AT_N, vr0 + head * AT_D, v_full + s);
+        tma_load_2d(v + AT_CHUNK, &tmV, j * AT_N + 64, vr0 + head * AT_D, v_full + s);
+        ++vj;
       }
-      if (!ok) {
+      if (vj < nkb) {
         // wait (bounded) for copies still in flight before the CTA may exit
         const uint64_t t0 = global_ns();
-        while (!mbar_try_wait(q_full, 0) && global_ns() - t0 < kWaitLimitNs) {
-        }
-        for (int j = (issued > AT_STAGES ? issued - AT_STAGES : 0); j < issued; ++j)
-          while (!mbar_try_wait(kv_full + j % AT_STAGES, (j / AT_STAGES) & 1) &&
-                 global_ns() - t0 < kWaitLimitNs) {
+        auto landed = [&](uint64_t* bar, uint32_t ph) {
+          while (!mbar_try_wait(bar, ph) && global_ns() - t0 < kWaitLimitNs) {
           }
+        };
+        landed(q_full, 0);
+        for (int j = max(0, kj - AT_STAGES); j < kj; ++j) landed(k_full + j % AT_STAGES, (j / AT_STAGES) & 1);
+        for (int j = max(0, vj - AT_STAGES); j < vj; ++j) landed(v_full + j % AT_STAGES, (j / AT_STAGES) & 1);
       }
-    }
-  } else if (warp == 1) {
-    // ---------------- MMA issuer (converged warp, one elected lane issues) ----------------
-    constexpr uint32_t idesc = F16 ? idesc_f16_f32(AT_M, AT_N) : idesc_bf16_f32(AT_M, AT_N);
-    const uint32_t q_addr = smem_u32(sQ), kv_addr = smem_u32(sKV);
-    // K step kk of a tile: 64-column chunk kk / 4, 32 bytes per step inside it (16-byte units)
-    auto koff = [](int kk) { return (uint64_t)(((kk >> 2) * AT_CHUNK + (kk & 3) * 32) >> 4); };
-    auto issue_s = [&](int x, int j) {
-      const uint64_t qd = sw128_desc(q_addr + x * AT_TILE);
-      const uint64_t kd = sw128_desc(kv_addr + (j % AT_STAGES) * 2 * AT_TILE);
-      if (elect_one()) {
+    } else if (warp == 1) {
+      // ---------------- MMA issuer (converged warp, one elected lane issues) ----------------
+      constexpr uint32_t idesc = F16 ? idesc_f16_f32(AT_M, AT_N) : idesc_bf16_f32(AT_M, AT_N);
+      const uint32_t q_addr = smem_u32(sQ), k_addr = smem_u32(sK), v_addr = smem_u32(sV);
+      // K step kk of a tile: 64-column chunk kk / 4, 32 bytes per step inside it (16-byte units)
+      auto koff = [](int kk) { return (uint64_t)(((kk >> 2) * AT_CHUNK + (kk & 3) * 32) >> 4); };
+      // S of query tile x and key tile j; release: the tile's K is no longer needed
+      auto issue_s = [&](int x, int j, bool release) {
+        const uint64_t qd = sw128_desc(q_addr + x * AT_TILE);
+        const uint64_t kd = sw128_desc(k_addr + (j % AT_STAGES) * AT_TILE);
+        if (elect_one()) {
 #pragma unroll
-        for (int kk = 0; kk < AT_D / 16; ++kk)
-          mma_bf16(tmem + x * 128, qd + koff(kk), kd + koff(kk), idesc, kk > 0 ? 1u : 0u);
-        mma_commit(s_full + x);
-      }
-      __syncwarp();
-    };
-    // commit: a barrier to signal once these products are done (null: none)
-    auto issue_pv = [&](int x, int j, uint64_t* commit) {
-      const uint64_t vd = sw128_desc(kv_addr + (j % AT_STAGES) * 2 * AT_TILE + AT_TILE);
-      if (elect_one()) {
-#pragma unroll
-        for (int kk = 0; kk < AT_N / 16; ++kk)
-          mma_bf16_ts(tmem + 256 + x * 128, tmem + x * 128 + kk * 8, vd + koff(kk), idesc,
-                      (j > 0 || kk > 0) ? 1u : 0u);
-        if (commit) mma_commit(commit);
-      }
-      __syncwarp();
-    };
-    bool ok = mbar_wait_warp(q_full, 0, abort_flag) && mbar_wait_warp(kv_full, 0, abort_flag);
-    if (ok) {
-      tc_fence_after();
-      issue_s(0, 0);
-      issue_s(1, 0);
-    }
-    for (int j = 0; j < nkb && ok; ++j) {
-      const bool more = j + 1 < nkb;
-      // tile A: PV_j, then S_{j+1} into the columns P_j came from (in issue order)
-      if (!mbar_wait_warp(p_full + 0, j & 1, abort_flag)) {
-        ok = false;
-        break;
-      }
-      tc_fence_after();
-      issue_pv(0, j, more ? nullptr : o_done + 0);
-      if (more) {
-        if (!mbar_wait_warp(kv_full + (j + 1) % AT_STAGES, ((j + 1) / AT_STAGES) & 1, abort_flag)) {
-          ok = false;
-          break;
+          for (int kk = 0; kk < AT_D / 16; ++kk)
+            mma_bf16(tmem + x * 128, qd + koff(kk), kd + koff(kk), idesc, kk > 0 ? 1u : 0u);
+          mma_commit(s_full + x);
+          if (release) mma_commit(k_empty + j % AT_STAGES);
         }
-        tc_fence_after();
-        issue_s(0, j + 1);
-      }
-      // tile B
-      if (!mbar_wait_warp(p_full + 1, j & 1, abort_flag)) {
-        ok = false;
-        break;
-      }
-      tc_fence_after();
-      issue_pv(1, j, kv_empty + j % AT_STAGES);
-      if (more) {
-        issue_s(1, j + 1);
-      } else {
-        if (elect_one()) mma_commit(o_done + 1);
         __syncwarp();
+      };
+      // commit: a barrier to signal once these products are done (null: none)
+      auto issue_pv = [&](int x, int j, uint64_t* commit) {
+        const uint64_t vd = sw128_desc(v_addr + (j % AT_STAGES) * AT_TILE);
+        if (elect_one()) {
+#pragma unroll
+          for (int kk = 0; kk < AT_N / 16; ++kk)
+            mma_bf16_ts(tmem + 256 + x * 128, tmem + x * 128 + kk * 8, vd + koff(kk), idesc,
+                        (j > 0 || kk > 0) ? 1u : 0u);
+          if (commit) mma_commit(commit);
+        }
+        __syncwarp();
+      };
+      auto wait = [&](uint64_t* bar, uint32_t ph) {
+        const bool w = mbar_wait_warp(bar, ph, abort_flag);
+        tc_fence_after();
+        return w;
+      };
+      bool ok = wait(q_full, 0) && wait(k_full, 0);
+      if (ok) {
+        issue_s(0, 0, false);
+        issue_s(1, 0, true);
       }
-    }
-    if (elect_one()) {
-      mma_commit(drain);
-      const uint64_t t0 = global_ns();
-      while (!mbar_try_wait(drain, 0) && global_ns() - t0 < kWaitLimitNs) {
+      for (int j = 0; j < nkb && ok; ++j) {
+        const int s = j % AT_STAGES, s1 = (j + 1) % AT_STAGES;
+        const bool more = j + 1 < nkb;
+        ok = wait(v_full + s, (j / AT_STAGES) & 1);
+        for (int x = 0; x < 2 && ok; ++x) {
+          // PV_j of this tile, then its S_{j+1} into the columns P_j came from (in issue order)
+          if (!(ok = wait(p_full + x, j & 1))) break;
+          issue_pv(x, j, x ? v_empty + s : (more ? nullptr : o_done + 0));
+          if (more) {
+            if (x == 0 && !(ok = wait(k_full + s1, ((j + 1) / AT_STAGES) & 1))) break;
+            issue_s(x, j + 1, x == 1);
+          } else if (x == 1) {
+            if (elect_one()) mma_commit(o_done + 1);
+            __syncwarp();
+          }
+        }
       }
+      if (elect_one()) {
+        mma_commit(drain);
+        const uint64_t t0 = global_ns();
+        while (!mbar_try_wait(drain, 0) && global_ns() - t0 < kWaitLimitNs) {
+        }
+      }
+      __syncwarp();
     }
-    __syncwarp();
   } else {
-    // ---------------- softmax warpgroups (warps 2..5: tile A, 6..9: tile B) ----------------
-    const int x = (warp - 2) >> 2;
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(AT_REGS_SOFTMAX));
+    // ---------------- softmax warpgroups (warps 4..7: tile A, 8..11: tile B) ----------------
+    const int x = (warp - 4) >> 2;
     const int quad = warp & 3;
-    const int row = quad * 32 + lane;
     const uint32_t lane_base = (uint32_t)(quad * 32) << 16;
     const uint32_t s_addr = tmem + lane_base + x * 128;
     const uint32_t o_addr = tmem + lane_base + 256 + x * 128;
@@ -376,18 +389,31 @@ __global__ void __launch_bounds__(AT_THREADS, 1)
       if (__all_sync(0xffffffffu, w)) {
         tc_fence_after();
         const float inv = 1.f / l;
-        const int q = q0 + x * AT_M + row;
+        // through shared memory (this tile's Q, which no product reads any more): four lanes
+        // hold 32 consecutive columns of a row, so a store covers eight rows' 64-byte runs
+        float* buf = reinterpret_cast<float*>(sQ + x * AT_TILE) + quad * 32 * AT_OLD;
+        const int r = lane >> 2, c8 = (lane & 3) * 8;
+        const int qw = q0 + x * AT_M + quad * 32 + r;
         void* o1 = br ? p.o_b1 : p.o;
         void* o2 = br ? p.o2_b1 : p.o2;
-        void* ob = (o2 && q >= p.o_split) ? o2 : o1;
-        __nv_bfloat16* orow = reinterpret_cast<__nv_bfloat16*>(ob) + (long)q * p.ldo + head * AT_D;
 #pragma unroll 1
-        for (int c = 0; c < AT_D / 32; ++c) {
+        for (int c = 0; c < AT_D; c += 32) {
           float o[32];
-          tmem_ld32(o_addr + c * 32, o);
+          tmem_ld32(o_addr + c, o);
 #pragma unroll
-          for (int i = 0; i < 32; ++i) o[i] *= inv;
-          if (q < p.nq) store_vals<32>(orow + c * 32, 0, o, 1);
+          for (int i = 0; i < 32; i += 4)
+            *reinterpret_cast<float4*>(buf + lane * AT_OLD + i) =
+                make_float4(o[i] * inv, o[i + 1] * inv, o[i + 2] * inv, o[i + 3] * inv);
+          __syncwarp();
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const int q = qw + 8 * u;
+            float v[8];
+            ld_chunk<8>(buf + (8 * u + r) * AT_OLD + c8, v);
+            if (q < p.nq)
+              store_vals<8>(o2 && q >= p.o_split ? o2 : o1, (long)q * p.ldo + head * AT_D + c + c8, v, kStoreBF16);
+          }
+          __syncwarp();
         }
       }
     }
