@@ -715,7 +715,9 @@ static int prof_event(bag_ctx* ctx) {
 // One enqueued segment of kernels on one stream (a step's prefix, a body of the
 // conditional, the suffix, a block, the per-sample preparation).  Every launch after
 // the segment's first is made with programmatic stream serialization unless profiling
-// (whose events sit between the kernels) or the context turned it off.
+// (whose events sit between the kernels) or the context turned it off.  fp32 backbones take
+// plain stream order: their short CUDA-core kernels have no set-up to overlap (toy fp32 sample
+// 1070 us with, 958 without; small guided bf16 sample 1723 with, 1764 without).
 struct Enq {
   bag_ctx* ctx;
   cudaStream_t s;
@@ -745,7 +747,7 @@ struct Enq {
   void chk(cudaError_t r) {
     if (e == cudaSuccess && r != cudaSuccess) e = r;
     if (count) ++*count;
-    g_pdl = ctx->pdl && !ctx->profiling;
+    g_pdl = ctx->pdl && ctx->act_bf16 && !ctx->profiling;
     if (pk >= 0) {
       const int pe1 = prof_event(ctx);
       if (pe1 >= 0) {
