@@ -23,24 +23,9 @@ namespace bag {
 // ---------------------------------------------------------------------------
 // LayerNorm + modulation (+ signal)
 // ---------------------------------------------------------------------------
-constexpr int LN_THREADS = 128;
-constexpr int LN_MAXV = 12;  // float4 per thread: cols <= 128 * 4 * 12 = 6144
-
-BAG_DEV float block_sum(float v, float* red) {
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-  __syncthreads();
-  if (lane == 0) red[warp] = v;
-  __syncthreads();
-  float s = 0.f;
-#pragma unroll
-  for (int w = 0; w < LN_THREADS / 32; ++w) s += red[w];
-  return s;
-}
-
 // Block-wide sum through a shared array that this CTA uses for nothing else: one barrier
 // (no barrier is needed before the writes, since no earlier reduction reads the array).
+template <int TH>
 BAG_DEV float block_sum_fresh(float v, float* red) {
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
@@ -49,13 +34,13 @@ BAG_DEV float block_sum_fresh(float v, float* red) {
   __syncthreads();
   float s = 0.f;
 #pragma unroll
-  for (int w = 0; w < LN_THREADS / 32; ++w) s += red[w];
+  for (int w = 0; w < TH / 32; ++w) s += red[w];
   return s;
 }
 
-// Four block-wide sums at once (one pair of barriers instead of four).
-// fresh: red is used by no earlier reduction of the CTA, so no barrier precedes the writes.
-BAG_DEV float4 block_sum4(float4 v, float4* red, bool fresh_red = false) {
+// Four block-wide sums at once, through an array used for nothing else.
+template <int TH>
+BAG_DEV float4 block_sum4_fresh(float4 v, float4* red) {
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) {
     v.x += __shfl_xor_sync(0xffffffffu, v.x, off);
@@ -64,12 +49,11 @@ BAG_DEV float4 block_sum4(float4 v, float4* red, bool fresh_red = false) {
     v.w += __shfl_xor_sync(0xffffffffu, v.w, off);
   }
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-  if (!fresh_red) __syncthreads();
   if (lane == 0) red[warp] = v;
   __syncthreads();
   float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-  for (int w = 0; w < LN_THREADS / 32; ++w) {
+  for (int w = 0; w < TH / 32; ++w) {
     s.x += red[w].x;
     s.y += red[w].y;
     s.z += red[w].z;
@@ -112,20 +96,27 @@ BAG_DEV void copy4(void* dst, const void* src, long off, int bf16) {
         *(reinterpret_cast<const float4*>(reinterpret_cast<const float*>(src) + off));
 }
 
-// VPT float4 per thread (cols <= 128 * 4 * VPT): the row stays in registers, and the
-// smallest VPT that holds it keeps the register count low enough for many rows per SM
-// (the kernel is latency-bound at low occupancy).
-//
-// CACHE: the final layer's pass also keeps the residual cache (see LnArgs).  As passes of
+// One CTA of TH threads per row, VPT float4 per thread (cols <= TH * 4 * VPT): the row stays
+// in registers, and the register limit (MINB CTAs per SM) keeps many rows in flight; the
+// kernel is bound by the latency of its phases (load, two reductions, store), not by a pipe.
+// LN_SIGNAL: with the trajectory signal.
+// LN_CACHE: the final layer's pass also keeps the residual cache (see LnArgs).  As passes of
 // their own, the cache update or the reuse (12 bytes an element each) and this pass took
 // 26 + 20 us on 4096 x 3072 (profiled launches), together they take 29 us; and the patch
 // embedding, which no longer writes the stream's copy on every step, 60 -> 39 us.
-template <int VPT, bool CACHE>
-__global__ void __launch_bounds__(LN_THREADS, VPT <= 6 ? 8 : (VPT <= 10 ? 5 : 4)) ln_mod_kernel(const LnArgs a) {
+// Threads, measured: 128 with six float4 each are best for plain rows up to 3072 columns
+// (4608 x 3072 from L2 16.2 -> 14.5 us with 48 registers instead of the signal's 64; 256 threads
+// 18.4); the passes with more operands per column and wider rows want more threads with fewer
+// columns (128 -> 256 threads: signal of 4096 x 3072 34.9 -> 30.6 us and final layer 29 -> 27 us
+// as profiled launches, 32,760 x 5120 188 -> 149 us, 6.75 TB/s).
+enum { LN_PLAIN = 0, LN_SIGNAL = 1, LN_CACHE = 2 };
+constexpr int LN_MAX_COLS = 6144;
+template <int TH, int VPT, int MINB, int MODE>
+__global__ void __launch_bounds__(TH, MINB) ln_mod_kernel(const LnArgs a) {
   grid_dep_sync();
   if (epi_skip(a.st, a.flag_want)) return;
   // one shared array per reduction of the row, so that each takes a single barrier
-  __shared__ float red_mean[LN_THREADS / 32], red_var[LN_THREADS / 32];
+  __shared__ float red_mean[TH / 32], red_var[TH / 32];
   const int row = blockIdx.x;
   if (row >= a.rows) return;
   if (threadIdx.x == 0 && a.prefetch_rows > 0 && row + a.prefetch_rows < a.rows) {
@@ -133,7 +124,7 @@ __global__ void __launch_bounds__(LN_THREADS, VPT <= 6 ? 8 : (VPT <= 10 ? 5 : 4)
     // its loads find the row in L2 (row strides are multiples of 16 bytes)
     const long pr = (long)row + a.prefetch_rows;
     l2_prefetch(a.x + pr * a.ldx, (uint32_t)a.cols * 4u);
-    if (a.sig_on) {
+    if constexpr (MODE == LN_SIGNAL) {
       const uint32_t rb = (uint32_t)a.cols * (a.y_bf16 ? 2u : 4u);
       const long off = pr * a.ldy * (a.y_bf16 ? 2 : 4);
       l2_prefetch(reinterpret_cast<const char*>(a.sig_ref2) + off, rb);
@@ -145,7 +136,7 @@ __global__ void __launch_bounds__(LN_THREADS, VPT <= 6 ? 8 : (VPT <= 10 ? 5 : 4)
   const int nv = a.cols / 4;
   float4 v[VPT];
   float s = 0.f;
-  if constexpr (CACHE) {
+  if constexpr (MODE == LN_CACHE) {
     const bool second = row >= a.split;
     const long crow = (long)(second ? row - a.split : row) * a.ldx;
     const float4* hin = reinterpret_cast<const float4*>(a.cache_in + crow);
@@ -155,7 +146,7 @@ __global__ void __launch_bounds__(LN_THREADS, VPT <= 6 ? 8 : (VPT <= 10 ? 5 : 4)
     float4 h[VPT];
 #pragma unroll
     for (int i = 0; i < VPT; ++i) {
-      const int c = threadIdx.x + i * LN_THREADS;
+      const int c = threadIdx.x + i * TH;
       if (c < nv) {
         v[i] = src[c];
         h[i] = hin[c];
@@ -163,7 +154,7 @@ __global__ void __launch_bounds__(LN_THREADS, VPT <= 6 ? 8 : (VPT <= 10 ? 5 : 4)
     }
 #pragma unroll
     for (int i = 0; i < VPT; ++i) {
-      const int c = threadIdx.x + i * LN_THREADS;
+      const int c = threadIdx.x + i * TH;
       if (c < nv) {
         if (full)
           R[c] = make_float4(v[i].x - h[i].x, v[i].y - h[i].y, v[i].z - h[i].z, v[i].w - h[i].w);
@@ -174,28 +165,28 @@ __global__ void __launch_bounds__(LN_THREADS, VPT <= 6 ? 8 : (VPT <= 10 ? 5 : 4)
   }
 #pragma unroll
   for (int i = 0; i < VPT; ++i) {
-    const int c = threadIdx.x + i * LN_THREADS;
+    const int c = threadIdx.x + i * TH;
     if (c < nv) {
-      if constexpr (!CACHE) v[i] = reinterpret_cast<const float4*>(x)[c];
+      if constexpr (MODE != LN_CACHE) v[i] = reinterpret_cast<const float4*>(x)[c];
       s += (v[i].x + v[i].y) + (v[i].z + v[i].w);
     }
   }
   float mean = 0.f, rstd = 1.f;  // identity: y = x
   if (!a.identity) {
-    mean = block_sum_fresh(s, red_mean) / (float)a.cols;
+    mean = block_sum_fresh<TH>(s, red_mean) / (float)a.cols;
     float q = 0.f;
 #pragma unroll
     for (int i = 0; i < VPT; ++i) {
-      const int c = threadIdx.x + i * LN_THREADS;
+      const int c = threadIdx.x + i * TH;
       if (c < nv) {
         const float dx = v[i].x - mean, dy = v[i].y - mean, dz = v[i].z - mean, dw = v[i].w - mean;
         q += (dx * dx + dy * dy) + (dz * dz + dw * dw);
       }
     }
-    rstd = rsqrtf(block_sum_fresh(q, red_var) / (float)a.cols + 1e-6f);
+    rstd = rsqrtf(block_sum_fresh<TH>(q, red_var) / (float)a.cols + 1e-6f);
   }
   // the previous step was fully computed: its observable (ref2) is the new reference
-  const bool refresh = a.sig_on && a.sig_ref_w && a.st && a.st->t > 0 && a.st->t_last == a.st->t - 1;
+  [[maybe_unused]] const bool refresh = MODE == LN_SIGNAL && a.sig_ref_w && a.st && a.st->t > 0 && a.st->t_last == a.st->t - 1;
   const float* sh;
   const float* sc;
   if (row < a.split) {
@@ -213,10 +204,10 @@ __global__ void __launch_bounds__(LN_THREADS, VPT <= 6 ? 8 : (VPT <= 10 ? 5 : 4)
   }
   if (sh) sh += (long)t * a.mod_step;
   if (sc) sc += (long)t * a.mod_step;
-  float sig_num = 0.f, sig_den = 0.f, sig_num2 = 0.f, sig_den2 = 0.f;
+  [[maybe_unused]] float sig_num = 0.f, sig_den = 0.f, sig_num2 = 0.f, sig_den2 = 0.f;
 #pragma unroll
   for (int i = 0; i < VPT; ++i) {
-    const int c = threadIdx.x + i * LN_THREADS;
+    const int c = threadIdx.x + i * TH;
     if (c < nv) {
       float y[4] = {(v[i].x - mean) * rstd, (v[i].y - mean) * rstd, (v[i].z - mean) * rstd,
                     (v[i].w - mean) * rstd};
@@ -235,7 +226,7 @@ __global__ void __launch_bounds__(LN_THREADS, VPT <= 6 ? 8 : (VPT <= 10 ? 5 : 4)
         y[3] += h4.w;
       }
       const long off = (long)row * a.ldy + 4 * c;
-      if (a.sig_on) {
+      if constexpr (MODE == LN_SIGNAL) {
         // both references are read before y is stored: sig_ref2 may be the y buffer
         // itself (the previous step's observable, replaced by this step's)
         float r[4], r2[4], yy[4];
@@ -267,9 +258,9 @@ __global__ void __launch_bounds__(LN_THREADS, VPT <= 6 ? 8 : (VPT <= 10 ? 5 : 4)
       }
     }
   }
-  if (a.sig_on) {
-    __shared__ float4 red4[LN_THREADS / 32];
-    const float4 t4 = block_sum4(make_float4(sig_num, sig_den, sig_num2, sig_den2), red4, true);
+  if constexpr (MODE == LN_SIGNAL) {
+    __shared__ float4 red4[TH / 32];
+    const float4 t4 = block_sum4_fresh<TH>(make_float4(sig_num, sig_den, sig_num2, sig_den2), red4);
     if (threadIdx.x == 0) reinterpret_cast<float4*>(a.sig_partial)[row] = t4;
   }
 }
@@ -285,29 +276,33 @@ static int sm_count() {
   return n;
 }
 
-cudaError_t ln_mod(const LnArgs& args, cudaStream_t s) {
-  if (args.rows <= 0) return cudaSuccess;
-  if (args.cols % 4 != 0 || args.cols > LN_THREADS * 4 * LN_MAXV) return cudaErrorInvalidValue;
-  LnArgs a = args;
-  // The signal pass reads two reference tensors last touched a step earlier (in HBM):
-  // each CTA prefetches into L2 the rows a CTA one wave later will read (distance = the
-  // CTAs resident on the GPU; bulk copies need 16-byte aligned rows).  The stack's
-  // LN-mods read rows the producing GEMM has just written (mostly still in L2): measured
-  // slower with the prefetch, so they take none.
+// Launch of one row per CTA.  The signal pass reads two reference tensors last touched a step
+// earlier (in HBM): each CTA prefetches into L2 the rows a CTA one wave later will read
+// (distance = the CTAs resident on the GPU; bulk copies need 16-byte aligned rows).  The
+// stack's LN-mods read rows the producing GEMM has just written (mostly still in L2):
+// measured slower with the prefetch, so they take none.
+template <int TH, int VPT, int MINB, int MODE>
+static cudaError_t launch_ln(LnArgs a, cudaStream_t s) {
   const bool aligned = ((a.ldx * 4) % 16 == 0) && ((a.cols * 4) % 16 == 0) &&
                        (a.ldy * (a.y_bf16 ? 2 : 4)) % 16 == 0;
-  const int per_sm = a.cols <= LN_THREADS * 4 * 6 ? 8 : (a.cols <= LN_THREADS * 4 * 10 ? 5 : 4);
-  a.prefetch_rows = (a.sig_on && aligned) ? sm_count() * per_sm : 0;
-  auto launch = [&](auto plain, auto cache) {
-    launch_kernel(a.cache_in ? cache : plain, a.rows, LN_THREADS, 0, s, a);
+  a.prefetch_rows = (MODE == LN_SIGNAL && aligned) ? sm_count() * MINB : 0;
+  return launch_kernel(ln_mod_kernel<TH, VPT, MINB, MODE>, a.rows, TH, 0, s, a);
+}
+
+cudaError_t ln_mod(const LnArgs& a, cudaStream_t s) {
+  if (a.rows <= 0) return cudaSuccess;
+  if (a.cols % 4 != 0 || a.cols > LN_MAX_COLS) return cudaErrorInvalidValue;
+  auto launch = [&](auto mode) {
+    constexpr int M = decltype(mode)::value;
+    if (a.cols > 5120) return launch_ln<256, 6, 4, M>(a, s);
+    if (a.cols > 3072) return launch_ln<256, 5, 5, M>(a, s);
+    if constexpr (M == LN_PLAIN) return launch_ln<128, 6, 10, M>(a, s);
+    return launch_ln<256, 3, M == LN_SIGNAL ? 7 : 6, M>(a, s);
   };
-  if (a.cols <= LN_THREADS * 4 * 6)
-    launch(ln_mod_kernel<6, false>, ln_mod_kernel<6, true>);
-  else if (a.cols <= LN_THREADS * 4 * 10)
-    launch(ln_mod_kernel<10, false>, ln_mod_kernel<10, true>);
-  else
-    launch(ln_mod_kernel<LN_MAXV, false>, ln_mod_kernel<LN_MAXV, true>);
-  return cudaGetLastError();
+  const cudaError_t r = a.sig_on ? launch(std::integral_constant<int, LN_SIGNAL>{})
+                                 : (a.cache_in ? launch(std::integral_constant<int, LN_CACHE>{})
+                                               : launch(std::integral_constant<int, LN_PLAIN>{}));
+  return r == cudaSuccess ? cudaGetLastError() : r;
 }
 
 // ---------------------------------------------------------------------------
