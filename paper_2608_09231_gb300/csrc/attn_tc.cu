@@ -55,6 +55,11 @@ constexpr int AT_THREADS = 384;
 // the two softmax groups take 48 each: 128 * 72 + 256 * 216 = 384 * 168
 constexpr int AT_REGS_ISSUE = 72, AT_REGS_SOFTMAX = 216;
 constexpr int AT_OLD = 36;         // floats a row in the output transpose
+// exchange of partial outputs (C > 1), over the Q, K and V tiles: 2 * AT_M rows of AT_D
+// floats (4 more a row against bank conflicts), then (maximum, sum) of each
+constexpr int AT_XLD = AT_D + 4;
+constexpr int AT_OFF_ML = 2 * AT_M * AT_XLD * 4;
+static_assert(AT_OFF_ML + 2 * AT_M * 8 <= AT_OFF_BAR, "the exchange fits the operand tiles");
 
 struct AttnTcParams {
   int nq, nk;
@@ -67,6 +72,8 @@ struct AttnTcParams {
   void* o_b1;
   void* o2_b1;
   float scale_log2;
+  int pairs;    // query tile pairs of a head
+  int whole;    // C > 1: units (pair, head) with a CTA of their own; the others take a cluster
   const DevState* st;
   int flag_want;
   int* err;
@@ -142,7 +149,12 @@ BAG_DEV void mma_bf16_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint3
 }
 }  // namespace
 
-template <bool F16>
+// C > 1: clusters of C CTAs.  The first p.whole units (query tile pair, head) have a CTA each,
+// as with C = 1; every later unit is shared by a cluster, each CTA walking its part of the
+// key tiles.  Rank r then collects 2 * AT_M / C rows of every CTA's unnormalised output,
+// maximum and sum through distributed shared memory and merges them in rank order.  Used
+// where whole units would leave a wave mostly idle (attention_split).
+template <bool F16, int C>
 __global__ void __launch_bounds__(AT_THREADS, 1)
     attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                    const __grid_constant__ CUtensorMap tmV, const AttnTcParams p) {
@@ -166,10 +178,20 @@ __global__ void __launch_bounds__(AT_THREADS, 1)
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-  const int head = blockIdx.y, q0 = blockIdx.x * 2 * AT_M;
+  const int rank = C > 1 ? (int)cluster_ctarank() : 0;
+  const bool split = C > 1 && (int)blockIdx.x >= p.whole;  // uniform over a cluster
+  int head = blockIdx.y, pair = blockIdx.x;
+  if constexpr (C > 1) {  // units along x
+    const int unit = split ? p.whole + ((int)blockIdx.x - p.whole) / C : (int)blockIdx.x;
+    head = unit / p.pairs;
+    pair = unit % p.pairs;
+  }
+  const int q0 = pair * 2 * AT_M;
   const int br = blockIdx.z;  // guidance branch (0 unless two branches share the launch)
   const int qr0 = q0 + br * p.br_q_rows, kr0 = br * p.br_k_rows, vr0 = br * p.br_v_rows;
-  const int nkb = (p.nk + AT_N - 1) / AT_N;
+  const int nkt = (p.nk + AT_N - 1) / AT_N;
+  const int j0 = split ? rank * nkt / C : 0;                     // this CTA's first key tile
+  const int nkb = (split ? (rank + 1) * nkt / C : nkt) - j0;      // and how many (>= 1)
 
   if (threadIdx.x == 0) {
     mbar_init(q_full, 1);
@@ -217,14 +239,14 @@ __global__ void __launch_bounds__(AT_THREADS, 1)
         if (!mbar_wait(k_empty + s, ph, abort_flag)) break;
         uint8_t* k = sK + s * AT_TILE;
         mbar_arrive_expect_tx(k_full + s, AT_TILE);
-        tma_load_2d(k, &tmK, head * AT_D, kr0 + j * AT_N, k_full + s);
-        tma_load_2d(k + AT_CHUNK, &tmK, head * AT_D + 64, kr0 + j * AT_N, k_full + s);
+        tma_load_2d(k, &tmK, head * AT_D, kr0 + (j0 + j) * AT_N, k_full + s);
+        tma_load_2d(k + AT_CHUNK, &tmK, head * AT_D + 64, kr0 + (j0 + j) * AT_N, k_full + s);
         ++kj;
         if (!mbar_wait(v_empty + s, ph, abort_flag)) break;
         uint8_t* v = sV + s * AT_TILE;
         mbar_arrive_expect_tx(v_full + s, AT_TILE);
-        tma_load_2d(v, &tmV, j * AT_N, vr0 + head * AT_D, v_full + s);
-        tma_load_2d(v + AT_CHUNK, &tmV, j * AT_N + 64, vr0 + head * AT_D, v_full + s);
+        tma_load_2d(v, &tmV, (j0 + j) * AT_N, vr0 + head * AT_D, v_full + s);
+        tma_load_2d(v + AT_CHUNK, &tmV, (j0 + j) * AT_N + 64, vr0 + head * AT_D, v_full + s);
         ++vj;
       }
       if (vj < nkb) {
@@ -302,7 +324,11 @@ __global__ void __launch_bounds__(AT_THREADS, 1)
         while (!mbar_try_wait(drain, 0) && global_ns() - t0 < kWaitLimitNs) {
         }
       }
-      __syncwarp();
+    }
+    __syncwarp();
+    if (split) {  // the two barriers of the exchange
+      cluster_sync_all();
+      cluster_sync_all();
     }
   } else {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(AT_REGS_SOFTMAX));
@@ -321,7 +347,7 @@ __global__ void __launch_bounds__(AT_THREADS, 1)
         break;
       }
       tc_fence_after();
-      const int kvalid = p.nk - j * AT_N;  // keys of this tile that exist (< 128 only at the end)
+      const int kvalid = p.nk - (j0 + j) * AT_N;  // keys of this tile that exist (< 128 only at the end)
       // the whole S row in registers: four loads, one wait
       uint32_t r[AT_N];
 #pragma unroll
@@ -349,6 +375,8 @@ __global__ void __launch_bounds__(AT_THREADS, 1)
         m_use = mx2;
         l *= alpha;
       }
+      // a tile of nothing but -inf scores before any other weighs nothing
+      const float neg_m = m_use == -INFINITY ? 0.f : -m_use;
       // P = exp2(s * scale - m) (masked keys give exp2(-inf) = 0), packed 16-bit pairs
       // written over the S columns already read
       float ls0 = 0.f, ls1 = 0.f;
@@ -359,7 +387,7 @@ __global__ void __launch_bounds__(AT_THREADS, 1)
         for (int i = 0; i < 32; i += 2) {
           float x0, x1;
           fma2(x0, x1, __uint_as_float(r[c * 32 + i]), __uint_as_float(r[c * 32 + i + 1]),
-               p.scale_log2, -m_use);
+               p.scale_log2, neg_m);
           const float a0 = ex2(x0), a1 = ex2(x1);
           add2(ls0, ls1, a0, a1);
           pk[i / 2] = F16 ? pack_f16x2(a0, a1) : pack_bf16x2(a0, a1);
@@ -384,37 +412,89 @@ __global__ void __launch_bounds__(AT_THREADS, 1)
       __syncwarp();
       if (lane == 0) mbar_arrive(p_full + x);
     }
-    if (ok) {
-      const bool w = mbar_wait(o_done + x, 0, abort_flag);
-      if (__all_sync(0xffffffffu, w)) {
-        tc_fence_after();
-        const float inv = 1.f / l;
-        // through shared memory (this tile's Q, which no product reads any more): four lanes
-        // hold 32 consecutive columns of a row, so a store covers eight rows' 64-byte runs
-        float* buf = reinterpret_cast<float*>(sQ + x * AT_TILE) + quad * 32 * AT_OLD;
-        const int r = lane >> 2, c8 = (lane & 3) * 8;
-        const int qw = q0 + x * AT_M + quad * 32 + r;
-        void* o1 = br ? p.o_b1 : p.o;
-        void* o2 = br ? p.o2_b1 : p.o2;
+    if (ok) ok = __all_sync(0xffffffffu, mbar_wait(o_done + x, 0, abort_flag));
+    tc_fence_after();
+    if (split) {
+      constexpr int RPO = 2 * AT_M / C;  // rows a rank merges
+      __syncwarp();
+      cluster_sync_all();  // every CTA's products are done: the operand tiles are free
+      if (ok) {
+        const int R = x * AT_M + quad * 32 + lane;
+        const int at = rank * RPO + R % RPO;
+        const uint32_t dst = mapa_shared(smem_u32(smem), (uint32_t)(R / RPO));
 #pragma unroll 1
         for (int c = 0; c < AT_D; c += 32) {
           float o[32];
           tmem_ld32(o_addr + c, o);
 #pragma unroll
           for (int i = 0; i < 32; i += 4)
-            *reinterpret_cast<float4*>(buf + lane * AT_OLD + i) =
-                make_float4(o[i] * inv, o[i + 1] * inv, o[i + 2] * inv, o[i + 3] * inv);
-          __syncwarp();
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const int q = qw + 8 * u;
-            float v[8];
-            ld_chunk<8>(buf + (8 * u + r) * AT_OLD + c8, v);
-            if (q < p.nq)
-              store_vals<8>(o2 && q >= p.o_split ? o2 : o1, (long)q * p.ldo + head * AT_D + c + c8, v, kStoreBF16);
-          }
-          __syncwarp();
+            st_cluster4(dst + (uint32_t)(at * AT_XLD + c + i) * 4, o[i], o[i + 1], o[i + 2], o[i + 3]);
         }
+        st_cluster2(dst + AT_OFF_ML + (uint32_t)at * 8, m_use, l);
+      }
+      __syncwarp();
+      cluster_sync_all();  // every part has arrived; no access to another CTA follows
+      const float* part = reinterpret_cast<const float*>(smem);
+      const float2* ml = reinterpret_cast<const float2*>(smem + AT_OFF_ML);
+      void* o1 = br ? p.o_b1 : p.o;
+      void* o2 = br ? p.o2_b1 : p.o2;
+#pragma unroll 2
+      for (int lr = warp - 4; lr < RPO; lr += 8) {  // a warp a row, four columns a lane
+        float2 f[C];
+        float m = -INFINITY, den = 0.f;
+#pragma unroll
+        for (int s = 0; s < C; ++s) {
+          f[s] = ml[s * RPO + lr];
+          m = fmaxf(m, f[s].x);
+        }
+        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int s = 0; s < C; ++s) {
+          const float w = f[s].x == -INFINITY ? 0.f : ex2(f[s].x - m);
+          const float4 o = *reinterpret_cast<const float4*>(part + (s * RPO + lr) * AT_XLD + lane * 4);
+          den += w * f[s].y;
+          acc.x += w * o.x;
+          acc.y += w * o.y;
+          acc.z += w * o.z;
+          acc.w += w * o.w;
+        }
+        const float inv = 1.f / den;
+        const int q = q0 + rank * RPO + lr;
+        if (q < p.nq) {
+          uint2 u;
+          u.x = pack_bf16x2(acc.x * inv, acc.y * inv);
+          u.y = pack_bf16x2(acc.z * inv, acc.w * inv);
+          *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(o2 && q >= p.o_split ? o2 : o1) +
+                                    (long)q * p.ldo + head * AT_D + lane * 4) = u;
+        }
+      }
+    } else if (ok) {
+      const float inv = 1.f / l;
+      // through shared memory (this tile's Q, which no product reads any more): four lanes
+      // hold 32 consecutive columns of a row, so a store covers eight rows' 64-byte runs
+      float* buf = reinterpret_cast<float*>(sQ + x * AT_TILE) + quad * 32 * AT_OLD;
+      const int r = lane >> 2, c8 = (lane & 3) * 8;
+      const int qw = q0 + x * AT_M + quad * 32 + r;
+      void* o1 = br ? p.o_b1 : p.o;
+      void* o2 = br ? p.o2_b1 : p.o2;
+#pragma unroll 1
+      for (int c = 0; c < AT_D; c += 32) {
+        float o[32];
+        tmem_ld32(o_addr + c, o);
+#pragma unroll
+        for (int i = 0; i < 32; i += 4)
+          *reinterpret_cast<float4*>(buf + lane * AT_OLD + i) =
+              make_float4(o[i] * inv, o[i + 1] * inv, o[i + 2] * inv, o[i + 3] * inv);
+        __syncwarp();
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int q = qw + 8 * u;
+          float v[8];
+          ld_chunk<8>(buf + (8 * u + r) * AT_OLD + c8, v);
+          if (q < p.nq)
+            store_vals<8>(o2 && q >= p.o_split ? o2 : o1, (long)q * p.ldo + head * AT_D + c + c8, v, kStoreBF16);
+        }
+        __syncwarp();
       }
     }
   }
@@ -426,12 +506,42 @@ __global__ void __launch_bounds__(AT_THREADS, 1)
   }
 }
 
+static int g_sms = 1;
+
 cudaError_t attention_tc_init() {
-  cudaError_t r = cudaFuncSetAttribute(attn_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       AT_SMEM);
-  if (r == cudaSuccess)
-    r = cudaFuncSetAttribute(attn_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, AT_SMEM);
+  const void* kernels[] = {(const void*)attn_tc_kernel<false, 1>, (const void*)attn_tc_kernel<false, 2>,
+                           (const void*)attn_tc_kernel<false, 4>, (const void*)attn_tc_kernel<true, 1>,
+                           (const void*)attn_tc_kernel<true, 2>,  (const void*)attn_tc_kernel<true, 4>};
+  cudaError_t r = cudaSuccess;
+  for (const void* k : kernels)
+    if (r == cudaSuccess) r = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, AT_SMEM);
+  int dev = 0;
+  if (r == cudaSuccess) r = cudaGetDevice(&dev);
+  if (r == cudaSuccess) r = cudaDeviceGetAttribute(&g_sms, cudaDevAttrMultiProcessorCount, dev);
   return r;
+}
+
+// CTAs per cluster and the units that keep a CTA of their own, for `units` (query tile pair,
+// head) of one guidance branch and `nkt` key tiles: a launch of fewer units than SMs shares
+// each unit among 2 or 4 CTAs; a longer one shares the units of its last wave where they
+// leave at least half of the SMs idle.  A key tile takes about 1.45 us and sharing about 7 us
+// (cluster launch, two barriers, the exchange), hence the least numbers of key tiles.  Planned
+// from one branch's units, so that guided and unguided samples give the same bits.
+// Measured: 7145 tokens x 24 heads (672 units on 152 SMs, the last 64 shared) 432 -> 399 us;
+// 1536 x 4 heads 25.6 -> 19.9 us, 3000 x 2 42.9 -> 25.2, 5000 x 8 122 -> 101; with 4 key tiles
+// (455 x 4), shared by four, 13.9 -> 16.9 us.
+static int attention_split(int units, int nkt, int* whole) {
+  *whole = units;
+  if (units < g_sms) {
+    // clusters of four reach 144 of 152 SMs
+    const int c = units * 4 <= g_sms - g_sms / 16 && nkt >= 12 ? 4 : (units * 2 <= g_sms && nkt >= 16 ? 2 : 1);
+    if (c > 1) *whole = 0;
+    return c;
+  }
+  const int rest = units % g_sms;
+  if (rest == 0 || rest * 2 > g_sms || nkt < 16 || (units - rest) % 2) return 1;
+  *whole = units - rest;
+  return 2;
 }
 
 int attention_tc_supported(const AttnArgs& a) {
@@ -471,11 +581,19 @@ cudaError_t attention_tc(const AttnArgs& a, int* err, cudaStream_t s) {
   p.st = a.st;
   p.flag_want = a.flag_want;
   p.err = err;
-  dim3 grid((a.nq + 2 * AT_M - 1) / (2 * AT_M), a.heads, nbr);
+  p.pairs = (a.nq + 2 * AT_M - 1) / (2 * AT_M);
+  const int units = p.pairs * a.heads;
+  const int c = attention_split(units, (a.nk + AT_N - 1) / AT_N, &p.whole);
+  const dim3 grid = c > 1 ? dim3((unsigned)(p.whole + (units - p.whole) * c), 1, nbr) : dim3(p.pairs, a.heads, nbr);
+  auto launch = [&](auto kernel) {
+    launch_cluster(kernel, c > 1 ? (unsigned)c : 0u, grid, AT_THREADS, AT_SMEM, s, tq, tk, tv, p);
+  };
   if (a.f16)
-    launch_kernel(attn_tc_kernel<true>, grid, AT_THREADS, AT_SMEM, s, tq, tk, tv, p);
+    c == 4 ? launch(attn_tc_kernel<true, 4>)
+           : (c == 2 ? launch(attn_tc_kernel<true, 2>) : launch(attn_tc_kernel<true, 1>));
   else
-    launch_kernel(attn_tc_kernel<false>, grid, AT_THREADS, AT_SMEM, s, tq, tk, tv, p);
+    c == 4 ? launch(attn_tc_kernel<false, 4>)
+           : (c == 2 ? launch(attn_tc_kernel<false, 2>) : launch(attn_tc_kernel<false, 1>));
   return cudaGetLastError();
 }
 

@@ -227,6 +227,14 @@ BAG_DEV void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::
                    : "memory");
 }
+// Four floats to a 16-byte aligned shared::cluster address
+BAG_DEV void st_cluster4(uint32_t addr, float a, float b, float c, float d) {
+  asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(a), "f"(b), "f"(c), "f"(d)
+               : "memory");
+}
+BAG_DEV void st_cluster2(uint32_t addr, float a, float b) {
+  asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(addr), "f"(a), "f"(b) : "memory");
+}
 // TMA load into this CTA's shared memory whose completion is signalled on an mbarrier
 // of either CTA of the pair (shared::cluster address).
 BAG_DEV void tma_load_2d_pair(void* smem_dst, const CUtensorMap* map, int x, int y,

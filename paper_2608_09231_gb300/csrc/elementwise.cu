@@ -452,9 +452,7 @@ __global__ void __cluster_dims__(RC_CTAS, 1, 1) __launch_bounds__(RC_THREADS)
   if (warp == 0) {
     s = warp_sum2(lane < RC_THREADS / 32 ? red[lane] : make_float2(0.f, 0.f));
     if (lane == 0)
-      asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(mapa_shared(smem_u32(total + rank), 0)),
-                   "f"(s.x), "f"(s.y)
-                   : "memory");
+      st_cluster2(mapa_shared(smem_u32(total + rank), 0), s.x, s.y);
   }
   __syncwarp();
   cluster_sync_all();  // the sums have arrived; no access to another CTA follows

@@ -787,11 +787,6 @@ constexpr int SK_STAGE_BYTES = SK_A_BYTES + SK_B_BYTES;
 constexpr int SK_RECV_BYTES = TC_BM * SK_LD * 4;  // S slots of 128 / S rows
 constexpr int SK_SMEM = SK_STAGES * SK_STAGE_BYTES + SK_RECV_BYTES + 1024 + 256;
 
-BAG_DEV void st_cluster4(uint32_t addr, float a, float b, float c, float d) {
-  asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(a), "f"(b), "f"(c), "f"(d)
-               : "memory");
-}
-
 template <int S>
 __global__ void __launch_bounds__(192)
     gemm_splitk_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUtensorMap tmB0,

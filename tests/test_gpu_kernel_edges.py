@@ -148,3 +148,34 @@ def test_rel_l1_routes(rows, cols, dtype, offset, lib):
     assert bool(((part[:, 1] - den.sum(1)).abs() <= 2e-6 * den.sum(1)).all())
     assert float(scratch[offset + 2 * rows]) == 0.0
     assert torch.equal(out, again) and torch.equal(out, noalloc)
+
+
+@pytest.mark.parametrize("nq,nk,heads", [
+    (100, 1408, 1),    # 11 key tiles: not shared
+    (100, 1536, 2),    # four CTAs a unit, three tiles each
+    (257, 1537, 3),    # one key in the 13th tile, one row in the last query pair
+    (10240, 2049, 1),  # 40 units: two CTAs, eight or nine tiles
+    (2560, 2000, 16),  # 160 units on 152 SMs: the last eight are shared
+])
+@pytest.mark.parametrize("dtype", [torch.float16, torch.bfloat16])
+def test_attention_shared_units(nq, nk, heads, dtype, lib):
+    """Units shared by a cluster against fp64: the output's bf16 rounding (2^-8 relative) plus
+    the operand type's rounding of P (2^-11 or 2^-8 of the largest output)."""
+    ctx = bag.create("tiny", T=2, B=1)
+    g = torch.Generator(device="cuda").manual_seed(nq + nk)
+    q, k, v = (torch.randn(n, heads, 128, generator=g, device="cuda").to(dtype) for n in (nq, nk, nk))
+    vpad = (nk + 127) // 128 * 128
+    vt = torch.zeros(heads, 128, vpad, device="cuda", dtype=dtype)
+    vt[:, :, :nk] = v.permute(1, 2, 0)
+    o = torch.full((nq + 1, heads * 128), 9.0, device="cuda", dtype=torch.bfloat16)
+    call = ctx.attention_f16 if dtype == torch.float16 else ctx.attention_bf16
+    call(q.reshape(nq, -1), k.reshape(nk, -1), vt, o, nq, nk, heads, 128, vpad)
+    torch.cuda.synchronize()
+    ctx.close()
+    for h in range(heads):
+        p = torch.softmax(q[:, h].double() @ k[:, h].double().T / 128 ** 0.5, -1)
+        ref = p @ v[:, h].double()
+        err = (o[:nq, 128 * h:128 * h + 128].double() - ref).abs()
+        share = 2.0 ** -10 if dtype == torch.float16 else 2.0 ** -8
+        assert bool((err <= 2.0 ** -8 * ref.abs() + share * ref.abs().max()).all()), h
+    assert bool((o[nq] == 9.0).all())
