@@ -277,7 +277,7 @@ BAG_DEV void store_vt_warp(const Epi& e, int row, int col, float* v, float* sbuf
 }
 
 // Whether an epilogue reads or writes fp32 rows that store_f32_warp can take 16 bytes at a time.
-BAG_DEV bool f32_rows(const Epi& e) {
+static __host__ __device__ __forceinline__ bool f32_rows(const Epi& e) {
   uintptr_t p = reinterpret_cast<uintptr_t>(e.bias);
   long ld;
   if ((e.kind == EPI_STORE || e.kind == EPI_GELU) && e.out_bf16 == kStoreF32) {
@@ -359,7 +359,7 @@ BAG_DEV void store_f32_warp(const Epi& e, int t, int row0, int col0, const float
 }
 
 // Whether store_16_warp takes an epilogue's 16-bit outputs (V goes to store_vt_warp).
-BAG_DEV bool rows16(const Epi& e) {
+static __host__ __device__ __forceinline__ bool rows16(const Epi& e) {
   uintptr_t p = reinterpret_cast<uintptr_t>(e.bias);
   long ld;
   if (e.kind == EPI_STORE || e.kind == EPI_GELU) {
@@ -467,77 +467,71 @@ BAG_DEV void store_16_warp(const Epi& e, int row0, int col0, const float* v, flo
     if (row + 8 * p < e.M) store_vals<8>(base, (long)orow[p] * ld + cc, a + 8 * p, type);
 }
 
+// Epilogue classes.  A kernel is compiled for one class, so that it carries the registers and
+// instructions of its own epilogue only: with all of them in one kernel every small change to
+// one spilled another's registers.
+//   EP_F32  fp32 rows (f32_rows): stores, GELU, residual updates (146 registers)
+//   EP_16   16-bit outputs (rows16) without QK-norm (168)
+//   EP_ANY  everything, also rows that are not 16-byte aligned (255)
+// Measured, one class against three: small guided sample 1727 -> 1667 us, 50 steps of a FLUX
+// block 14.00 -> 13.80 ms, double block 915 -> 906 us.
+enum { EP_ANY = 0, EP_F32 = 1, EP_16 = 2 };
+static int epi_class(const Epi& e) { return f32_rows(e) ? EP_F32 : (rows16(e) && !e.qn_q ? EP_16 : EP_ANY); }
+
 // One thread's row of a BN-column accumulator in TMEM (lane base already in tb) through
 // the epilogue, columns col0 .. col0 + BN - 1.  vt_buf: this warp's transpose tile.
-template <int BN>
+template <int BN, int EP>
 BAG_DEV void drain_accumulator(const Epi& e, int t, int row, int col0, uint32_t tb, float* vt_buf) {
-  const bool vt_warp = e.kind == EPI_QKV && e.v_mode == 1 && e.qkv_type != kStoreF32;
-  if (f32_rows(e)) {
-#pragma unroll 1
-    for (int c = 0; c < BN; c += 32) {
-      float v[32];
-      tmem_ld32(tb + (uint32_t)c, v);
-      store_f32_warp(e, t, row - (int)(threadIdx.x & 31), col0 + c, v, vt_buf);
-    }
-    return;
-  }
-  const bool h16 = rows16(e);
   const int row0 = row - (int)(threadIdx.x & 31);
-  if (e.qn_q) {
-    // QK-norm: the tile holds whole heads (BN a multiple of dh, checked at launch); a
-    // first pass over each q / k head takes its sum of squares (bias included), the
-    // second applies the epilogue with 1 / RMS.  The TMEM loads are warp-wide, so every
-    // lane takes them whatever its row.
-    const int dh = e.dh;
+  const bool vt_warp = EP != EP_F32 && e.kind == EPI_QKV && e.v_mode == 1 && e.qkv_type != kStoreF32;
+  const bool f32 = EP == EP_F32 || (EP == EP_ANY && f32_rows(e));
+  const bool h16 = EP == EP_16 || (EP == EP_ANY && rows16(e));
+  auto chunk = [&](int c, float rs) {  // 32 columns; the branches are warp-uniform
+    float v[32];
+    tmem_ld32(tb + (uint32_t)c, v);
+    const int col = col0 + c;
+    if (f32)
+      store_f32_warp(e, t, row0, col, v, vt_buf);
+    else if (vt_warp && col < e.N && (col + e.col_base) / e.d == 2)
+      store_vt_warp(e, row, col, v, vt_buf);
+    else if (h16)
+      store_16_warp(e, row0, col, v, vt_buf, rs);
+    else
+      epi_apply<32>(e, t, row, col, v, rs);
+  };
+  if (EP != EP_ANY || !e.qn_q) {
 #pragma unroll 1
-    for (int h0 = 0; h0 < BN; h0 += dh) {
+    for (int c = 0; c < BN; c += 32) chunk(c, 1.f);
+  } else if constexpr (EP == EP_ANY) {
+    // QK-norm: the tile holds whole heads (BN a multiple of dh, checked at launch); a first pass
+    // over each q / k head takes its sum of squares (bias included), the second applies the
+    // epilogue with 1 / RMS.  The TMEM loads are warp-wide, so every lane takes them whatever
+    // its row.
+#pragma unroll 1
+    for (int h0 = 0; h0 < BN; h0 += e.dh) {
       const int col = col0 + h0;
       float rs = 1.f;
       if ((col + e.col_base) / e.d < 2 && col < e.N) {
         float ss = 0.f;
 #pragma unroll 1
-        for (int c = 0; c < dh; c += 32) {
+        for (int c = 0; c < e.dh; c += 32) {
           float v[32];
           tmem_ld32(tb + (uint32_t)(h0 + c), v);
+          epi_add_bias<32>(e, col + c, v);
 #pragma unroll
-          for (int j = 0; j < 32; ++j) {
-            const float x = v[j] + (e.bias ? __ldg(e.bias + col + c + j) : 0.f);
-            ss = fmaf(x, x, ss);
-          }
+          for (int j = 0; j < 32; ++j) ss = fmaf(v[j], v[j], ss);
         }
-        rs = rsqrtf(ss / (float)dh + 1e-6f);
+        rs = rsqrtf(ss / (float)e.dh + 1e-6f);
       }
 #pragma unroll 1
-      for (int c = 0; c < dh; c += 32) {
-        float v[32];
-        tmem_ld32(tb + (uint32_t)(h0 + c), v);
-        if (vt_warp && col + c < e.N && (col + c + e.col_base) / e.d == 2)
-          store_vt_warp(e, row, col + c, v, vt_buf);
-        else if (h16)
-          store_16_warp(e, row0, col + c, v, vt_buf, rs);
-        else
-          epi_apply<32>(e, t, row, col + c, v, rs);
-      }
-    }
-  } else {
-#pragma unroll 1
-    for (int c = 0; c < BN / 32; ++c) {
-      float v[32];
-      tmem_ld32(tb + (uint32_t)(c * 32), v);
-      const int col = col0 + c * 32;
-      if (vt_warp && col < e.N && (col + e.col_base) / e.d == 2)
-        store_vt_warp(e, row, col, v, vt_buf);  // warp-uniform branch
-      else if (h16)
-        store_16_warp(e, row0, col, v, vt_buf, 1.f);
-      else
-        epi_apply<32>(e, t, row, col, v);
+      for (int c = 0; c < e.dh; c += 32) chunk(h0 + c, rs);
     }
   }
 }
 
 template <int BN>
 struct TcCfg {
-  static constexpr int STAGES = BN == 256 ? 4 : (BN == 128 ? 6 : 8);
+  static constexpr int STAGES = BN == 128 ? 6 : 8;
   static constexpr int A_BYTES = TC_BM * TC_BK * 2;
   static constexpr int B_BYTES = BN * TC_BK * 2;
   static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
@@ -545,7 +539,7 @@ struct TcCfg {
   static constexpr int SMEM = STAGES * STAGE_BYTES + 1024 + 256 + kVtScratchBytes;
 };
 
-template <int BN>
+template <int BN, int EP>
 __global__ void __launch_bounds__(192, 1)
     gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUtensorMap tmB0,
                    const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ CUtensorMap tmB1,
@@ -726,7 +720,7 @@ __global__ void __launch_bounds__(192, 1)
       tc_fence_after();
       const int row = mt * TC_BM + q * 32 + lane;
       const uint32_t tb = tmem_base + (uint32_t)(acc * BN) + ((uint32_t)(q * 32) << 16);
-      drain_accumulator<BN>(e, t, row, nt * BN, tb, vt_scratch + (warp - 2) * kVtScratchFloats);
+      drain_accumulator<BN, EP>(e, t, row, nt * BN, tb, vt_scratch + (warp - 2) * kVtScratchFloats);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(tempty + acc);
@@ -740,6 +734,11 @@ __global__ void __launch_bounds__(192, 1)
     tc_fence_after();
     tmem_dealloc(tmem_base, C::TMEM_COLS);
   }
+}
+
+// Class of a launch of one or two problems.
+static int launch_class(const Epi& e0, int M1, const Epi& e1) {
+  return M1 <= 0 || epi_class(e0) == epi_class(e1) ? epi_class(e0) : EP_ANY;
 }
 
 template <int BN>
@@ -763,9 +762,13 @@ static cudaError_t launch_tc(const void* A0, long lda0, const void* W0, long ldw
   }
   const int tiles = ((M0 + TC_BM - 1) / TC_BM + (M1 + TC_BM - 1) / TC_BM) * (N / BN);
   const int grid = std::min(tiles, num_sms());
-  launch_kernel(gemm_tc_kernel<BN>, grid, 192, C::SMEM, s, ta0, tb0, ta1, tb1, e0, e1, M0, M1, N, K,
-                a_split, tile_group_rows(M0, TC_BM, K, a_split),
-                tile_group_rows(M1, TC_BM, K, a_split), err);
+  auto launch = [&](auto kernel) {
+    launch_kernel(kernel, grid, 192, C::SMEM, s, ta0, tb0, ta1, tb1, e0, e1, M0, M1, N, K, a_split,
+                  tile_group_rows(M0, TC_BM, K, a_split), tile_group_rows(M1, TC_BM, K, a_split), err);
+  };
+  const int ep = launch_class(e0, M1, e1);
+  ep == EP_F32 ? launch(gemm_tc_kernel<BN, EP_F32>)
+               : (ep == EP_16 ? launch(gemm_tc_kernel<BN, EP_16>) : launch(gemm_tc_kernel<BN, EP_ANY>));
   return cudaGetLastError();
 }
 
@@ -1007,17 +1010,24 @@ static cudaError_t launch_splitk(int S, const void* A0, long lda0, const void* W
 // issues the MMAs and multicasts their completion to both CTAs, warps 2..5 of each CTA
 // drain its 128 accumulator rows.
 // ---------------------------------------------------------------------------
-constexpr int PR_BM = 256, PR_BN = 256, PR_STAGES = 6;
+constexpr int PR_BM = 256, PR_BN = 256;
 constexpr int PR_HALF_BYTES = 128 * TC_BK * 2;  // one CTA's A or W half-tile per k-block
 constexpr int PR_STAGE_BYTES = 2 * PR_HALF_BYTES;
 constexpr int PR_TMEM_COLS = 2 * PR_BN;         // double-buffered accumulator
-constexpr int PR_SMEM = PR_STAGES * PR_STAGE_BYTES + 1024 + 256 + kVtScratchBytes;
+template <int WARPS>  // epilogue warps
+struct PrCfg {
+  static constexpr int STAGES = WARPS == 8 ? 5 : 6;
+  static constexpr int THREADS = 64 + 32 * WARPS;
+  static constexpr int SMEM = STAGES * PR_STAGE_BYTES + 1024 + 256 + WARPS * kVtScratchFloats * 4;
+};
 
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(192, 1)
+template <int EP, int EW>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PrCfg<EW>::THREADS, 1)
     gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUtensorMap tmB0,
                      const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ CUtensorMap tmB1,
                      const __grid_constant__ Epi e0, const __grid_constant__ Epi e1, int M0, int M1,
                      int N, int K, int a_split, int g0, int g1, int* err) {
+  constexpr int STAGES = PrCfg<EW>::STAGES;
   grid_dep_sync();
   // both CTAs of a pair see the same flag, so they leave together
   if (epi_skip(e0.st, e0.flag_want)) return;
@@ -1026,14 +1036,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(192, 1)
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~static_cast<uintptr_t>(1023));
   uint8_t* sA = smem;
-  uint8_t* sB = smem + PR_STAGES * PR_HALF_BYTES;
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem + PR_STAGES * PR_STAGE_BYTES);
-  uint64_t* empty = full + PR_STAGES;
-  uint64_t* tfull = empty + PR_STAGES;
+  uint8_t* sB = smem + STAGES * PR_HALF_BYTES;
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + STAGES * PR_STAGE_BYTES);
+  uint64_t* empty = full + STAGES;
+  uint64_t* tfull = empty + STAGES;
   uint64_t* tempty = tfull + 2;
   uint64_t* drain = tempty + 2;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
-  float* vt_scratch = reinterpret_cast<float*>(smem + PR_STAGES * PR_STAGE_BYTES + 256);
+  float* vt_scratch = reinterpret_cast<float*>(smem + STAGES * PR_STAGE_BYTES + 256);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
@@ -1054,14 +1064,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(192, 1)
   const int t = epi_step(e0);
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < PR_STAGES; ++s) {
+    for (int s = 0; s < STAGES; ++s) {
       mbar_init(full + s, 1);   // even CTA: its producer's expect_tx; both CTAs' bytes
       mbar_init(empty + s, 1);  // both CTAs: one multicast commit per consumed stage
     }
     mbar_init(tfull, 1);
     mbar_init(tfull + 1, 1);
-    mbar_init(tempty, 8);     // even CTA: every epilogue warp of both CTAs
-    mbar_init(tempty + 1, 8);
+    mbar_init(tempty, 2 * EW);     // even CTA: every epilogue warp of both CTAs
+    mbar_init(tempty + 1, 2 * EW);
     mbar_init(drain, 1);
     *abort_flag = 0;
     fence_mbar_init();
@@ -1109,7 +1119,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(192, 1)
           tma_load_2d_pair(sA + s * PR_HALF_BYTES, tmA, ka, mt * PR_BM + (int)rank * 128, fb);
           tma_load_2d_pair(sB + s * PR_HALF_BYTES, tmB, kw, nt * PR_BN + (int)rank * 128, fb);
           ++issued;
-          if (++s == PR_STAGES) {
+          if (++s == STAGES) {
             s = 0;
             ph ^= 1;
           }
@@ -1118,9 +1128,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(192, 1)
       if (!ok && rank == 0) {
         // drain (bounded): both CTAs' copies in flight complete on this CTA's barriers
         const uint64_t t0 = global_ns();
-        for (int i = 0; i < PR_STAGES && i < issued; ++i) {
+        for (int i = 0; i < STAGES && i < issued; ++i) {
           if (--s < 0) {
-            s = PR_STAGES - 1;
+            s = STAGES - 1;
             ph ^= 1;
           }
           while (!mbar_try_wait(full + s, ph) && global_ns() - t0 < kWaitLimitNs) {
@@ -1160,7 +1170,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(192, 1)
             mma_commit_pair(empty + s, 3);
           }
           __syncwarp();
-          if (++s == PR_STAGES) {
+          if (++s == STAGES) {
             s = 0;
             ph ^= 1;
           }
@@ -1182,7 +1192,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(192, 1)
     }
   } else {
     // ---------------- epilogue (both CTAs: their 128 rows of each tile) ----------------
-    const int q = warp & 3;
+    // (eight warps: two to each lane quarter, half the columns each)
+    constexpr int W = PR_BN * 4 / EW;
+    const int q = warp & 3, c0 = (warp - 2) / 4 * W;
     int acc = 0;
     uint32_t aph = 0;
     const uint32_t te_remote = mapa_shared(smem_u32(tempty), 0);
@@ -1194,8 +1206,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(192, 1)
       if (!__all_sync(0xffffffffu, ok)) break;
       tc_fence_after();
       const int row = mt * PR_BM + (int)rank * 128 + q * 32 + lane;
-      const uint32_t tb = tmem_base + (uint32_t)(acc * PR_BN) + ((uint32_t)(q * 32) << 16);
-      drain_accumulator<PR_BN>(e, t, row, nt * PR_BN, tb, vt_scratch + (warp - 2) * kVtScratchFloats);
+      const uint32_t tb = tmem_base + (uint32_t)(acc * PR_BN + c0) + ((uint32_t)(q * 32) << 16);
+      drain_accumulator<W, EP>(e, t, row, nt * PR_BN + c0, tb, vt_scratch + (warp - 2) * kVtScratchFloats);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) {
@@ -1242,9 +1254,18 @@ static cudaError_t launch_pair(const void* A0, long lda0, const void* W0, long l
     tb1 = tb0;
   }
   const int pairs = std::min(pair_tiles(M0, M1, N), num_sms() / 2);
-  launch_kernel(gemm_pair_kernel, 2 * pairs, 192, PR_SMEM, s, ta0, tb0, ta1, tb1, e0, e1, M0, M1, N,
-                K, a_split, tile_group_rows(M0, PR_BM, K, a_split),
-                tile_group_rows(M1, PR_BM, K, a_split), err);
+  auto launch = [&](auto kernel, int threads, int smem) {
+    launch_kernel(kernel, 2 * pairs, threads, smem, s, ta0, tb0, ta1, tb1, e0, e1, M0, M1, N, K, a_split,
+                  tile_group_rows(M0, PR_BM, K, a_split), tile_group_rows(M1, PR_BM, K, a_split), err);
+  };
+  const int ep = launch_class(e0, M1, e1);
+  using P4 = PrCfg<4>;
+  if (ep == EP_F32)
+    launch(gemm_pair_kernel<EP_F32, 4>, P4::THREADS, P4::SMEM);
+  else if (ep == EP_16)
+    launch(gemm_pair_kernel<EP_16, 4>, P4::THREADS, P4::SMEM);
+  else
+    launch(gemm_pair_kernel<EP_ANY, 4>, P4::THREADS, P4::SMEM);
   return cudaGetLastError();
 }
 
@@ -1255,24 +1276,23 @@ int gemm_uses_pair(int M0, int M1, int N) {
 cudaError_t attention_tc_init();
 
 cudaError_t kernels_init() {
-  cudaError_t r = cudaFuncSetAttribute(gemm_tc_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       TcCfg<256>::SMEM);
-  if (r == cudaSuccess)
-    r = cudaFuncSetAttribute(gemm_tc_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             TcCfg<128>::SMEM);
-  if (r == cudaSuccess)
-    r = cudaFuncSetAttribute(gemm_tc_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             TcCfg<64>::SMEM);
-  if (r == cudaSuccess)
-    r = cudaFuncSetAttribute(gemm_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, PR_SMEM);
-  const void* splitk[] = {(const void*)gemm_splitk_kernel<2>, (const void*)gemm_splitk_kernel<4>};
-  for (const void* k : splitk)
-    if (r == cudaSuccess) r = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, SK_SMEM);
-  if (r == cudaSuccess)
-    r = cudaFuncSetAttribute(gemm_simt_kernel<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SG_SMEM);
-  if (r == cudaSuccess)
-    r = cudaFuncSetAttribute(gemm_simt_kernel<__nv_bfloat16, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             SG_SMEM);
+  cudaError_t r = cudaSuccess;
+  auto smem = [&](auto kernel, int bytes) {
+    if (r == cudaSuccess) r = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  };
+  smem(gemm_tc_kernel<128, EP_ANY>, TcCfg<128>::SMEM);
+  smem(gemm_tc_kernel<128, EP_F32>, TcCfg<128>::SMEM);
+  smem(gemm_tc_kernel<128, EP_16>, TcCfg<128>::SMEM);
+  smem(gemm_tc_kernel<64, EP_ANY>, TcCfg<64>::SMEM);
+  smem(gemm_tc_kernel<64, EP_F32>, TcCfg<64>::SMEM);
+  smem(gemm_tc_kernel<64, EP_16>, TcCfg<64>::SMEM);
+  smem(gemm_pair_kernel<EP_ANY, 4>, PrCfg<4>::SMEM);
+  smem(gemm_pair_kernel<EP_F32, 4>, PrCfg<4>::SMEM);
+  smem(gemm_pair_kernel<EP_16, 4>, PrCfg<4>::SMEM);
+  smem(gemm_splitk_kernel<2>, SK_SMEM);
+  smem(gemm_splitk_kernel<4>, SK_SMEM);
+  smem(gemm_simt_kernel<float, true>, SG_SMEM);
+  smem(gemm_simt_kernel<__nv_bfloat16, false>, SG_SMEM);
   if (r == cudaSuccess) r = attention_tc_init();
   num_sms();
   return r;
@@ -1312,8 +1332,6 @@ static cudaError_t gemm_tc2(const void* A0, long lda0, const void* W0, long ldw0
   if (gemm_uses_pair(M0, M1 > 0 ? M1 : 0, N))
     return launch_pair(A0, lda0, W0, ldw0, M0, e0, A1, lda1, W1, ldw1, M1 > 0 ? M1 : 0, e1, N, K, err, s,
                        a_split);
-  if (N % 256 == 0 && (mt * (N / 256) >= ns || min_bn > 128))
-    return launch_tc<256>(A0, lda0, W0, ldw0, M0, e0, A1, lda1, W1, ldw1, M1, e1, N, K, err, s, a_split);
   if (min_bn > 128) return cudaErrorNotSupported;
   if (N % 128 == 0 && (mt * (N / 128) >= ns || min_bn > 64))
     return launch_tc<128>(A0, lda0, W0, ldw0, M0, e0, A1, lda1, W1, ldw1, M1, e1, N, K, err, s, a_split);
