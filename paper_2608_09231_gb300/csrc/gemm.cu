@@ -223,7 +223,6 @@ static int tile_group_rows(int M, int BM, int K, int a_split) {
 // 33 words; fp32 rows: 36 words, so that 16-byte accesses are aligned and conflict-free).
 constexpr int kF32Ld = 36;
 constexpr int kVtScratchFloats = 32 * kF32Ld;
-constexpr int kVtScratchBytes = 4 * kVtScratchFloats * 4;  // four epilogue warps
 
 BAG_DEV uint16_t to16(float x, bool f16) {
   return f16 ? __half_as_ushort(__float2half_rn(x)) : __bfloat16_as_ushort(__float2bfloat16_rn(x));
@@ -529,18 +528,24 @@ BAG_DEV void drain_accumulator(const Epi& e, int t, int row, int col0, uint32_t 
   }
 }
 
-template <int BN>
+// Epilogue warps: a launch on this kernel has a tile or two per SM, so its drain is hidden
+// behind little; eight warps (two to each lane quarter, half the columns each) halve it, where
+// the class leaves them the registers.  Small guided sample 1667 -> 1648 us, small Wan-shaped
+// sample 1115 -> 1098 us.
+template <int BN, int EP>
 struct TcCfg {
-  static constexpr int STAGES = BN == 128 ? 6 : 8;
+  static constexpr int WARPS = EP == EP_ANY ? 4 : 8;
+  static constexpr int THREADS = 64 + 32 * WARPS;
+  static constexpr int STAGES = (BN == 128 ? 6 : 8) - (WARPS == 8);
   static constexpr int A_BYTES = TC_BM * TC_BK * 2;
   static constexpr int B_BYTES = BN * TC_BK * 2;
   static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
   static constexpr int TMEM_COLS = 2 * BN;
-  static constexpr int SMEM = STAGES * STAGE_BYTES + 1024 + 256 + kVtScratchBytes;
+  static constexpr int SMEM = STAGES * STAGE_BYTES + 1024 + 256 + WARPS * kVtScratchFloats * 4;
 };
 
 template <int BN, int EP>
-__global__ void __launch_bounds__(192, 1)
+__global__ void __launch_bounds__(TcCfg<BN, EP>::THREADS, 1)
     gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUtensorMap tmB0,
                    const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ CUtensorMap tmB1,
                    const __grid_constant__ Epi e0, const __grid_constant__ Epi e1, int M0, int M1,
@@ -549,7 +554,7 @@ __global__ void __launch_bounds__(192, 1)
   // Two independent problems with the same N and K may share one launch (problem 1 has
   // M1 rows, possibly 0): their tiles form one list, problem 0's first, so a small
   // problem fills the SMs the large one leaves idle in its last wave.
-  using C = TcCfg<BN>;
+  using C = TcCfg<BN, EP>;
   if (epi_skip(e0.st, e0.flag_want)) return;
   epi_bump(e0);
   extern __shared__ uint8_t smem_raw[];
@@ -591,8 +596,8 @@ __global__ void __launch_bounds__(192, 1)
     }
     mbar_init(tfull, 1);
     mbar_init(tfull + 1, 1);
-    mbar_init(tempty, 4);       // one arrival per epilogue warp
-    mbar_init(tempty + 1, 4);
+    mbar_init(tempty, C::WARPS);  // one arrival per epilogue warp
+    mbar_init(tempty + 1, C::WARPS);
     mbar_init(drain, 1);
     *abort_flag = 0;
     fence_mbar_init();
@@ -707,8 +712,9 @@ __global__ void __launch_bounds__(192, 1)
     }
     __syncwarp();
   } else {
-    // ---------------- epilogue (warps 2..5 cover TMEM lane quarters 2,3,0,1) ----------------
-    const int q = warp & 3;
+    // ---------------- epilogue (each four warps cover TMEM lane quarters 2,3,0,1) ----------------
+    constexpr int W = BN * 4 / C::WARPS;
+    const int q = warp & 3, c0 = (warp - 2) / 4 * W;
     int acc = 0;
     uint32_t aph = 0;
     for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
@@ -719,8 +725,8 @@ __global__ void __launch_bounds__(192, 1)
       if (!__all_sync(0xffffffffu, ok)) break;
       tc_fence_after();
       const int row = mt * TC_BM + q * 32 + lane;
-      const uint32_t tb = tmem_base + (uint32_t)(acc * BN) + ((uint32_t)(q * 32) << 16);
-      drain_accumulator<BN, EP>(e, t, row, nt * BN, tb, vt_scratch + (warp - 2) * kVtScratchFloats);
+      const uint32_t tb = tmem_base + (uint32_t)(acc * BN + c0) + ((uint32_t)(q * 32) << 16);
+      drain_accumulator<W, EP>(e, t, row, nt * BN + c0, tb, vt_scratch + (warp - 2) * kVtScratchFloats);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(tempty + acc);
@@ -746,7 +752,6 @@ static cudaError_t launch_tc(const void* A0, long lda0, const void* W0, long ldw
                              const Epi& e0, const void* A1, long lda1, const void* W1, long ldw1,
                              int M1, const Epi& e1, int N, int K, int* err, cudaStream_t s,
                              int a_split) {
-  using C = TcCfg<BN>;
   const uint64_t ka = (uint64_t)K * (a_split ? 2 : 1);
   CUtensorMap ta0, tb0, ta1, tb1;
   if (encode_tmap_2d_bf16(&ta0, A0, ka, (uint64_t)M0, (uint64_t)lda0 * 2, TC_BK, TC_BM) ||
@@ -762,13 +767,17 @@ static cudaError_t launch_tc(const void* A0, long lda0, const void* W0, long ldw
   }
   const int tiles = ((M0 + TC_BM - 1) / TC_BM + (M1 + TC_BM - 1) / TC_BM) * (N / BN);
   const int grid = std::min(tiles, num_sms());
-  auto launch = [&](auto kernel) {
-    launch_kernel(kernel, grid, 192, C::SMEM, s, ta0, tb0, ta1, tb1, e0, e1, M0, M1, N, K, a_split,
+  auto launch = [&](auto kernel, int threads, int smem) {
+    launch_kernel(kernel, grid, threads, smem, s, ta0, tb0, ta1, tb1, e0, e1, M0, M1, N, K, a_split,
                   tile_group_rows(M0, TC_BM, K, a_split), tile_group_rows(M1, TC_BM, K, a_split), err);
   };
   const int ep = launch_class(e0, M1, e1);
-  ep == EP_F32 ? launch(gemm_tc_kernel<BN, EP_F32>)
-               : (ep == EP_16 ? launch(gemm_tc_kernel<BN, EP_16>) : launch(gemm_tc_kernel<BN, EP_ANY>));
+  if (ep == EP_F32)
+    launch(gemm_tc_kernel<BN, EP_F32>, TcCfg<BN, EP_F32>::THREADS, TcCfg<BN, EP_F32>::SMEM);
+  else if (ep == EP_16)
+    launch(gemm_tc_kernel<BN, EP_16>, TcCfg<BN, EP_16>::THREADS, TcCfg<BN, EP_16>::SMEM);
+  else
+    launch(gemm_tc_kernel<BN, EP_ANY>, TcCfg<BN, EP_ANY>::THREADS, TcCfg<BN, EP_ANY>::SMEM);
   return cudaGetLastError();
 }
 
@@ -1014,7 +1023,10 @@ constexpr int PR_BM = 256, PR_BN = 256;
 constexpr int PR_HALF_BYTES = 128 * TC_BK * 2;  // one CTA's A or W half-tile per k-block
 constexpr int PR_STAGE_BYTES = 2 * PR_HALF_BYTES;
 constexpr int PR_TMEM_COLS = 2 * PR_BN;         // double-buffered accumulator
-template <int WARPS>  // epilogue warps
+// WARPS epilogue warps.  Four drain a tile while the next one is multiplied; with few K blocks
+// the drain is the longer part, and eight (two to each lane quarter, half the columns each)
+// halve it, at the price of a stage of the ring.
+template <int WARPS>
 struct PrCfg {
   static constexpr int STAGES = WARPS == 8 ? 5 : 6;
   static constexpr int THREADS = 64 + 32 * WARPS;
@@ -1259,8 +1271,13 @@ static cudaError_t launch_pair(const void* A0, long lda0, const void* W0, long l
                   tile_group_rows(M0, PR_BM, K, a_split), tile_group_rows(M1, PR_BM, K, a_split), err);
   };
   const int ep = launch_class(e0, M1, e1);
+  // fp32 rows with at most 16 K blocks take eight epilogue warps: 4096 x 3072 x 128 27.2 -> 22.5
+  // us as a profiled launch, 1373 x 12288 x 3072 with GELU 74.8 -> 75.8
   using P4 = PrCfg<4>;
-  if (ep == EP_F32)
+  using P8 = PrCfg<8>;
+  if (ep == EP_F32 && (a_split ? 2 : 1) * (K / TC_BK) <= 16)
+    launch(gemm_pair_kernel<EP_F32, 8>, P8::THREADS, P8::SMEM);
+  else if (ep == EP_F32)
     launch(gemm_pair_kernel<EP_F32, 4>, P4::THREADS, P4::SMEM);
   else if (ep == EP_16)
     launch(gemm_pair_kernel<EP_16, 4>, P4::THREADS, P4::SMEM);
@@ -1280,14 +1297,15 @@ cudaError_t kernels_init() {
   auto smem = [&](auto kernel, int bytes) {
     if (r == cudaSuccess) r = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   };
-  smem(gemm_tc_kernel<128, EP_ANY>, TcCfg<128>::SMEM);
-  smem(gemm_tc_kernel<128, EP_F32>, TcCfg<128>::SMEM);
-  smem(gemm_tc_kernel<128, EP_16>, TcCfg<128>::SMEM);
-  smem(gemm_tc_kernel<64, EP_ANY>, TcCfg<64>::SMEM);
-  smem(gemm_tc_kernel<64, EP_F32>, TcCfg<64>::SMEM);
-  smem(gemm_tc_kernel<64, EP_16>, TcCfg<64>::SMEM);
+  smem(gemm_tc_kernel<128, EP_ANY>, TcCfg<128, EP_ANY>::SMEM);
+  smem(gemm_tc_kernel<128, EP_F32>, TcCfg<128, EP_F32>::SMEM);
+  smem(gemm_tc_kernel<128, EP_16>, TcCfg<128, EP_16>::SMEM);
+  smem(gemm_tc_kernel<64, EP_ANY>, TcCfg<64, EP_ANY>::SMEM);
+  smem(gemm_tc_kernel<64, EP_F32>, TcCfg<64, EP_F32>::SMEM);
+  smem(gemm_tc_kernel<64, EP_16>, TcCfg<64, EP_16>::SMEM);
   smem(gemm_pair_kernel<EP_ANY, 4>, PrCfg<4>::SMEM);
   smem(gemm_pair_kernel<EP_F32, 4>, PrCfg<4>::SMEM);
+  smem(gemm_pair_kernel<EP_F32, 8>, PrCfg<8>::SMEM);
   smem(gemm_pair_kernel<EP_16, 4>, PrCfg<4>::SMEM);
   smem(gemm_splitk_kernel<2>, SK_SMEM);
   smem(gemm_splitk_kernel<4>, SK_SMEM);
