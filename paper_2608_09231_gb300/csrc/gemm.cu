@@ -471,11 +471,12 @@ BAG_DEV void store_16_warp(const Epi& e, int row0, int col0, const float* v, flo
 // one spilled another's registers.
 //   EP_F32  fp32 rows (f32_rows): stores, GELU, residual updates (146 registers)
 //   EP_16   16-bit outputs (rows16) without QK-norm (168)
-//   EP_ANY  everything, also rows that are not 16-byte aligned (255)
-// Measured, one class against three: small guided sample 1727 -> 1667 us, 50 steps of a FLUX
-// block 14.00 -> 13.80 ms, double block 915 -> 906 us.
-enum { EP_ANY = 0, EP_F32 = 1, EP_16 = 2 };
-static int epi_class(const Epi& e) { return f32_rows(e) ? EP_F32 : (rows16(e) && !e.qn_q ? EP_16 : EP_ANY); }
+//   EP_16N  16-bit outputs with QK-norm (168)
+//   EP_ANY  everything without QK-norm, also rows that are not 16-byte aligned (254)
+// Measured, one class against four: small guided sample 1727 -> 1634 us, 50 steps of a FLUX
+// block 14.00 -> 13.80 ms, double block 915 -> 896 us.
+enum { EP_ANY = 0, EP_F32 = 1, EP_16 = 2, EP_16N = 3 };
+static int epi_class(const Epi& e) { return f32_rows(e) ? EP_F32 : (rows16(e) ? (e.qn_q ? EP_16N : EP_16) : EP_ANY); }
 
 // One thread's row of a BN-column accumulator in TMEM (lane base already in tb) through
 // the epilogue, columns col0 .. col0 + BN - 1.  vt_buf: this warp's transpose tile.
@@ -484,7 +485,7 @@ BAG_DEV void drain_accumulator(const Epi& e, int t, int row, int col0, uint32_t 
   const int row0 = row - (int)(threadIdx.x & 31);
   const bool vt_warp = EP != EP_F32 && e.kind == EPI_QKV && e.v_mode == 1 && e.qkv_type != kStoreF32;
   const bool f32 = EP == EP_F32 || (EP == EP_ANY && f32_rows(e));
-  const bool h16 = EP == EP_16 || (EP == EP_ANY && rows16(e));
+  const bool h16 = EP == EP_16 || EP == EP_16N || (EP == EP_ANY && rows16(e));
   auto chunk = [&](int c, float rs) {  // 32 columns; the branches are warp-uniform
     float v[32];
     tmem_ld32(tb + (uint32_t)c, v);
@@ -498,10 +499,10 @@ BAG_DEV void drain_accumulator(const Epi& e, int t, int row, int col0, uint32_t 
     else
       epi_apply<32>(e, t, row, col, v, rs);
   };
-  if (EP != EP_ANY || !e.qn_q) {
+  if constexpr (EP != EP_16N) {
 #pragma unroll 1
     for (int c = 0; c < BN; c += 32) chunk(c, 1.f);
-  } else if constexpr (EP == EP_ANY) {
+  } else {
     // QK-norm: the tile holds whole heads (BN a multiple of dh, checked at launch); a first pass
     // over each q / k head takes its sum of squares (bias included), the second applies the
     // epilogue with 1 / RMS.  The TMEM loads are warp-wide, so every lane takes them whatever
@@ -534,7 +535,7 @@ BAG_DEV void drain_accumulator(const Epi& e, int t, int row, int col0, uint32_t 
 // sample 1115 -> 1098 us.
 template <int BN, int EP>
 struct TcCfg {
-  static constexpr int WARPS = EP == EP_ANY ? 4 : 8;
+  static constexpr int WARPS = EP == EP_F32 || EP == EP_16 ? 8 : 4;
   static constexpr int THREADS = 64 + 32 * WARPS;
   static constexpr int STAGES = (BN == 128 ? 6 : 8) - (WARPS == 8);
   static constexpr int A_BYTES = TC_BM * TC_BK * 2;
@@ -776,6 +777,8 @@ static cudaError_t launch_tc(const void* A0, long lda0, const void* W0, long ldw
     launch(gemm_tc_kernel<BN, EP_F32>, TcCfg<BN, EP_F32>::THREADS, TcCfg<BN, EP_F32>::SMEM);
   else if (ep == EP_16)
     launch(gemm_tc_kernel<BN, EP_16>, TcCfg<BN, EP_16>::THREADS, TcCfg<BN, EP_16>::SMEM);
+  else if (ep == EP_16N)
+    launch(gemm_tc_kernel<BN, EP_16N>, TcCfg<BN, EP_16N>::THREADS, TcCfg<BN, EP_16N>::SMEM);
   else
     launch(gemm_tc_kernel<BN, EP_ANY>, TcCfg<BN, EP_ANY>::THREADS, TcCfg<BN, EP_ANY>::SMEM);
   return cudaGetLastError();
@@ -1281,6 +1284,8 @@ static cudaError_t launch_pair(const void* A0, long lda0, const void* W0, long l
     launch(gemm_pair_kernel<EP_F32, 4>, P4::THREADS, P4::SMEM);
   else if (ep == EP_16)
     launch(gemm_pair_kernel<EP_16, 4>, P4::THREADS, P4::SMEM);
+  else if (ep == EP_16N)
+    launch(gemm_pair_kernel<EP_16N, 4>, P4::THREADS, P4::SMEM);
   else
     launch(gemm_pair_kernel<EP_ANY, 4>, P4::THREADS, P4::SMEM);
   return cudaGetLastError();
@@ -1300,6 +1305,8 @@ cudaError_t kernels_init() {
   smem(gemm_tc_kernel<128, EP_ANY>, TcCfg<128, EP_ANY>::SMEM);
   smem(gemm_tc_kernel<128, EP_F32>, TcCfg<128, EP_F32>::SMEM);
   smem(gemm_tc_kernel<128, EP_16>, TcCfg<128, EP_16>::SMEM);
+  smem(gemm_tc_kernel<128, EP_16N>, TcCfg<128, EP_16N>::SMEM);
+  smem(gemm_tc_kernel<64, EP_16N>, TcCfg<64, EP_16N>::SMEM);
   smem(gemm_tc_kernel<64, EP_ANY>, TcCfg<64, EP_ANY>::SMEM);
   smem(gemm_tc_kernel<64, EP_F32>, TcCfg<64, EP_F32>::SMEM);
   smem(gemm_tc_kernel<64, EP_16>, TcCfg<64, EP_16>::SMEM);
@@ -1307,6 +1314,7 @@ cudaError_t kernels_init() {
   smem(gemm_pair_kernel<EP_F32, 4>, PrCfg<4>::SMEM);
   smem(gemm_pair_kernel<EP_F32, 8>, PrCfg<8>::SMEM);
   smem(gemm_pair_kernel<EP_16, 4>, PrCfg<4>::SMEM);
+  smem(gemm_pair_kernel<EP_16N, 4>, PrCfg<4>::SMEM);
   smem(gemm_splitk_kernel<2>, SK_SMEM);
   smem(gemm_splitk_kernel<4>, SK_SMEM);
   smem(gemm_simt_kernel<float, true>, SG_SMEM);
@@ -1339,7 +1347,9 @@ static cudaError_t gemm_tc2(const void* A0, long lda0, const void* W0, long ldw0
   // QK-norm epilogues need whole heads in a tile: BN a multiple of dh
   const bool qkn = e0.qn_q || (M1 > 0 && e1.qn_q);
   const int min_bn = qkn ? e0.dh : 64;
-  if (qkn && (e0.dh % 32 || (M1 > 0 && e1.dh != e0.dh) || min_bn > 256)) return cudaErrorNotSupported;
+  // and come with 16-byte aligned 16-bit operands (the contexts' buffers)
+  if (qkn && (e0.dh % 32 || (M1 > 0 && e1.dh != e0.dh) || min_bn > 256 || launch_class(e0, M1, e1) != EP_16N))
+    return cudaErrorNotSupported;
   if (e0.kind != EPI_QKV && (M1 <= 0 || e1.kind != EPI_QKV)) {
     const int mtp = e0.plan_rows > 0 ? (e0.plan_rows + TC_BM - 1) / TC_BM : mt;
     const int split = splitk_ctas(mtp * (N / SK_BN), (a_split ? 2 : 1) * (K / TC_BK), ns);
