@@ -978,12 +978,12 @@ __global__ void __launch_bounds__(192)
 // per SM (clusters of eight leave 32 of the 152 SMs without a place)
 // (1: the unsplit kernels).  A guided launch may hold twice the planned tiles; two CTAs fit
 // on an SM.
-#ifndef BAG_SPLITK_MIN_KB
-#define BAG_SPLITK_MIN_KB 4
-#endif
+// Fewest blocks a CTA: 2 against 4 makes the small Wan-shaped sample 1113 -> 1037 us, the small
+// guided one 1630 -> 1600 (8: 1.5 % slower than 4).  Up to two CTAs an SM: small guided 1592 -> 1663.
+constexpr int SK_MIN_KB = 2;
 static int splitk_ctas(int tiles, int kit, int ns) {
   for (int s = 4; s > 1; s /= 2)
-    if (tiles * s <= ns && kit >= s * BAG_SPLITK_MIN_KB) return s;
+    if (tiles * s <= ns && kit >= s * SK_MIN_KB) return s;
   return 1;
 }
 
