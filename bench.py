@@ -384,11 +384,12 @@ def job_seconds_per_sample(ms_per_step_max, world):
 
 
 def budget_overhead(sweep, prof, T):
-    """How s/sample scales with the budget (the benchmark spec: with B/T plus a measured gate and
-    skip overhead).  sweep: {B: s/sample}; prof: the profiled sample's per-class times.
+    """How s/sample scales with the budget (with B/T plus the measured gate
+    and skip overhead).  sweep: {B: s/sample}; prof: the profiled sample's per-class times.
     A least-squares line s(B) = slope * B + fixed over the swept budgets gives the cost of
     one more full step and the budget-independent part; the profiled sample gives the
-    per-step cost of the method's own kernels (signal, gate, cache refresh / reuse)."""
+    per-step cost of the method's own kernels (signal, gate, stream set-up; the cache is
+    part of the final norm)."""
     out = {}
     pts = sorted((int(b), float(v)) for b, v in sweep.items())
     if len(pts) >= 2:

@@ -1,18 +1,18 @@
 // C ABI of the BAG sampler: context (weights, activation arena, device state), the
 // per-sample conditioning precompute, one denoising step as a CUDA graph whose
-// full-network body and residual-reuse body hang off a conditional node that the gate
-// kernel sets on the device, and the single-operation entry points.
+// full-network body hangs off a conditional node that the gate kernel sets on the device,
+// and the single-operation entry points.
 //
 // One step, as enqueued (Algorithm 2, one iteration):
-//   prefix : patch embed  h_in = x W_pe^T + b  (also seeds the image stream)
+//   prefix : patch embed  t += 1, h_in = x W_pe^T + b
 //            signal       m_t = LN-mod of h_in with block 0's first modulation (or h_in
 //                         itself, the paper's post-patch-embedding observable), fused
 //                         with the per-row partial sums of |m_t - m_last| and |m_last|;
 //                         after a full step it also takes m_last <- m_{t-1}
 //            gate         drift, gate MLP, forced rules, counters, log, decision
-//   full   : text tokens -> stream, every block, R = h_out - h_in
-//   reuse  : h_out = h_in + R
-//   suffix : final LN-mod + projection fused with the Euler update, t += 1
+//   full   : text tokens and h_in -> stream, every block
+//   suffix : final LN-mod of h_out (full step: of the stream, with R = h_out - h_in kept;
+//            reused step: of h_in + R) + projection fused with the Euler update
 #include <algorithm>
 #include <cmath>
 #include <cstdlib>
