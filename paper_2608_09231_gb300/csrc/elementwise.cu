@@ -80,6 +80,17 @@ BAG_DEV void load4(const void* p, long off, int bf16, float* r) {
   }
 }
 
+// Four floats of a row that this SM reads once: they take no L1 lines from the modulation
+// vectors, which every row reads.  4608 x 3072 from HBM 24.4 -> 23.5 us, 50 steps of a FLUX block
+// 13.51 -> 13.39 ms (from L2 14.4 -> 15.2 us on one buffer over and over).
+BAG_DEV float4 ld_once(const float4* p) {
+  float4 v;
+  asm volatile("ld.global.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "l"(p));
+  return v;
+}
+
 // Bulk prefetch of `bytes` (a multiple of 16, 16-byte aligned) into L2.
 BAG_DEV void l2_prefetch(const void* p, uint32_t bytes) {
   asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(reinterpret_cast<uint64_t>(p)), "r"(bytes)
@@ -148,8 +159,8 @@ __global__ void __launch_bounds__(TH, MINB) ln_mod_kernel(const LnArgs a) {
     for (int i = 0; i < VPT; ++i) {
       const int c = threadIdx.x + i * TH;
       if (c < nv) {
-        v[i] = src[c];
-        h[i] = hin[c];
+        v[i] = ld_once(src + c);
+        h[i] = ld_once(hin + c);
       }
     }
 #pragma unroll
@@ -167,7 +178,7 @@ __global__ void __launch_bounds__(TH, MINB) ln_mod_kernel(const LnArgs a) {
   for (int i = 0; i < VPT; ++i) {
     const int c = threadIdx.x + i * TH;
     if (c < nv) {
-      if constexpr (MODE != LN_CACHE) v[i] = reinterpret_cast<const float4*>(x)[c];
+      if constexpr (MODE != LN_CACHE) v[i] = ld_once(reinterpret_cast<const float4*>(x) + c);
       s += (v[i].x + v[i].y) + (v[i].z + v[i].w);
     }
   }
