@@ -1,12 +1,14 @@
 // Projections of the DiT block: C[M,N] = A[M,K] W[N,K]^T with a fused epilogue.
 //
-// bf16 operands run on the 5th-generation tensor cores: a persistent, warp-specialised
-// kernel with one TMA producer warp, one MMA-issuing warp and four epilogue warps.
-// Operand tiles (128 x 64 of A, BN x 64 of W, 128-byte swizzle) stream through a
-// multi-stage shared-memory ring guarded by mbarriers; tcgen05.mma accumulates a
-// 128 x BN fp32 tile in tensor memory, double-buffered so the epilogue of one tile
-// overlaps the main loop of the next.  fp32 operands (the fp32 configuration, which
-// must hold 1e-4 relative parity) use a CUDA-core kernel with the same epilogue.
+// bf16 operands run on the 5th-generation tensor cores: warp-specialised kernels with one TMA
+// producer warp, one MMA-issuing warp and four or eight epilogue warps.  Operand tiles (64
+// columns wide, 128-byte swizzle) stream through a multi-stage shared-memory ring guarded by
+// mbarriers; tcgen05.mma accumulates fp32 tiles in tensor memory.  Three of them: CTA pairs
+// with 256 x 256 tiles, and single CTAs with 128 x 128 or 128 x 64 tiles (both persistent,
+// accumulators double-buffered so that the epilogue of one tile overlaps the main loop of the
+// next), and clusters that split K where there are few tiles.  fp32 operands (the fp32
+// configuration, which must hold 1e-4 relative parity) use a CUDA-core kernel with the same
+// epilogue.
 #include <algorithm>
 #include <cstdio>
 #include <mutex>
@@ -472,7 +474,8 @@ BAG_DEV void store_16_warp(const Epi& e, int row0, int col0, const float* v, flo
 //   EP_F32  fp32 rows (f32_rows): stores, GELU, residual updates (146 registers)
 //   EP_16   16-bit outputs (rows16) without QK-norm (168)
 //   EP_16N  16-bit outputs with QK-norm (168)
-//   EP_ANY  everything without QK-norm, also rows that are not 16-byte aligned (254)
+//   EP_ANY  everything without QK-norm, also rows that are not 16-byte aligned, and launches of
+//           two problems whose classes differ (254)
 // Measured, one class against four: small guided sample 1727 -> 1634 us, 50 steps of a FLUX
 // block 14.00 -> 13.80 ms, double block 915 -> 896 us.
 enum { EP_ANY = 0, EP_F32 = 1, EP_16 = 2, EP_16N = 3 };
