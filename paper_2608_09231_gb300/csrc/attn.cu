@@ -27,27 +27,31 @@ BAG_DEV float4 ldv4(const void* p, long i) {
     return make_float4(ldv<T>(p, i), ldv<T>(p, i + 1), ldv<T>(p, i + 2), ldv<T>(p, i + 3));
 }
 
-// CTA = eight queries of one head; its eight warps take the key tiles (32 keys) in turn,
-// each with its own running maximum, sum and output for all eight queries, merged in warp
-// order at the end.  Scores: lane = key, which reads its own K row four elements at a time
+// CTA = eight queries of one head; its warps take the key tiles (32 keys) in turn, each with
+// its own running maximum, sum and output for all eight queries, merged in warp order at the
+// end.  Scores: lane = key, which reads its own K row four elements at a time
 // against the queries broadcast from shared memory (8 x 4 products per K load); the
 // weights pass through shared memory so that the output has lane = head dimensions and
 // reads V rows coalesced.  Bound: latency (the fp32 backbones have a few hundred tokens);
 // few queries per CTA and the keys split over warps keep every SM busy with a short chain.
 // Measured against sixteen queries per CTA whose four warps walked all keys one barrier
-// after another (profiled launches): 288 tokens x 4 heads of 64 41 -> 20 us.
-constexpr int SA_Q = 8, SA_WARPS = 8, SA_KT = 32;
+// after another (profiled launches): 288 tokens x 4 heads of 64 41 -> 19.2 us with eight warps,
+// which leave the ninth tile for a second round; 14.4 with twelve, 16.4 with sixteen.  Heads
+// of 64 take twelve past 256 keys; heads of 128 eight (the outputs to merge take 4 KB a warp).
+constexpr int SA_Q = 8, SA_KT = 32;
 
-template <typename T, int DH>
+template <typename T, int DH, int SA_WARPS>
 __global__ void __launch_bounds__(SA_WARPS * 32) attn_simt_kernel(const AttnArgs a) {
   grid_dep_sync();
   if (epi_skip(a.st, a.flag_want)) return;
   constexpr int R = DH / 32;  // head dimensions per lane: lane * R .. lane * R + R - 1
   __shared__ __align__(16) float Qs[SA_Q][DH];
-  __shared__ __align__(16) float Ps[SA_WARPS][SA_Q][SA_KT];
-  __shared__ float Os[SA_WARPS][SA_Q][DH], ms[SA_WARPS][SA_Q], ls[SA_WARPS][SA_Q];
+  // a warp's weights of one key tile, and at the end its outputs, share its part of Os
+  __shared__ __align__(16) float Os[SA_WARPS][SA_Q][DH];
+  __shared__ float ms[SA_WARPS][SA_Q], ls[SA_WARPS][SA_Q];
   const int head = blockIdx.y, q0 = blockIdx.x * SA_Q;
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  float(*Ps)[SA_KT] = reinterpret_cast<float(*)[SA_KT]>(Os[warp]);
   const float scale = rsqrtf((float)DH);
   for (int i = threadIdx.x; i < SA_Q * DH; i += blockDim.x) {
     const int r = i / DH, c = i % DH, q = q0 + r;
@@ -92,7 +96,7 @@ __global__ void __launch_bounds__(SA_WARPS * 32) attn_simt_kernel(const AttnArgs
       const float base = mn == -INFINITY ? 0.f : mn;
       const float p = expf(si - base);  // 0 past the last key
       const float corr = expf(m[i] - base);
-      Ps[warp][i][lane] = p;
+      Ps[i][lane] = p;
       l[i] = l[i] * corr + p;
 #pragma unroll
       for (int r = 0; r < R; ++r) o[i][r] *= corr;
@@ -113,7 +117,7 @@ __global__ void __launch_bounds__(SA_WARPS * 32) attn_simt_kernel(const AttnArgs
       }
 #pragma unroll
       for (int i = 0; i < SA_Q; ++i) {
-        const float4 p4 = *reinterpret_cast<const float4*>(&Ps[warp][i][j]);
+        const float4 p4 = *reinterpret_cast<const float4*>(&Ps[i][j]);
 #pragma unroll
         for (int r = 0; r < R; ++r) {
           o[i][r] += p4.x * v[0][r];
@@ -124,6 +128,7 @@ __global__ void __launch_bounds__(SA_WARPS * 32) attn_simt_kernel(const AttnArgs
       }
     }
   }
+  __syncwarp();  // every lane has read the last tile's weights
 #pragma unroll
   for (int i = 0; i < SA_Q; ++i) {
 #pragma unroll
@@ -172,19 +177,15 @@ cudaError_t attention(const AttnArgs& a, int* err, cudaStream_t s, int force_sim
   }
   if (a.f16 || a.nbr > 1) return cudaErrorNotSupported;  // tensor-core kernel only
   dim3 grid((a.nq + SA_Q - 1) / SA_Q, a.heads);
-  if (a.dh == 64) {
-    if (a.bf16)
-      launch_kernel(attn_simt_kernel<__nv_bfloat16, 64>, grid, SA_WARPS * 32, 0, s, a);
-    else
-      launch_kernel(attn_simt_kernel<float, 64>, grid, SA_WARPS * 32, 0, s, a);
-  } else if (a.dh == 128) {
-    if (a.bf16)
-      launch_kernel(attn_simt_kernel<__nv_bfloat16, 128>, grid, SA_WARPS * 32, 0, s, a);
-    else
-      launch_kernel(attn_simt_kernel<float, 128>, grid, SA_WARPS * 32, 0, s, a);
-  } else {
+  auto launch = [&](auto kernel, int warps) { launch_kernel(kernel, grid, warps * 32, 0, s, a); };
+  if (a.dh == 64 && a.nk > 8 * SA_KT)
+    a.bf16 ? launch(attn_simt_kernel<__nv_bfloat16, 64, 12>, 12) : launch(attn_simt_kernel<float, 64, 12>, 12);
+  else if (a.dh == 64)
+    a.bf16 ? launch(attn_simt_kernel<__nv_bfloat16, 64, 8>, 8) : launch(attn_simt_kernel<float, 64, 8>, 8);
+  else if (a.dh == 128)
+    a.bf16 ? launch(attn_simt_kernel<__nv_bfloat16, 128, 8>, 8) : launch(attn_simt_kernel<float, 128, 8>, 8);
+  else
     return cudaErrorInvalidValue;
-  }
   return cudaGetLastError();
 }
 

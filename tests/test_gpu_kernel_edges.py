@@ -41,11 +41,14 @@ def test_gate_reduction_and_logit_at_thread_edges(grid, gate_kind, lib):
     (2, 128, (1, 3, 9), 5),      # 32 tokens: whole tiles
     (3, 192, (1, 4, 7), 5),      # 33 tokens: one row and one key past a tile
     (2, 256, (1, 1, 250), 7),    # 257 tokens, head width 128: a second round of key tiles
+    (2, 128, (1, 1, 249), 7),    # 256 and 257 tokens: eight warps, twelve
+    (2, 128, (1, 1, 250), 7),
+    (2, 128, (1, 1, 378), 7),    # 385 tokens: a second round of the twelve
     (2, 128, (1, 17, 29), 20),   # 513 tokens
 ])
 def test_fp32_backbone_at_tile_edges(heads, hidden, grid, n_txt, lib):
     """The fp32 projections (32 x 32 tiles, K in slices of 64 split over eight warps) and the
-    fp32 attention (eight queries a CTA, key tiles of 32 over eight warps): latents against
+    fp32 attention (eight queries a CTA, key tiles of 32 over eight or twelve warps): latents against
     the fp64 oracle to 1e-5 of their RMS (fp32 sums over up to 640 products)."""
     dh = hidden // heads
     cfg = configs.get_config("tiny", hidden=hidden, heads=heads, mlp=4 * hidden, grid=grid, n_txt=n_txt, n_single=1,
