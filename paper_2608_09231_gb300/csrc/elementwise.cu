@@ -446,6 +446,9 @@ constexpr long RC_BYTES = 512l << 10;
 template <typename T, bool VEC>
 __global__ void __cluster_dims__(RC_CTAS, 1, 1) __launch_bounds__(RC_THREADS)
     rel_l1_cluster_kernel(const T* a, const T* b, long rows, long cols, float* partial, float* out) {
+  // rank 0's shared memory may be written once rank 0 is known to run: arrive here, wait before
+  // the store, so that the rows in between hide the barrier
+  cluster_arrive();
   grid_dep_sync();
   __shared__ float2 red[RC_THREADS / 32];
   __shared__ __align__(8) float2 total[RC_CTAS];
@@ -460,6 +463,7 @@ __global__ void __cluster_dims__(RC_CTAS, 1, 1) __launch_bounds__(RC_THREADS)
   }
   if (lane == 0) red[warp] = s;
   __syncthreads();
+  cluster_wait();
   if (warp == 0) {
     s = warp_sum2(lane < RC_THREADS / 32 ? red[lane] : make_float2(0.f, 0.f));
     if (lane == 0)
