@@ -436,13 +436,23 @@ __global__ void __launch_bounds__(RF_THREADS) rel_l1_finalize_kernel(const float
   if (threadIdx.x == 0) rel_l1_store(out, s);
 }
 
-// Small inputs in one launch: a cluster of eight CTAs, a warp per row in turn, the CTAs'
-// sums exchanged through distributed shared memory and added in rank order.  A call costs its
-// launches on the host (one 4.1 us, two 8.2 us a call in a loop); on the GPU eight SMs keep up
-// with the two kernels to about RC_BYTES of both inputs (256 x 256 fp32 3.00 us against 2.6; 1024 x 256
-// fp32 5.5 us against 3.0).
+// Small inputs in one launch: a cluster of eight CTAs, a warp per row, the CTAs' sums
+// exchanged through distributed shared memory and added in rank order.  It saves a call one
+// of its two launches, which are most of a small call's time; the rule is for the time of calls
+// in a loop.  One launch against two, us a call (and on the device, in a graph): 1 x 1024 fp32
+// 4.1 (2.8) against 5.1 (2.8), 64 x 512 fp32 4.1 (2.8) against 5.2 (2.9), 128 x 512 bf16 4.1 (2.8)
+// against 5.0 (2.8), 256 x 256 fp32 4.9 (2.9) against 5.2 (2.9).  Past each limit it loses: more
+// rows than warps, 512 x 128 fp32 6.0 against 5.2; wider rows, which one warp walks alone, 16 x
+// 2048 fp32 6.1 against 5.1, 1 x 65,536 fp32 49 against 25, unaligned 64 x 255 6.1 against 5.0;
+// more bytes, 256 x 512 fp32 5.1 (3.3) against 5.1 (2.9).
 constexpr int RC_CTAS = 8, RC_THREADS = 1024;
-constexpr long RC_BYTES = 512l << 10;
+constexpr int RC_ROWS = RC_CTAS * RC_THREADS / 32;
+constexpr long RC_BYTES = 512l << 10;  // of both inputs
+// Widest row: four loads a lane (16-byte groups, or elements).
+template <typename T, bool VEC>
+constexpr long rc_cols() {
+  return 4 * 32 * (VEC ? 16 / (long)sizeof(T) : 1);
+}
 template <typename T, bool VEC>
 __global__ void __cluster_dims__(RC_CTAS, 1, 1) __launch_bounds__(RC_THREADS)
     rel_l1_cluster_kernel(const T* a, const T* b, long rows, long cols, float* partial, float* out) {
@@ -455,11 +465,10 @@ __global__ void __cluster_dims__(RC_CTAS, 1, 1) __launch_bounds__(RC_THREADS)
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   const uint32_t rank = cluster_ctarank();
   float2 s = make_float2(0.f, 0.f);
-  for (long row = warp * RC_CTAS + (int)rank; row < rows; row += RC_CTAS * RC_THREADS / 32) {
-    const float2 p = warp_sum2(rel_l1_row<T, VEC>(a + row * cols, b + row * cols, cols, lane, 32));
-    if (lane == 0) rel_l1_partial(partial, row, p);
-    s.x += p.x;
-    s.y += p.y;
+  const long row = warp * RC_CTAS + (int)rank;
+  if (row < rows) {
+    s = warp_sum2(rel_l1_row<T, VEC>(a + row * cols, b + row * cols, cols, lane, 32));
+    if (lane == 0) rel_l1_partial(partial, row, s);
   }
   if (lane == 0) red[warp] = s;
   __syncthreads();
@@ -492,9 +501,9 @@ cudaError_t rel_l1(const void* a, const void* b, int bf16, long rows, long cols,
     constexpr bool V = decltype(v)::value;
     const T* ta = static_cast<const T*>(a);
     const T* tb = static_cast<const T*>(b);
-    if (rows <= RC_BYTES / (2 * es) / cols)
+    if (rows <= RC_ROWS && cols <= rc_cols<T, V>() && rows * cols * 2 * es <= RC_BYTES)
       return launch_kernel(rel_l1_cluster_kernel<T, V>, RC_CTAS, RC_THREADS, 0, s, ta, tb, rows, cols, scratch, out);
-    // from two rows per warp slot of an SM on, a warp a row
+    // from eight rows an SM on, a warp a row
     cudaError_t r;
     if (rows >= (long)sm_count() * 8)
       r = launch_kernel(rel_l1_kernel<T, V, 1>, (unsigned)((rows + 3) / 4), RL_THREADS, 0, s, ta, tb, rows, cols,

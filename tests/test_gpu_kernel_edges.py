@@ -117,16 +117,20 @@ def test_fp32_output_rows(M, N, K, epilogue, offset, pad, lib):
 
 
 @pytest.mark.parametrize("rows,cols", [
-    (1, 1), (3, 8), (129, 256),   # one cluster: fewer rows than warps, a round and one row
-    (300, 255),                   # one cluster (bf16), rows that are not 16-byte groups
+    (1, 1), (3, 8), (129, 256),   # one cluster: fewer rows than warps
+    (256, 127), (256, 256),       # a row a warp; elements, 16-byte groups, the byte limit (fp32)
+    (256, 129), (257, 64), (128, 513), (256, 264),  # just past a limit: elements, rows, width (fp32), bytes (fp32)
+    (300, 255),                   # rows that are not 16-byte groups
+    (1, 65536), (8, 16384),       # few bytes in wide rows: four warps a row
     (1215, 520), (1217, 1023),    # around a warp per row (eight rows an SM)
     (64, 40000), (4099, 130)])
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
 @pytest.mark.parametrize("offset", [0, 1])  # inputs and scratch off 16-byte alignment
 def test_rel_l1_routes(rows, cols, dtype, offset, lib):
     """Every route of the relative L1 (cluster, four warps or one a row; 16-byte groups or
-    elements): sums against fp64 to 2e-6 (fp32 chains of at most a few hundred terms, then a
-    tree), the same bits again and through the allocation-free entry."""
+    elements): sums against fp64 to 2e-6 (fp32 chains of at most 512 terms, each rounding at
+    most 2^-24 of the sum and of either sign, then a tree), the same bits again and through the
+    allocation-free entry."""
     ctx = bag.create("tiny", T=2, B=1)
     g = torch.Generator(device="cuda").manual_seed(rows * 7 + cols)
 
@@ -151,6 +155,28 @@ def test_rel_l1_routes(rows, cols, dtype, offset, lib):
     assert bool(((part[:, 1] - den.sum(1)).abs() <= 2e-6 * den.sum(1)).all())
     assert float(scratch[offset + 2 * rows]) == 0.0
     assert torch.equal(out, again) and torch.equal(out, noalloc)
+
+
+@pytest.mark.parametrize("dtype,cols", [(torch.float32, 65536), (torch.bfloat16, 131072)])
+@pytest.mark.parametrize("offset", [0, 1])
+def test_rel_l1_of_one_wide_row_is_not_left_to_one_warp(dtype, cols, offset, lib):
+    """512 KB in one row take less time than the 1 MB of a row twice as wide, whose route does
+    not depend on the size (one warp alone took 49 to 320 us for the former, against 46 to 52)."""
+    us = []
+    for n in (cols, 2 * cols):
+        a, b = (torch.randn(n + offset, device="cuda").to(dtype)[offset:].reshape(1, n) for _ in range(2))
+        out = torch.zeros(3, device="cuda")
+        best = 1e9
+        for _ in range(8):
+            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            e0.record()
+            for _ in range(50):
+                bag.rel_l1_noalloc(a, b, 1, n, out)
+            e1.record()
+            torch.cuda.synchronize()
+            best = min(best, e0.elapsed_time(e1) * 20)
+        us.append(best)
+    assert us[0] <= 0.8 * us[1], us
 
 
 @pytest.mark.parametrize("nq,nk,heads", [
