@@ -977,16 +977,21 @@ __global__ void __launch_bounds__(192)
 }
 
 // CTAs per tile for a launch of `tiles` 128 x 64 tiles and `kit` K blocks: the largest
-// split, up to 4, that leaves every CTA SK_MIN_KB blocks and keeps the launch within one CTA
-// per SM (clusters of eight leave 32 of the 152 SMs without a place)
-// (1: the unsplit kernels).  A guided launch may hold twice the planned tiles; two CTAs fit
+// split, up to 4, that keeps the launch within one CTA per SM (clusters of eight leave 32 of
+// the 152 SMs without a place; up to two CTAs an SM made the small guided sample 1592 -> 1663
+// us); 1: the unsplit kernels.  A guided launch may hold twice the planned tiles; two CTAs fit
 // on an SM.
-// Fewest blocks a CTA: 2 against 4 makes the small Wan-shaped sample 1113 -> 1037 us, the small
-// guided one 1630 -> 1600 (8: 1.5 % slower than 4).  Up to two CTAs an SM: small guided 1592 -> 1663.
-constexpr int SK_MIN_KB = 2;
+// From SK_MIN_KB K blocks on.  As single calls, unsplit against split (us): 32 x 1024 x 256, two
+// CTAs, 6.2 against 7.9; 32 x 1024 x 448 7.0 against 8.5; eight blocks, 300 x 512 x 512, four
+// CTAs, 8.2 against 8.5 and with GELU 8.7 in both; 300 x 512 x 1024 9.8 against 9.0; two CTAs,
+// 1000 x 512 x 1024, 10.0 against 9.8.  In the samples, where programmatic launch hides the
+// cluster's start, eight blocks already gain (small Wan-shaped sample 1113 -> 1037 us, small
+// guided one 1630 -> 1600).
+constexpr int SK_MIN_KB = 8;
 static int splitk_ctas(int tiles, int kit, int ns) {
+  if (kit < SK_MIN_KB) return 1;
   for (int s = 4; s > 1; s /= 2)
-    if (tiles * s <= ns && kit >= s * SK_MIN_KB) return s;
+    if (tiles * s <= ns) return s;
   return 1;
 }
 

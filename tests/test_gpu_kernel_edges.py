@@ -93,6 +93,29 @@ def test_split_k_gemm(M, N, K, epilogue, lib):
     assert bool((C[M] == -7.0).all())
 
 
+@pytest.mark.parametrize("M,N", [(32, 1024), (32, 4096)])
+def test_gemm_of_four_k_blocks_costs_no_more_than_three(M, N, lib):
+    """Around the K block count where a launch starts to split K: the call with one block more
+    (split in two it took 1.3 to 1.4 times as long)."""
+    ctx = bag.create("tiny", T=2, B=1)
+    us = []
+    for K in (192, 256):
+        A, W = torch.randn(M, K, device="cuda").bfloat16(), torch.randn(N, K, device="cuda").bfloat16()
+        C = torch.empty(M, N, device="cuda")
+        best = 1e9
+        for _ in range(8):
+            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            e0.record()
+            for _ in range(100):
+                ctx.gemm_bf16(A, W, None, C, M, N, K)
+            e1.record()
+            torch.cuda.synchronize()
+            best = min(best, e0.elapsed_time(e1) * 10)
+        us.append(best)
+    ctx.close()
+    assert us[1] <= 1.2 * us[0], us
+
+
 @pytest.mark.parametrize("M,N,K", [(33, 64, 128), (1300, 1280, 64), (2500, 3072, 64)])  # BN 64, BN 128, CTA pairs
 @pytest.mark.parametrize("epilogue", [0, 1])
 @pytest.mark.parametrize("offset,pad", [(0, 0), (4, 4), (1, 3)])  # 16-byte rows and not
