@@ -35,9 +35,12 @@ BAG_DEV float4 ldv4(const void* p, long i) {
 // reads V rows coalesced.  Bound: latency (the fp32 backbones have a few hundred tokens);
 // few queries per CTA and the keys split over warps keep every SM busy with a short chain.
 // Measured against sixteen queries per CTA whose four warps walked all keys one barrier
-// after another (profiled launches): 288 tokens x 4 heads of 64 41 -> 19.2 us with eight warps,
-// which leave the ninth tile for a second round; 14.4 with twelve, 16.4 with sixteen.  Heads
-// of 64 take twelve past 256 keys; heads of 128 eight (the outputs to merge take 4 KB a warp).
+// after another (profiled launches, heads of 64): 288 tokens x 4 heads 41 us, 17.9 with eight
+// warps, which leave the ninth tile for a second round, 13.7 with twelve; 512 x 4 69 us, 26 and
+// 36; 1024 x 16 366 us, 286 and 352.  Twelve warps win only where they take all tiles in one
+// round and every CTA has an SM to itself: 384 x 2 (96 CTAs) 15.2 us against 18.6 with eight,
+// but 320 x 4 (160 CTAs) 22.8 against 21.8, 288 x 6 23.8 against 21.9, and with two rounds in
+// both 512 x 2 21.9 against 19.8.  Heads of 128 take eight (the outputs to merge take 4 KB a warp).
 constexpr int SA_Q = 8, SA_KT = 32;
 
 template <typename T, int DH, int SA_WARPS>
@@ -178,7 +181,8 @@ cudaError_t attention(const AttnArgs& a, int* err, cudaStream_t s, int force_sim
   if (a.f16 || a.nbr > 1) return cudaErrorNotSupported;  // tensor-core kernel only
   dim3 grid((a.nq + SA_Q - 1) / SA_Q, a.heads);
   auto launch = [&](auto kernel, int warps) { launch_kernel(kernel, grid, warps * 32, 0, s, a); };
-  if (a.dh == 64 && a.nk > 8 * SA_KT)
+  const bool one_round = a.nk > 8 * SA_KT && a.nk <= 12 * SA_KT && (long)grid.x * grid.y <= sm_count();
+  if (a.dh == 64 && one_round)
     a.bf16 ? launch(attn_simt_kernel<__nv_bfloat16, 64, 12>, 12) : launch(attn_simt_kernel<float, 64, 12>, 12);
   else if (a.dh == 64)
     a.bf16 ? launch(attn_simt_kernel<__nv_bfloat16, 64, 8>, 8) : launch(attn_simt_kernel<float, 64, 8>, 8);

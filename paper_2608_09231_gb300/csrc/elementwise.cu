@@ -276,7 +276,7 @@ __global__ void __launch_bounds__(TH, MINB) ln_mod_kernel(const LnArgs a) {
   }
 }
 
-static int sm_count() {
+int sm_count() {
   static int n = 0;
   if (!n) {
     int dev = 0;

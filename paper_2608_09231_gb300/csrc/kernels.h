@@ -47,6 +47,8 @@ inline cudaError_t launch_kernel(void (*k)(P...), dim3 grid, dim3 block, size_t 
   return launch_cluster(k, 0u, grid, block, smem, s, std::forward<A>(args)...);
 }
 
+int sm_count();  // SMs of the device
+
 // Per-sample state the step kernels read and write on the device, so that a whole
 // denoising step can be replayed from a CUDA graph with no host round trip.
 struct DevState {
