@@ -154,7 +154,12 @@ BAG_DEV void mma_bf16_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint3
 // key tiles.  Rank r then collects 2 * AT_M / C rows of every CTA's unnormalised output,
 // maximum and sum through distributed shared memory and merges them in rank order.  Used
 // where whole units would leave a wave mostly idle (attention_split).
-template <bool F16, int C>
+// ROWS (C = 1): the output leaves from registers, a row a lane.  With few rows there are few
+// stores to gather, and the way through shared memory is four more steps at the end of a short
+// call: 64 queries x 64 keys x 2 heads 8.9 against 7.9 us a call, 64 x 64 x 40 9.1 against 8.8,
+// 128 x 128 x 16 8.8 against 8.5, 128 x 128 x 40 9.1 against 9.4, 256 x 256 x 24 10.9 against 13.0
+// (attention_rows).  A kernel of its own: as a branch it made 7145 x 24 1.7 % slower.
+template <bool F16, int C, bool ROWS = false>
 __global__ void __launch_bounds__(AT_THREADS, 1)
     attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                    const __grid_constant__ CUtensorMap tmV, const AttnTcParams p) {
@@ -468,6 +473,22 @@ __global__ void __launch_bounds__(AT_THREADS, 1)
                                     (long)q * p.ldo + head * AT_D + lane * 4) = u;
         }
       }
+    } else if (ROWS) {
+      if (ok) {
+        const float inv = 1.f / l;
+        const int q = q0 + x * AT_M + quad * 32 + lane;
+        void* o1 = br ? p.o_b1 : p.o;
+        void* o2 = br ? p.o2_b1 : p.o2;
+        void* ob = o2 && q >= p.o_split ? o2 : o1;
+#pragma unroll 1
+        for (int c = 0; c < AT_D; c += 32) {
+          float o[32];
+          tmem_ld32(o_addr + c, o);
+#pragma unroll
+          for (int i = 0; i < 32; ++i) o[i] *= inv;
+          if (q < p.nq) store_vals<32>(ob, (long)q * p.ldo + head * AT_D + c, o, kStoreBF16);
+        }
+      }
     } else if (ok) {
       const float inv = 1.f / l;
       // through shared memory (this tile's Q, which no product reads any more): four lanes
@@ -511,7 +532,8 @@ static int g_sms = 1;
 cudaError_t attention_tc_init() {
   const void* kernels[] = {(const void*)attn_tc_kernel<false, 1>, (const void*)attn_tc_kernel<false, 2>,
                            (const void*)attn_tc_kernel<false, 4>, (const void*)attn_tc_kernel<true, 1>,
-                           (const void*)attn_tc_kernel<true, 2>,  (const void*)attn_tc_kernel<true, 4>};
+                           (const void*)attn_tc_kernel<true, 2>,  (const void*)attn_tc_kernel<true, 4>,
+                           (const void*)attn_tc_kernel<false, 1, true>, (const void*)attn_tc_kernel<true, 1, true>};
   cudaError_t r = cudaSuccess;
   for (const void* k : kernels)
     if (r == cudaSuccess) r = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, AT_SMEM);
@@ -543,6 +565,9 @@ static int attention_split(int units, int nkt, int* whole) {
   *whole = units - rest;
   return 2;
 }
+
+// Whether an unshared launch writes its output a row a lane (see attn_tc_kernel).
+static bool attention_rows(int nq, int heads) { return nq <= AT_M && (long)nq * heads <= 2560; }
 
 int attention_tc_supported(const AttnArgs& a) {
   if (!a.bf16 || a.dh != AT_D || a.v_mode != 1) return 0;
@@ -588,7 +613,10 @@ cudaError_t attention_tc(const AttnArgs& a, int* err, cudaStream_t s) {
   auto launch = [&](auto kernel) {
     launch_cluster(kernel, c > 1 ? (unsigned)c : 0u, grid, AT_THREADS, AT_SMEM, s, tq, tk, tv, p);
   };
-  if (a.f16)
+  const bool rows = c == 1 && attention_rows(a.nq, a.heads);
+  if (rows)
+    a.f16 ? launch(attn_tc_kernel<true, 1, true>) : launch(attn_tc_kernel<false, 1, true>);
+  else if (a.f16)
     c == 4 ? launch(attn_tc_kernel<true, 4>)
            : (c == 2 ? launch(attn_tc_kernel<true, 2>) : launch(attn_tc_kernel<true, 1>));
   else

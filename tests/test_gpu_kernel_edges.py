@@ -66,6 +66,36 @@ def test_fp32_backbone_at_tile_edges(heads, hidden, grid, n_txt, lib):
     assert float(np.max(np.abs(x.cpu().numpy() - ref))) <= 1e-5 * rms
 
 
+def test_attention_of_few_rows_takes_the_short_way_out(lib):
+    """Device time (captured) of 64 queries x 64 keys: two heads against 48, whose output goes
+    through shared memory as the two heads' once did (0.98 of the time then, 0.86 now)."""
+    ctx = bag.create("tiny", T=2, B=1)
+    s = torch.cuda.Stream()
+    ctx.set_stream(s.cuda_stream)
+    graphs, keep = [], []
+    for heads in (2, 48):
+        q, k = (torch.randn(64, heads * 128, device="cuda").half() for _ in range(2))
+        vt, o = torch.randn(heads, 128, 128, device="cuda").half(), torch.empty(64, heads * 128, device="cuda").bfloat16()
+        keep.append((q, k, vt, o))
+        graphs.append(torch.cuda.CUDAGraph())
+        with torch.cuda.graph(graphs[-1], stream=s):
+            for _ in range(40):
+                ctx.attention_f16(q, k, vt, o, 64, 64, heads, 128, 128)
+    us = [1e9, 1e9]
+    for _ in range(30):  # in turn: the clock is the same for both
+        for i, graph in enumerate(graphs):
+            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            e0.record()
+            for _ in range(5):
+                graph.replay()
+            e1.record()
+            torch.cuda.synchronize()
+            us[i] = min(us[i], e0.elapsed_time(e1) * 5)
+    del graphs
+    ctx.close()
+    assert us[0] <= 0.92 * us[1], us
+
+
 def test_fp32_attention_of_twice_the_tokens(lib):
     """From 256 to 512 tokens x 4 heads (four times the work, launches that fill the GPU once and
     twice): 1.9 times the time with eight warps a CTA, 2.6 with twelve at the larger one."""
@@ -230,11 +260,15 @@ def test_rel_l1_of_one_wide_row_is_not_left_to_one_warp(dtype, cols, offset, lib
     (257, 1537, 3),    # one key in the 13th tile, one row in the last query pair
     (10240, 2049, 1),  # 40 units: two CTAs, eight or nine tiles
     (2560, 2000, 16),  # 160 units on 152 SMs: the last eight are shared
+    (1, 1, 1),         # one row, one key
+    (128, 130, 20),    # the most rows written a row a lane
+    (128, 64, 21),     # and past it: through shared memory
+    (129, 128, 2),     # one row in the second tile of the pair
 ])
 @pytest.mark.parametrize("dtype", [torch.float16, torch.bfloat16])
-def test_attention_shared_units(nq, nk, heads, dtype, lib):
-    """Units shared by a cluster against fp64: the output's bf16 rounding (2^-8 relative) plus
-    the operand type's rounding of P (2^-11 or 2^-8 of the largest output)."""
+def test_attention_shared_units_and_few_rows(nq, nk, heads, dtype, lib):
+    """Units shared by a cluster, and few rows, against fp64: the output's bf16 rounding (2^-8
+    relative) plus the operand type's rounding of P (2^-11 or 2^-8 of the largest output)."""
     ctx = bag.create("tiny", T=2, B=1)
     g = torch.Generator(device="cuda").manual_seed(nq + nk)
     q, k, v = (torch.randn(n, heads, 128, generator=g, device="cuda").to(dtype) for n in (nq, nk, nk))
