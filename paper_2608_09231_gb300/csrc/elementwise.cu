@@ -313,7 +313,8 @@ cudaError_t ln_mod(const LnArgs& a, cudaStream_t s) {
   const cudaError_t r = a.sig_on ? launch(std::integral_constant<int, LN_SIGNAL>{})
                                  : (a.cache_in ? launch(std::integral_constant<int, LN_CACHE>{})
                                                : launch(std::integral_constant<int, LN_PLAIN>{}));
-  return r == cudaSuccess ? cudaGetLastError() : r;
+  const cudaError_t last = cudaGetLastError();  // also taken off the thread, or the next check reports it again
+  return r == cudaSuccess ? last : r;
 }
 
 // ---------------------------------------------------------------------------
@@ -521,7 +522,8 @@ cudaError_t rel_l1(const void* a, const void* b, int bf16, long rows, long cols,
     r = vec ? run(uint16_t{}, std::true_type{}) : run(uint16_t{}, std::false_type{});
   else
     r = vec ? run(float{}, std::true_type{}) : run(float{}, std::false_type{});
-  return r == cudaSuccess ? cudaGetLastError() : r;
+  const cudaError_t last = cudaGetLastError();
+  return r == cudaSuccess ? last : r;
 }
 
 // ---------------------------------------------------------------------------

@@ -1014,10 +1014,11 @@ static cudaError_t launch_splitk(int S, const void* A0, long lda0, const void* W
   }
   const int tiles = ((M0 + TC_BM - 1) / TC_BM + (M1 + TC_BM - 1) / TC_BM) * (N / SK_BN);
   auto launch = [&](auto kernel) {
-    return launch_cluster(kernel, (unsigned)S, (unsigned)(tiles * S), 192, SK_SMEM, s, ta0, tb0, ta1, tb1, e0, e1,
-                          M0, M1, N, K, a_split, err);
+    launch_cluster(kernel, (unsigned)S, (unsigned)(tiles * S), 192, SK_SMEM, s, ta0, tb0, ta1, tb1, e0, e1, M0, M1,
+                   N, K, a_split, err);
   };
-  return S == 4 ? launch(gemm_splitk_kernel<4>) : launch(gemm_splitk_kernel<2>);
+  S == 4 ? launch(gemm_splitk_kernel<4>) : launch(gemm_splitk_kernel<2>);
+  return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------

@@ -1,6 +1,8 @@
 """GPU kernels at the sizes where they can go wrong (tile edges, remainders, the smallest
 and largest of a range), against the fp64 oracle or a plain fp64 restatement of the op."""
 
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -230,6 +232,29 @@ def test_rel_l1_routes(rows, cols, dtype, offset, lib):
     assert bool(((part[:, 1] - den.sum(1)).abs() <= 2e-6 * den.sum(1)).all())
     assert float(scratch[offset + 2 * rows]) == 0.0
     assert torch.equal(out, again) and torch.equal(out, noalloc)
+
+
+@pytest.mark.parametrize("rows,cols", [(64, 64), (300, 64), (1300, 64)])  # one launch, two (four warps a row, one)
+def test_a_failed_launch_leaves_no_error_to_the_next_call(rows, cols, lib):
+    """A launch on a stream whose capture was invalidated fails on the host; the next call, on
+    another stream, succeeds.  (Synchronising a stream that is being captured invalidates it.)"""
+    ctx = bag.create("tiny", T=2, B=1)
+    a, out = torch.randn(rows, cols, device="cuda"), torch.zeros(3, device="cuda")
+    total, n = torch.zeros_like(a), rows * cols
+    s = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    driver, handle, graph = ctypes.CDLL("libcuda.so.1"), ctypes.c_void_p(s.cuda_stream), ctypes.c_void_p()
+    bag.rel_l1_noalloc(a, a, rows, cols, out)  # looks up its scratch outside the capture
+    torch.cuda.synchronize()
+    assert driver.cuStreamBeginCapture_v2(handle, 2) == 0  # relaxed: no other stream or thread is concerned
+    assert driver.cuStreamSynchronize(handle) != 0
+    with pytest.raises(bag.BagError):
+        bag.rel_l1_noalloc(a, a, rows, cols, out, s.cuda_stream)
+    assert driver.cuStreamEndCapture(handle, ctypes.byref(graph)) != 0
+    ctx.residual_add(total, a, a, n)
+    torch.cuda.synchronize()
+    ctx.close()
+    assert torch.equal(total, a + a)
 
 
 @pytest.mark.parametrize("dtype,cols", [(torch.float32, 65536), (torch.bfloat16, 131072)])
