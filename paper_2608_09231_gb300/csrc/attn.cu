@@ -112,11 +112,15 @@ __global__ void __launch_bounds__(SA_WARPS * 32) attn_simt_kernel(const AttnArgs
       float v[4][R];
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
-        const long kk = min(kb + j + u, a.nk - 1);  // past the last key the weight is zero
+        // past the last key weight and value are zero (a zero weight times an infinity is not)
+        const bool in = kb + j + u < a.nk;
+        const long kk = min(kb + j + u, a.nk - 1);
 #pragma unroll
-        for (int r = 0; r < R; ++r)
-          v[u][r] = a.v_mode == 0 ? ldv<T>(a.v, kk * a.ldv + head * DH + lane * R + r)
-                                  : ldv<T>(a.v, (long)(head * DH + lane * R + r) * a.vpad + kk);
+        for (int r = 0; r < R; ++r) {
+          const float x = a.v_mode == 0 ? ldv<T>(a.v, kk * a.ldv + head * DH + lane * R + r)
+                                        : ldv<T>(a.v, (long)(head * DH + lane * R + r) * a.vpad + kk);
+          v[u][r] = in ? x : 0.f;
+        }
       }
 #pragma unroll
       for (int i = 0; i < SA_Q; ++i) {

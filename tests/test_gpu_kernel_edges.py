@@ -68,6 +68,33 @@ def test_fp32_backbone_at_tile_edges(heads, hidden, grid, n_txt, lib):
     assert float(np.max(np.abs(x.cpu().numpy() - ref))) <= 1e-5 * rms
 
 
+@pytest.mark.parametrize("nk", [1, 33, 34, 36, 289])  # one to three keys past a group of four, none
+@pytest.mark.parametrize("transposed", [0, 1])
+@pytest.mark.parametrize("dh", [64, 128])
+def test_cuda_core_attention_with_an_infinite_value(nk, transposed, dh, lib):
+    """An infinity in the last key's value makes that column infinite (every weight is positive
+    here), not NaN, and no other."""
+    ctx = bag.create("tiny", T=2, B=1)
+    g = torch.Generator(device="cuda").manual_seed(nk)
+    q, k, v = (torch.randn(n, dh, generator=g, device="cuda").bfloat16() for n in (9, nk, nk))
+    v[nk - 1, 3] = float("inf")
+    vpad = (nk + 7) // 8 * 8 if transposed else 0
+    vv = v
+    if transposed:
+        vv = torch.zeros(dh, vpad, device="cuda", dtype=torch.bfloat16)
+        vv[:, :nk] = v.T
+    o = torch.zeros(9, dh, device="cuda", dtype=torch.bfloat16)
+    ctx.attention_bf16(q, k, vv, o, 9, nk, 1, dh, vpad, 1)
+    torch.cuda.synchronize()
+    ctx.close()
+    want = torch.softmax(q.double() @ k.double().T / dh ** 0.5, -1) @ v.double()
+    assert bool(torch.isinf(o[:, 3]).all()) and bool(torch.isfinite(want[:, 4:]).all())
+    rest = [c for c in range(dh) if c != 3]
+    err = (o.double() - want)[:, rest].abs()
+    # fp32 throughout, the output's bf16 rounding
+    assert bool((err <= 2.0 ** -8 * want[:, rest].abs() + 1e-5).all())
+
+
 def test_attention_of_few_rows_takes_the_short_way_out(lib):
     """Device time (captured) of 64 queries x 64 keys: two heads against 48, whose output goes
     through shared memory as the two heads' once did (0.98 of the time then, 0.86 now)."""
