@@ -69,14 +69,6 @@ static int num_sms() {
 // ---------------------------------------------------------------------------
 // CUDA-core GEMM (fp32 or bf16 operands, fp32 accumulation)
 // ---------------------------------------------------------------------------
-template <typename T>
-BAG_DEV float ld_f(const T* p) {
-  if constexpr (sizeof(T) == 2)
-    return __bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(p));
-  else
-    return *p;
-}
-
 // One CTA computes a 32 x 32 tile; its eight warps split every 64-wide K slice (8 columns
 // each), so that each warp holds the whole tile (4 x 8 per lane) and the partial tiles are
 // summed in warp order at the end.  Bound: latency.  The fp32 backbones are small (a few
@@ -86,6 +78,10 @@ BAG_DEV float ld_f(const T* p) {
 // memory (eight rows x 16 bytes hit all 32 banks).
 // Measured against 64 x 64 tiles with one K chain per CTA, scalar loads and no prefetch
 // (profiled launches): 288 x 256 x 1280 158 -> 21 us, 288 x 1792 x 256 37 -> 22 us.
+// bf16 operands (cross-checks of the tensor-core kernels) are fetched a slice ahead into
+// registers: loaded and stored in one go they took 988 us for 2048 x 2048 x 2048 (64 x 64 tiles
+// 753), now 507, unaligned 649; 1024 x 1024 x 1024 151 (131), now 76; 4096 x 4096 x 512 1047 (701),
+// now 605, unaligned 756.
 constexpr int SG_T = 32, SG_BK = 64, SG_LD = SG_BK + 4, SG_STAGES = 4, SG_WARPS = 8;
 constexpr int SG_TILE = SG_T * SG_LD;  // floats of one operand's tile in one stage
 constexpr int SG_SMEM = SG_STAGES * 2 * SG_TILE * 4;
@@ -97,23 +93,46 @@ BAG_DEV void cp_async16(float* dst, const void* src, bool valid) {
                : "memory");
 }
 
-// Rows r0 .. r0 + 31 of P (columns k0 .. k0 + 63) into shared memory, zeros outside.
-// VEC: fp32 rows of 16-byte aligned float4 groups (K a multiple of 4).
-template <typename T, bool VEC>
-BAG_DEV void sg_load(float* dst, const T* __restrict__ P, long ld, int r0, int rows, int k0, int K) {
-  if constexpr (VEC) {
+// Rows r0 .. r0 + 31 of P (columns k0 .. k0 + 63) into shared memory, zeros outside, copied
+// asynchronously: fp32 rows of 16-byte aligned float4 groups (K a multiple of 4).
+BAG_DEV void sg_load_async(float* dst, const float* __restrict__ P, long ld, int r0, int rows, int k0, int K) {
 #pragma unroll
-    for (int i = threadIdx.x; i < SG_T * SG_BK / 4; i += SG_WARPS * 32) {
-      const int r = i / (SG_BK / 4), c = (i % (SG_BK / 4)) * 4;
-      const bool ok = r0 + r < rows && k0 + c < K;
-      cp_async16(dst + r * SG_LD + c, ok ? P + (long)(r0 + r) * ld + k0 + c : P, ok);
-    }
-  } else {
-    for (int i = threadIdx.x; i < SG_T * SG_BK; i += SG_WARPS * 32) {
-      const int r = i / SG_BK, c = i % SG_BK;
-      dst[r * SG_LD + c] = r0 + r < rows && k0 + c < K ? ld_f(P + (long)(r0 + r) * ld + k0 + c) : 0.f;
+  for (int i = threadIdx.x; i < SG_T * SG_BK / 4; i += SG_WARPS * 32) {
+    const int r = i / (SG_BK / 4), c = (i % (SG_BK / 4)) * 4;
+    const bool ok = r0 + r < rows && k0 + c < K;
+    cp_async16(dst + r * SG_LD + c, ok ? P + (long)(r0 + r) * ld + k0 + c : P, ok);
+  }
+}
+
+// The same slice of a bf16 operand, which has to be converted, in two steps with the products
+// of a slice in between: into registers (eight values a thread), then into shared memory.
+// VEC: one 16-byte load (K and ld multiples of 8, P 16-byte aligned); else eight single ones.
+static_assert(SG_T * SG_BK == 8 * SG_WARPS * 32, "eight values of an operand's slice a thread");
+template <bool VEC>
+BAG_DEV uint4 sg_fetch(const __nv_bfloat16* __restrict__ P, long ld, int r0, int rows, int k0, int K) {
+  const int r = r0 + threadIdx.x / (SG_BK / 8), c = k0 + threadIdx.x % (SG_BK / 8) * 8;
+  uint4 v = make_uint4(0u, 0u, 0u, 0u);
+  const unsigned short* p = reinterpret_cast<const unsigned short*>(P) + (long)r * ld + c;
+  if (r < rows && c < K) {
+    if constexpr (VEC) {
+      v = __ldg(reinterpret_cast<const uint4*>(p));
+    } else {
+      uint32_t x[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) x[u] = c + u < K ? __ldg(p + u) : 0u;
+      v = make_uint4(x[0] | x[1] << 16, x[2] | x[3] << 16, x[4] | x[5] << 16, x[6] | x[7] << 16);
     }
   }
+  return v;
+}
+BAG_DEV void sg_put(float* dst, uint4 v) {
+  float4* d = reinterpret_cast<float4*>(dst + threadIdx.x / (SG_BK / 8) * SG_LD + threadIdx.x % (SG_BK / 8) * 8);
+  auto pair = [](uint32_t a, uint32_t b) {
+    return make_float4(__uint_as_float(a << 16), __uint_as_float(a & 0xffff0000u), __uint_as_float(b << 16),
+                       __uint_as_float(b & 0xffff0000u));
+  };
+  d[0] = pair(v.x, v.y);
+  d[1] = pair(v.z, v.w);
 }
 
 template <typename T, bool VEC>
@@ -130,19 +149,37 @@ __global__ void __launch_bounds__(SG_WARPS * 32) gemm_simt_kernel(const T* __res
   const int num_n = (N + SG_T - 1) / SG_T;
   const int m0 = blockIdx.x / num_n * SG_T, n0 = blockIdx.x % num_n * SG_T;
   const int nk = (K + SG_BK - 1) / SG_BK;
-  auto load = [&](int kb) {
-    if (kb < nk) {
-      float* d = sg + (kb % SG_STAGES) * 2 * SG_TILE;
-      sg_load<T, VEC>(d, A, lda, m0, M, kb * SG_BK, K);
-      sg_load<T, VEC>(d + SG_TILE, W, ldw, n0, N, kb * SG_BK, K);
+  [[maybe_unused]] uint4 fa, fw;  // bf16: the slice after the last one in the ring
+  [[maybe_unused]] auto fetch = [&](int kb) {
+    if constexpr (sizeof(T) == 2) {
+      if (kb < nk) {
+        fa = sg_fetch<VEC>(A, lda, m0, M, kb * SG_BK, K);
+        fw = sg_fetch<VEC>(W, ldw, n0, N, kb * SG_BK, K);
+      }
     }
-    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  auto load = [&](int kb) {
+    float* d = sg + (kb % SG_STAGES) * 2 * SG_TILE;
+    if constexpr (sizeof(T) == 2) {
+      if (kb < nk) {
+        sg_put(d, fa);
+        sg_put(d + SG_TILE, fw);
+      }
+      fetch(kb + 1);
+    } else {
+      if (kb < nk) {
+        sg_load_async(d, A, lda, m0, M, kb * SG_BK, K);
+        sg_load_async(d + SG_TILE, W, ldw, n0, N, kb * SG_BK, K);
+      }
+      asm volatile("cp.async.commit_group;" ::: "memory");
+    }
   };
   float acc[4][8];
 #pragma unroll
   for (int i = 0; i < 4; ++i)
 #pragma unroll
     for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
+  fetch(0);
   for (int kb = 0; kb < SG_STAGES - 1; ++kb) load(kb);
   for (int kb = 0; kb < nk; ++kb) {
     asm volatile("cp.async.wait_group %0;" ::"n"(SG_STAGES - 2) : "memory");
@@ -1327,6 +1364,7 @@ cudaError_t kernels_init() {
   smem(gemm_splitk_kernel<2>, SK_SMEM);
   smem(gemm_splitk_kernel<4>, SK_SMEM);
   smem(gemm_simt_kernel<float, true>, SG_SMEM);
+  smem(gemm_simt_kernel<__nv_bfloat16, true>, SG_SMEM);
   smem(gemm_simt_kernel<__nv_bfloat16, false>, SG_SMEM);
   if (r == cudaSuccess) r = attention_tc_init();
   num_sms();
@@ -1405,15 +1443,15 @@ cudaError_t gemm(const void* A, long lda, const void* W, long ldw, int M, int N,
   if (N % 4 != 0) return cudaErrorInvalidValue;
   const long tiles = (long)((N + SG_T - 1) / SG_T) * ((M + SG_T - 1) / SG_T);
   if (tiles > 0x7fffffffL) return cudaErrorInvalidValue;
+  const uintptr_t ptrs = reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(W);
   if (in_bf16) {
-    launch_kernel(gemm_simt_kernel<__nv_bfloat16, false>, (unsigned)tiles, SG_WARPS * 32, SG_SMEM, s,
-                  reinterpret_cast<const __nv_bfloat16*>(A), lda,
+    const bool vec = K % 8 == 0 && lda % 8 == 0 && ldw % 8 == 0 && (ptrs & 15) == 0;
+    launch_kernel(vec ? gemm_simt_kernel<__nv_bfloat16, true> : gemm_simt_kernel<__nv_bfloat16, false>,
+                  (unsigned)tiles, SG_WARPS * 32, SG_SMEM, s, reinterpret_cast<const __nv_bfloat16*>(A), lda,
                   reinterpret_cast<const __nv_bfloat16*>(W), ldw, M, N, K, e);
   } else {
     // the fp32 backbones' operands: rows of whole float4 groups
-    if (K % 4 || lda % 4 || ldw % 4 ||
-        ((reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(W)) & 15))
-      return cudaErrorNotSupported;
+    if (K % 4 || lda % 4 || ldw % 4 || (ptrs & 15)) return cudaErrorNotSupported;
     launch_kernel(gemm_simt_kernel<float, true>, (unsigned)tiles, SG_WARPS * 32, SG_SMEM, s,
                   reinterpret_cast<const float*>(A), lda, reinterpret_cast<const float*>(W), ldw, M, N, K, e);
   }

@@ -13,6 +13,20 @@ from paper_2608_09231_gb300 import bag, configs, synth
 pytestmark = pytest.mark.gpu
 
 
+def call_us(call, n):
+    """Microseconds a call, the least of eight loops of n calls."""
+    best = 1e9
+    for _ in range(8):
+        e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        e0.record()
+        for _ in range(n):
+            call()
+        e1.record()
+        torch.cuda.synchronize()
+        best = min(best, 1e3 * e0.elapsed_time(e1) / n)
+    return best
+
+
 @pytest.mark.parametrize("gate_kind", ["mlp3", "flux6", "wan6"])
 @pytest.mark.parametrize("grid", [(1, 1, 1), (1, 1, 127), (1, 8, 16), (1, 3, 43), (1, 33, 31), (1, 32, 32), (1, 25, 61)])
 def test_gate_reduction_and_logit_at_thread_edges(grid, gate_kind, lib):
@@ -66,6 +80,39 @@ def test_fp32_backbone_at_tile_edges(heads, hidden, grid, n_txt, lib):
     ref = O.sample(cfg, synth.make_weights(cfg), synth.make_gate(cfg["gate_seed"]), inp, T=2, B=2)["x"]
     rms = float(np.sqrt(np.mean(ref ** 2)))
     assert float(np.max(np.abs(x.cpu().numpy() - ref))) <= 1e-5 * rms
+
+
+@pytest.mark.parametrize("M,N,K", [(1, 64, 64), (33, 64, 192), (31, 128, 320), (65, 192, 1024)])
+@pytest.mark.parametrize("offset", [0, 1, 4])  # 16-byte rows and not
+def test_cuda_core_gemm_of_bf16_rows(M, N, K, offset, lib):
+    """One K slice, a ring's worth and more, with 16-byte loads and single ones, against fp64:
+    the fp32 sum over K, bounded by 4 K 2^-24 sum|a||w|; rows around the operands hold NaN."""
+    ctx = bag.create("tiny", T=2, B=1)
+    g = torch.Generator(device="cuda").manual_seed(M + N + K + offset)
+
+    def rows(n):
+        buf = torch.full((n + 2, K + offset), float("nan"), device="cuda").bfloat16()
+        buf[1:n + 1, offset:] = torch.randn(n, K, generator=g, device="cuda").bfloat16()
+        return buf[1:n + 1, offset:]
+
+    A, W, C = rows(M), rows(N), torch.full((M + 1, N), -7.0, device="cuda")
+    ctx.gemm_bf16(A, W, None, C, M, N, K, 0, 1)
+    torch.cuda.synchronize()
+    ctx.close()
+    err = (C[:M].double() - A.double() @ W.double().T).abs()
+    assert bool((err <= 4 * K * 2.0 ** -24 * (A.double().abs() @ W.double().abs().T)).all())
+    assert bool((C[M] == -7.0).all())
+
+
+def test_cuda_core_gemm_of_bf16_rows_keeps_its_time(lib):
+    """2048 x 2048 x 2048: no more than the 753 us of 64 x 64 tiles (507 with operands fetched a
+    slice ahead, 988 without)."""
+    ctx = bag.create("tiny", T=2, B=1)
+    A, W = (torch.randn(2048, 2048, device="cuda").bfloat16() for _ in range(2))
+    C = torch.empty(2048, 2048, device="cuda")
+    us = call_us(lambda: ctx.gemm_bf16(A, W, None, C, 2048, 2048, 2048, 0, 1), 10)
+    ctx.close()
+    assert us <= 753, us
 
 
 @pytest.mark.parametrize("nk", [1, 33, 34, 36, 289])  # one to three keys past a group of four, none
@@ -183,16 +230,7 @@ def test_gemm_of_four_k_blocks_costs_no_more_than_three(M, N, lib):
     for K in (192, 256):
         A, W = torch.randn(M, K, device="cuda").bfloat16(), torch.randn(N, K, device="cuda").bfloat16()
         C = torch.empty(M, N, device="cuda")
-        best = 1e9
-        for _ in range(8):
-            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-            e0.record()
-            for _ in range(100):
-                ctx.gemm_bf16(A, W, None, C, M, N, K)
-            e1.record()
-            torch.cuda.synchronize()
-            best = min(best, e0.elapsed_time(e1) * 10)
-        us.append(best)
+        us.append(call_us(lambda: ctx.gemm_bf16(A, W, None, C, M, N, K), 100))
     ctx.close()
     assert us[1] <= 1.2 * us[0], us
 
@@ -293,16 +331,7 @@ def test_rel_l1_of_one_wide_row_is_not_left_to_one_warp(dtype, cols, offset, lib
     for n in (cols, 2 * cols):
         a, b = (torch.randn(n + offset, device="cuda").to(dtype)[offset:].reshape(1, n) for _ in range(2))
         out = torch.zeros(3, device="cuda")
-        best = 1e9
-        for _ in range(8):
-            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-            e0.record()
-            for _ in range(50):
-                bag.rel_l1_noalloc(a, b, 1, n, out)
-            e1.record()
-            torch.cuda.synchronize()
-            best = min(best, e0.elapsed_time(e1) * 20)
-        us.append(best)
+        us.append(call_us(lambda: bag.rel_l1_noalloc(a, b, 1, n, out), 50))
     assert us[0] <= 0.8 * us[1], us
 
 
