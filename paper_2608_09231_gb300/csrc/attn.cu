@@ -18,13 +18,36 @@ BAG_DEV float ldv(const void* p, long i) {
     return reinterpret_cast<const float*>(p)[i];
 }
 
-// Four consecutive elements (fp32 rows of the contexts are 16-byte aligned).
-template <typename T>
-BAG_DEV float4 ldv4(const void* p, long i) {
-  if constexpr (sizeof(T) == 4)
-    return *reinterpret_cast<const float4*>(reinterpret_cast<const float*>(p) + i);
-  else
-    return make_float4(ldv<T>(p, i), ldv<T>(p, i + 1), ldv<T>(p, i + 2), ldv<T>(p, i + 3));
+// N consecutive elements (2 or 4).  VEC: one load (fp32 rows of the contexts are 16-byte
+// aligned; bf16 rows 8-byte); else one each.  bf16 with one load per element, against one per
+// four: 1024 tokens x 8 heads of 64 330 -> 145 us, 2048 x 8 of 128 2272 -> 871 (keys and values
+// staged in shared memory for sixteen queries: 203 and 1887); transposed V 525 -> 195 (313).
+template <typename T, bool VEC, int N>
+BAG_DEV void ldvn(const void* p, long i, float* v) {
+  if constexpr (VEC && sizeof(T) == 2) {
+    uint32_t w[N / 2];
+    if constexpr (N == 4) {
+      const uint2 u = *reinterpret_cast<const uint2*>(reinterpret_cast<const T*>(p) + i);
+      w[0] = u.x;
+      w[1] = u.y;
+    } else {
+      w[0] = *reinterpret_cast<const uint32_t*>(reinterpret_cast<const T*>(p) + i);
+    }
+#pragma unroll
+    for (int k = 0; k < N / 2; ++k) {
+      v[2 * k] = __uint_as_float(w[k] << 16);
+      v[2 * k + 1] = __uint_as_float(w[k] & 0xffff0000u);
+    }
+  } else if constexpr (VEC && N == 4) {
+    const float4 f = *reinterpret_cast<const float4*>(reinterpret_cast<const float*>(p) + i);
+    v[0] = f.x;
+    v[1] = f.y;
+    v[2] = f.z;
+    v[3] = f.w;
+  } else {
+#pragma unroll
+    for (int k = 0; k < N; ++k) v[k] = ldv<T>(p, i + k);
+  }
 }
 
 // CTA = eight queries of one head; its warps take the key tiles (32 keys) in turn, each with
@@ -43,7 +66,7 @@ BAG_DEV float4 ldv4(const void* p, long i) {
 // both 512 x 2 21.9 against 19.8.  Heads of 128 take eight (the outputs to merge take 4 KB a warp).
 constexpr int SA_Q = 8, SA_KT = 32;
 
-template <typename T, int DH, int SA_WARPS>
+template <typename T, int DH, int SA_WARPS, bool VEC = true>
 __global__ void __launch_bounds__(SA_WARPS * 32) attn_simt_kernel(const AttnArgs a) {
   grid_dep_sync();
   if (epi_skip(a.st, a.flag_want)) return;
@@ -77,14 +100,15 @@ __global__ void __launch_bounds__(SA_WARPS * 32) attn_simt_kernel(const AttnArgs
     for (int i = 0; i < SA_Q; ++i) s[i] = 0.f;
 #pragma unroll 8
     for (int c = 0; c < DH; c += 4) {
-      const float4 k4 = ldv4<T>(a.k, krow + c);
+      float k4[4];
+      ldvn<T, VEC, 4>(a.k, krow + c, k4);
 #pragma unroll
       for (int i = 0; i < SA_Q; ++i) {
         const float4 q4 = *reinterpret_cast<const float4*>(&Qs[i][c]);
-        s[i] += q4.x * k4.x;
-        s[i] += q4.y * k4.y;
-        s[i] += q4.z * k4.z;
-        s[i] += q4.w * k4.w;
+        s[i] += q4.x * k4[0];
+        s[i] += q4.y * k4[1];
+        s[i] += q4.z * k4[2];
+        s[i] += q4.w * k4[3];
       }
     }
     __syncwarp();  // every lane has read the previous tile's weights
@@ -109,17 +133,23 @@ __global__ void __launch_bounds__(SA_WARPS * 32) attn_simt_kernel(const AttnArgs
     const int nkt = min(SA_KT, a.nk - kb);
 #pragma unroll 2
     for (int j = 0; j < nkt; j += 4) {
-      float v[4][R];
+      float v[4][R];  // past the last key weight and value are zero (a zero weight times an infinity is not)
+      if (a.v_mode == 0) {
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        // past the last key weight and value are zero (a zero weight times an infinity is not)
-        const bool in = kb + j + u < a.nk;
-        const long kk = min(kb + j + u, a.nk - 1);
+        for (int u = 0; u < 4; ++u) {
+          const bool in = kb + j + u < a.nk;
+          ldvn<T, VEC, R>(a.v, (long)min(kb + j + u, a.nk - 1) * a.ldv + head * DH + lane * R, v[u]);
+#pragma unroll
+          for (int r = 0; r < R; ++r) v[u][r] = in ? v[u][r] : 0.f;
+        }
+      } else {
+        // four keys of a column: in bounds also at the end (vpad is a multiple of 8)
 #pragma unroll
         for (int r = 0; r < R; ++r) {
-          const float x = a.v_mode == 0 ? ldv<T>(a.v, kk * a.ldv + head * DH + lane * R + r)
-                                        : ldv<T>(a.v, (long)(head * DH + lane * R + r) * a.vpad + kk);
-          v[u][r] = in ? x : 0.f;
+          float x[4];
+          ldvn<T, VEC, 4>(a.v, (long)(head * DH + lane * R + r) * a.vpad + kb + j, x);
+#pragma unroll
+          for (int u = 0; u < 4; ++u) v[u][r] = kb + j + u < a.nk ? x[u] : 0.f;
         }
       }
 #pragma unroll
@@ -186,12 +216,18 @@ cudaError_t attention(const AttnArgs& a, int* err, cudaStream_t s, int force_sim
   dim3 grid((a.nq + SA_Q - 1) / SA_Q, a.heads);
   auto launch = [&](auto kernel, int warps) { launch_kernel(kernel, grid, warps * 32, 0, s, a); };
   const bool one_round = a.nk > 8 * SA_KT && a.nk <= 12 * SA_KT && (long)grid.x * grid.y <= sm_count();
+  const bool vec = ((reinterpret_cast<uintptr_t>(a.k) | reinterpret_cast<uintptr_t>(a.v)) & 7) == 0 &&
+                   a.ldk % 4 == 0 && (a.v_mode ? a.vpad : a.ldv) % 4 == 0;  // bf16 rows
+  using B = __nv_bfloat16;
   if (a.dh == 64 && one_round)
-    a.bf16 ? launch(attn_simt_kernel<__nv_bfloat16, 64, 12>, 12) : launch(attn_simt_kernel<float, 64, 12>, 12);
+    !a.bf16 ? launch(attn_simt_kernel<float, 64, 12>, 12)
+            : (vec ? launch(attn_simt_kernel<B, 64, 12>, 12) : launch(attn_simt_kernel<B, 64, 12, false>, 12));
   else if (a.dh == 64)
-    a.bf16 ? launch(attn_simt_kernel<__nv_bfloat16, 64, 8>, 8) : launch(attn_simt_kernel<float, 64, 8>, 8);
+    !a.bf16 ? launch(attn_simt_kernel<float, 64, 8>, 8)
+            : (vec ? launch(attn_simt_kernel<B, 64, 8>, 8) : launch(attn_simt_kernel<B, 64, 8, false>, 8));
   else if (a.dh == 128)
-    a.bf16 ? launch(attn_simt_kernel<__nv_bfloat16, 128, 8>, 8) : launch(attn_simt_kernel<float, 128, 8>, 8);
+    !a.bf16 ? launch(attn_simt_kernel<float, 128, 8>, 8)
+            : (vec ? launch(attn_simt_kernel<B, 128, 8>, 8) : launch(attn_simt_kernel<B, 128, 8, false>, 8));
   else
     return cudaErrorInvalidValue;
   return cudaGetLastError();
