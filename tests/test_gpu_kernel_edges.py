@@ -145,6 +145,48 @@ def test_cuda_core_attention_of_bf16_rows(n, nk, heads, dh, transposed, offset, 
     assert bool((o[n] == 9.0).all()) and bool((o[:, heads * dh:] == 9.0).all())
 
 
+@pytest.mark.parametrize("cols", [4, 508, 3072, 3076, 5116, 5120, 5124, 6144])
+def test_ln_mod_widths(cols, lib):
+    """Around each change of threads and columns a thread (128 threads to 3072 columns, 256 with
+    five or six float4 each past it), the narrowest and the widest row: the output's bf16 rounding
+    and fp32 statistics; the rows around it stay untouched."""
+    ctx = bag.create("tiny", T=2, B=1)
+    g = torch.Generator(device="cuda").manual_seed(cols)
+    x = 2.0 * torch.randn(5, cols, generator=g, device="cuda") + 0.5
+    sh, sc = (0.5 * torch.randn(cols, generator=g, device="cuda") for _ in range(2))
+    y = torch.full((7, cols), 9.0, device="cuda").bfloat16()
+    ctx.ln_mod(x, sh, sc, y[1:], 5, cols)
+    torch.cuda.synchronize()
+    ctx.close()
+    xd = x.double()
+    ref = (xd - xd.mean(1, keepdim=True)) / (xd.var(1, unbiased=False, keepdim=True) + 1e-6).sqrt()
+    ref = ref * (1 + sc.double()) + sh.double()
+    assert bool(((y[1:6].double() - ref).abs() <= 2.0 ** -8 * ref.abs() + 1e-5).all())
+    assert bool((y[0] == 9.0).all() and (y[6] == 9.0).all())
+
+
+def test_signal_and_cache_passes_of_wide_rows(lib):
+    """The signal pass and the final layer's pass with the residual cache past 5120 columns (six
+    float4 a thread): a sample with reused steps at width 5248 against the fp64 oracle, to the
+    2e-2 x RMS of bf16 operands, and the logged drift to 1e-2 (bf16 observables)."""
+    cfg = configs.get_config("tiny", hidden=5248, heads=41, mlp=1024, dtype="bf16", grid=(1, 3, 7), n_txt=5,
+                             n_single=1, rope_axes=(16, 56, 56))
+    mask = [1, 0, 0, 1, 0]
+    inp = synth.make_inputs(cfg)
+    ctx = bag.create(cfg, T=5, B=2)
+    ctx.set_policy(bag.POLICY_MASK, np.array(mask, np.uint8))
+    x = torch.from_numpy(inp["x"].copy()).cuda()
+    m, log, nfe = ctx.run(x, torch.from_numpy(inp["txt"]).cuda().bfloat16(), torch.from_numpy(inp["pooled"]).cuda())
+    ctx.close()
+    assert list(m) == mask and nfe == 2
+    inp["txt"] = synth.bf16_round(inp["txt"])
+    ref = O.sample(cfg, synth.make_weights(cfg), synth.make_gate(cfg["gate_seed"]), inp, T=5, B=2, policy=mask)
+    rms = float(np.sqrt(np.mean(ref["x"] ** 2)))
+    assert float(np.max(np.abs(x.cpu().numpy() - ref["x"]))) <= 2e-2 * rms
+    for t in range(1, 5):
+        assert abs(float(log[t, 2]) - ref["log"][t]["drift"]) <= 1e-2 * ref["log"][t]["drift"], t
+
+
 def test_cuda_core_attention_of_bf16_rows_keeps_its_time(lib):
     """1024 tokens x 8 heads of 64: no more than the 203 us of the kernel that staged keys and
     values in shared memory (145 with vector loads, 330 with single ones)."""
@@ -233,16 +275,22 @@ def test_fp32_attention_of_twice_the_tokens(lib):
 
 
 @pytest.mark.parametrize("M,N,K", [
-    (1, 64, 512),        # one row, two CTAs of four K blocks
-    (127, 64, 64 * 9),   # nine blocks over two CTAs
-    (129, 128, 64 * 17), # four CTAs, 4 or 5 blocks each, one row in the last row tile
-    (300, 192, 64 * 35), # eight CTAs
-    (1100, 512, 1024),   # 72 tiles: two CTAs
-    (640, 1024, 2048),   # 80 tiles: not split
+    (1, 64, 64 * 7),      # seven K blocks: not split
+    (1, 64, 512),         # the least that is: one row, four CTAs of two K blocks
+    (127, 64, 64 * 9),    # four CTAs, one with three blocks
+    (129, 128, 64 * 17),  # four CTAs, four or five blocks each, one row in the last row tile
+    (300, 192, 64 * 35),  # nine tiles, eight or nine blocks each
+    (2432, 128, 512),     # 38 tiles, the most for four CTAs
+    (1650, 192, 512),     # 39 tiles: two CTAs of four blocks
+    (1100, 512, 64 * 17), # 72 tiles, two CTAs, eight and nine blocks
+    (1100, 512, 1024),    # even shares
+    (2400, 256, 64 * 9),  # 76 tiles, the most for two CTAs, four and five blocks
+    (1400, 448, 64 * 9),  # 77 tiles: not split
+    (640, 1024, 2048),    # 80 tiles: not split
 ])
 @pytest.mark.parametrize("epilogue", [0, 1])
 def test_split_k_gemm(M, N, K, epilogue, lib):
-    """Shapes around the split-K rule (tiles x CTAs against the SM count, K blocks per CTA)
+    """Shapes around the split-K rule (tiles x CTAs against 152 SMs, at least eight K blocks)
     against fp64: a bf16 product's fp32 sum over K, bounded by 4 K 2^-24 sum|a||w|."""
     ctx = bag.create("tiny", T=2, B=1)
     g = torch.Generator(device="cuda").manual_seed(M + N + K)
@@ -276,7 +324,12 @@ def test_gemm_of_four_k_blocks_costs_no_more_than_three(M, N, lib):
     assert us[1] <= 1.2 * us[0], us
 
 
-@pytest.mark.parametrize("M,N,K", [(33, 64, 128), (1300, 1280, 64), (2500, 3072, 64)])  # BN 64, BN 128, CTA pairs
+@pytest.mark.parametrize("M,N,K", [
+    (33, 64, 128), (1300, 1280, 64),     # 128 x 64 tiles: one, 110 x 2 of them
+    (1300, 1920, 64), (1217, 2176, 448), # 128 x 128 tiles: 165, and 170 with one row in the last row tile
+    (2500, 3072, 64),                    # CTA pairs, eight epilogue warps
+    (2500, 3072, 1088),                  # four (17 K blocks)
+])
 @pytest.mark.parametrize("epilogue", [0, 1])
 @pytest.mark.parametrize("offset,pad", [(0, 0), (4, 4), (1, 3)])  # 16-byte rows and not
 def test_fp32_output_rows(M, N, K, epilogue, offset, pad, lib):
