@@ -307,8 +307,10 @@ cudaError_t ln_mod(const LnArgs& a, cudaStream_t s) {
     constexpr int M = decltype(mode)::value;
     if (a.cols > 5120) return launch_ln<256, 6, 4, M>(a, s);
     if (a.cols > 3072) return launch_ln<256, 5, 5, M>(a, s);
-    if constexpr (M == LN_PLAIN) return launch_ln<128, 6, 10, M>(a, s);
-    return launch_ln<256, 3, M == LN_SIGNAL ? 7 : 6, M>(a, s);
+    if constexpr (M == LN_PLAIN)
+      return launch_ln<128, 6, 10, M>(a, s);
+    else
+      return launch_ln<256, 3, M == LN_SIGNAL ? 7 : 6, M>(a, s);
   };
   const cudaError_t r = a.sig_on ? launch(std::integral_constant<int, LN_SIGNAL>{})
                                  : (a.cache_in ? launch(std::integral_constant<int, LN_CACHE>{})

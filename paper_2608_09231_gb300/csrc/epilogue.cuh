@@ -115,16 +115,11 @@ BAG_DEV void epi_add_bias(const Epi& e, int col0, float* v) {
   }
 }
 
-// EPI_QKV q / k columns (region 0 / 1): per-head RMSNorm (when the block has it), then
-// the rotation of joint-sequence row jr; cc is the column within the region.
+// EPI_QKV q / k columns: the rotation of joint-sequence row jr; cc is the column within the
+// region.  (Per-head RMSNorm is applied in store_16_warp alone.)
 template <int NV>
-BAG_DEV void epi_qk_transform(const Epi& e, int jr, int cc, int region, float* v, float rs) {
-  if (region < 2 && e.qn_q) {  // per-head RMSNorm of q and k, before the rotation
-    const float* w = (region == 0 ? e.qn_q : e.qn_k) + cc % e.dh;
-#pragma unroll
-    for (int j = 0; j < NV; ++j) v[j] = v[j] * rs * __ldg(w + j);
-  }
-  if (region < 2 && e.rope) {
+BAG_DEV void epi_rotate(const Epi& e, int jr, int cc, float* v) {
+  if (e.rope) {
     const int e0 = cc % e.dh;
     const float2* cs = e.rope + (long)jr * (e.dh / 2) + e0 / 2;
     if constexpr (NV % 4 == 0) {
@@ -152,10 +147,8 @@ BAG_DEV void epi_qk_transform(const Epi& e, int jr, int cc, int region, float* v
   }
 }
 
-// rs: EPI_QKV with QK-norm, 1 / RMS of the head that columns col0 .. col0 + NV - 1 of
-// this row belong to (computed by the caller over the whole head).
 template <int NV>
-BAG_DEV void epi_apply(const Epi& e, int t, int row, int col0, float* v, float rs = 1.f) {
+BAG_DEV void epi_apply(const Epi& e, int t, int row, int col0, float* v) {
   if (row >= e.M || col0 >= e.N) return;
   epi_add_bias<NV>(e, col0, v);
   switch (e.kind) {
@@ -190,28 +183,13 @@ BAG_DEV void epi_apply(const Epi& e, int t, int row, int col0, float* v, float r
       const int jr = row - (br1 ? e.br_rows : 0) + e.row_off;  // joint-sequence row
       const long qr = jr + (br1 ? e.br_qk : 0);                // q / k / v buffer row
       const int cc = lc - region * e.d;
-      if (region < 2) epi_qk_transform<NV>(e, jr, cc, region, v, rs);
+      if (region < 2) epi_rotate<NV>(e, jr, cc, v);
       if (region == 0) {
         store_vals<NV>(e.q, qr * e.ldqk + cc, v, e.qkv_type);
       } else if (region == 1) {
         store_vals<NV>(e.k, qr * e.ldqk + cc, v, e.qkv_type);
-      } else if (e.v_mode == 0) {
+      } else {  // (transposed V goes through store_vt_warp)
         store_vals<NV>(e.v, qr * e.ldqk + cc, v, e.qkv_type);
-      } else {
-        // transposed per head: vt[(head * dh + e) * vpad + token]
-        if (e.qkv_type == kStoreF16) {
-          __half* vt = reinterpret_cast<__half*>(e.v) + (br1 ? e.br_vt : 0);
-#pragma unroll
-          for (int j = 0; j < NV; ++j) vt[(long)(cc + j) * e.vpad + jr] = __float2half_rn(v[j]);
-        } else if (e.qkv_type == kStoreBF16) {
-          __nv_bfloat16* vt = reinterpret_cast<__nv_bfloat16*>(e.v) + (br1 ? e.br_vt : 0);
-#pragma unroll
-          for (int j = 0; j < NV; ++j) vt[(long)(cc + j) * e.vpad + jr] = __float2bfloat16_rn(v[j]);
-        } else {
-          float* vt = reinterpret_cast<float*>(e.v) + (br1 ? e.br_vt : 0);
-#pragma unroll
-          for (int j = 0; j < NV; ++j) vt[(long)(cc + j) * e.vpad + jr] = v[j];
-        }
       }
       break;
     }

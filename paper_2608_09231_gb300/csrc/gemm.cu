@@ -512,7 +512,7 @@ BAG_DEV void store_16_warp(const Epi& e, int row0, int col0, const float* v, flo
 //   EP_16   16-bit outputs (rows16) without QK-norm (168)
 //   EP_16N  16-bit outputs with QK-norm (168)
 //   EP_ANY  everything without QK-norm, also rows that are not 16-byte aligned, and launches of
-//           two problems whose classes differ (254)
+//           two problems whose classes differ (226)
 // Measured, one class against four: small guided sample 1727 -> 1634 us, 50 steps of a FLUX
 // block 14.00 -> 13.80 ms, double block 915 -> 896 us.
 enum { EP_ANY = 0, EP_F32 = 1, EP_16 = 2, EP_16N = 3 };
@@ -537,7 +537,7 @@ BAG_DEV void drain_accumulator(const Epi& e, int t, int row, int col0, uint32_t 
     else if (h16)
       store_16_warp(e, row0, col, v, vt_buf, rs);
     else
-      epi_apply<32>(e, t, row, col, v, rs);
+      epi_apply<32>(e, t, row, col, v);
   };
   if constexpr (EP != EP_16N) {
 #pragma unroll 1
@@ -817,9 +817,12 @@ static cudaError_t launch_tc(const void* A0, long lda0, const void* W0, long ldw
     launch(gemm_tc_kernel<BN, EP_F32>, TcCfg<BN, EP_F32>::THREADS, TcCfg<BN, EP_F32>::SMEM);
   else if (ep == EP_16)
     launch(gemm_tc_kernel<BN, EP_16>, TcCfg<BN, EP_16>::THREADS, TcCfg<BN, EP_16>::SMEM);
-  else if (ep == EP_16N)
-    launch(gemm_tc_kernel<BN, EP_16N>, TcCfg<BN, EP_16N>::THREADS, TcCfg<BN, EP_16N>::SMEM);
-  else
+  else if (ep == EP_16N) {
+    if constexpr (BN == 128)
+      launch(gemm_tc_kernel<BN, EP_16N>, TcCfg<BN, EP_16N>::THREADS, TcCfg<BN, EP_16N>::SMEM);
+    else
+      return cudaErrorNotSupported;  // whole heads of 128 in a tile
+  } else
     launch(gemm_tc_kernel<BN, EP_ANY>, TcCfg<BN, EP_ANY>::THREADS, TcCfg<BN, EP_ANY>::SMEM);
   return cudaGetLastError();
 }
@@ -1352,7 +1355,6 @@ cudaError_t kernels_init() {
   smem(gemm_tc_kernel<128, EP_F32>, TcCfg<128, EP_F32>::SMEM);
   smem(gemm_tc_kernel<128, EP_16>, TcCfg<128, EP_16>::SMEM);
   smem(gemm_tc_kernel<128, EP_16N>, TcCfg<128, EP_16N>::SMEM);
-  smem(gemm_tc_kernel<64, EP_16N>, TcCfg<64, EP_16N>::SMEM);
   smem(gemm_tc_kernel<64, EP_ANY>, TcCfg<64, EP_ANY>::SMEM);
   smem(gemm_tc_kernel<64, EP_F32>, TcCfg<64, EP_F32>::SMEM);
   smem(gemm_tc_kernel<64, EP_16>, TcCfg<64, EP_16>::SMEM);
@@ -1391,11 +1393,10 @@ static cudaError_t gemm_tc2(const void* A0, long lda0, const void* W0, long ldw0
   if (a_split && (lda0 < 2L * K || (M1 > 0 && lda1 < 2L * K))) return cudaErrorInvalidValue;
   const int ns = num_sms();
   const int mt = (M0 + TC_BM - 1) / TC_BM + (M1 + TC_BM - 1) / TC_BM;
-  // QK-norm epilogues need whole heads in a tile: BN a multiple of dh
+  // QK-norm epilogues need whole heads in a tile (bf16 backbones have heads of 128) and 16-byte
+  // aligned 16-bit operands (the contexts' buffers)
   const bool qkn = e0.qn_q || (M1 > 0 && e1.qn_q);
-  const int min_bn = qkn ? e0.dh : 64;
-  // and come with 16-byte aligned 16-bit operands (the contexts' buffers)
-  if (qkn && (e0.dh % 32 || (M1 > 0 && e1.dh != e0.dh) || min_bn > 256 || launch_class(e0, M1, e1) != EP_16N))
+  if (qkn && (e0.dh != 128 || (M1 > 0 && e1.dh != 128) || launch_class(e0, M1, e1) != EP_16N))
     return cudaErrorNotSupported;
   if (e0.kind != EPI_QKV && (M1 <= 0 || e1.kind != EPI_QKV)) {
     const int mtp = e0.plan_rows > 0 ? (e0.plan_rows + TC_BM - 1) / TC_BM : mt;
@@ -1407,10 +1408,9 @@ static cudaError_t gemm_tc2(const void* A0, long lda0, const void* W0, long ldw0
   if (gemm_uses_pair(M0, M1 > 0 ? M1 : 0, N))
     return launch_pair(A0, lda0, W0, ldw0, M0, e0, A1, lda1, W1, ldw1, M1 > 0 ? M1 : 0, e1, N, K, err, s,
                        a_split);
-  if (min_bn > 128) return cudaErrorNotSupported;
-  if (N % 128 == 0 && (mt * (N / 128) >= ns || min_bn > 64))
+  if (N % 128 == 0 && (mt * (N / 128) >= ns || qkn))
     return launch_tc<128>(A0, lda0, W0, ldw0, M0, e0, A1, lda1, W1, ldw1, M1, e1, N, K, err, s, a_split);
-  if (min_bn > 64) return cudaErrorNotSupported;
+  if (qkn) return cudaErrorNotSupported;
   return launch_tc<64>(A0, lda0, W0, ldw0, M0, e0, A1, lda1, W1, ldw1, M1, e1, N, K, err, s, a_split);
 }
 
@@ -1440,6 +1440,8 @@ cudaError_t gemm(const void* A, long lda, const void* W, long ldw, int M, int N,
     return gemm_tc2(A, lda, W, ldw, M, e, nullptr, 0, nullptr, 0, 0, e, N, K, err, s, a_split);
   }
   if (a_split) return cudaErrorInvalidValue;
+  // transposed V and QK-norm are epilogues of the tensor-core kernels
+  if (e.kind == EPI_QKV && (e.v_mode != 0 || e.qn_q)) return cudaErrorNotSupported;
   if (N % 4 != 0) return cudaErrorInvalidValue;
   const long tiles = (long)((N + SG_T - 1) / SG_T) * ((M + SG_T - 1) / SG_T);
   if (tiles > 0x7fffffffL) return cudaErrorInvalidValue;
