@@ -143,7 +143,8 @@ typedef struct bag_ctx bag_ctx;
  * no later call allocates.  *out receives the context (NULL on failure).  Consecutive
  * kernels of a bf16 context's step are launched with programmatic stream serialization (each
  * kernel waits on the device for its predecessor); the environment variable BAG_PDL=0, read
- * here, launches them with plain stream order instead.
+ * here, launches them with plain stream order instead, as it does the two kernels of this
+ * context's bag_rel_l1 (bag_rel_l1_noalloc, which has no context, always chains its two).
  * Errors: EINVAL (bad arch/T/B), ENOMEM, ECUDA, EUNSUPPORTED. */
 bag_status bag_create(const bag_arch* arch, int T, int B, bag_ctx** out);
 

@@ -52,7 +52,10 @@ constexpr int AT_SMEM = AT_OFF_BAR + 256 + 1024;
 constexpr int AT_TMEM_COLS = 512;  // S_A [0,128) S_B [128,256) O_A [256,384) O_B [384,512)
 constexpr int AT_THREADS = 384;
 // registers a thread: 168 at launch (65,536 / 384); the issuing warps' group gives up 96 and
-// the two softmax groups take 48 each: 128 * 72 + 256 * 216 = 384 * 168
+// the two softmax groups take 48 each: 128 * 72 + 256 * 216 = 384 * 168.  How much moves matters
+// little: 72 / 216, 88 / 208 and 104 / 200 take 170, 170 and 172 us (4608 tokens x 24 heads), 408,
+// 420 and 406 (7145 x 24), 3289, 3290 and 3373 (16,384 x 40), with 236, 208 and 28 bytes of spill
+// loads reported by ptxas; without setmaxnreg 4608 x 24 takes 176.
 constexpr int AT_REGS_ISSUE = 72, AT_REGS_SOFTMAX = 216;
 constexpr int AT_OLD = 36;         // floats a row in the output transpose
 // exchange of partial outputs (C > 1), over the Q, K and V tiles: 2 * AT_M rows of AT_D

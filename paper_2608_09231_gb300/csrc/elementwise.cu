@@ -81,8 +81,10 @@ BAG_DEV void load4(const void* p, long off, int bf16, float* r) {
 }
 
 // Four floats of a row that this SM reads once: they take no L1 lines from the modulation
-// vectors, which every row reads.  4608 x 3072 from HBM 24.4 -> 23.5 us, 50 steps of a FLUX block
-// 13.51 -> 13.39 ms (from L2 14.4 -> 15.2 us on one buffer over and over).
+// vectors, which every row reads.  Kept for 50 steps of a FLUX block, 13.51 -> 13.39 ms.  Single
+// launches on the device, plain loads against these: 4608 x 3072 over rotating buffers 17.7 ->
+// 17.1 us but 12.8 -> 14.1 on one buffer, whose rows are in L2; 4608 x 5120 27.0 -> 25.6 and 27.3
+// -> 23.1; 32,760 x 5120 148 -> 149.
 BAG_DEV float4 ld_once(const float4* p) {
   float4 v;
   asm volatile("ld.global.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];"

@@ -1069,7 +1069,7 @@ static cudaError_t launch_splitk(int S, const void* A0, long lda0, const void* W
 // limit of the single-CTA kernel.  Roles as in gemm_tc_kernel: warp 0 of each CTA loads
 // its halves (completion signalled on the even CTA's barrier), warp 1 of the even CTA
 // issues the MMAs and multicasts their completion to both CTAs, warps 2..5 of each CTA
-// drain its 128 accumulator rows.
+// (2..9 for fp32 rows with few K blocks) drain its 128 accumulator rows.
 // ---------------------------------------------------------------------------
 constexpr int PR_BM = 256, PR_BN = 256;
 constexpr int PR_HALF_BYTES = 128 * TC_BK * 2;  // one CTA's A or W half-tile per k-block
