@@ -1220,7 +1220,7 @@ static float* img_stream(bag_ctx* ctx, int br = 0) {
 static void enq_prefix(Enq& q, int use_cond, unsigned long long handle) {
   bag_ctx* ctx = q.ctx;
   const long d = ctx->d;
-  Epi pe = base_epi(ctx, ctx->st, -1);
+  Epi pe = base_epi(ctx, nullptr, -1);  // reads no step: its own thread is advancing it
   pe.kind = EPI_STORE;
   pe.bias = (const float*)ctx->G.at("pe_b").p;
   pe.out = ctx->h_in;
