@@ -326,6 +326,7 @@ def test_gemm_of_four_k_blocks_costs_no_more_than_three(M, N, lib):
 
 @pytest.mark.parametrize("M,N,K", [
     (33, 64, 128), (1300, 1280, 64),     # 128 x 64 tiles: one, 110 x 2 of them
+    (33, 64, 512), (1100, 512, 576),     # K split over four CTAs, over two
     (1300, 1920, 64), (1217, 2176, 448), # 128 x 128 tiles: 165, and 170 with one row in the last row tile
     (2500, 3072, 64),                    # CTA pairs, eight epilogue warps
     (2500, 3072, 1088),                  # four (17 K blocks)
